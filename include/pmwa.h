@@ -400,9 +400,10 @@ int pmwa_profile_read(pmwa_handle* h, double* ms, int64_t* launches, int32_t n);
    candidates (Step 3), 1 leg merge (Step 3), 2 worm creation (Step 4),
    3 scattering (Step 5) outside the block-wide passes (all of it for a
    domain of at most 32 worms, whose passes run in one warp), 4 output +
-   measurement (Step 6), 5 per-pass set-up of the block-wide passes
-   (grouping, move descriptors, random words), 6 their moves; 7 (a count,
-   not cycles) the rounds of independent moves the block-wide passes took;
+   measurement (Step 6), 5 the block-wide passes up to the moves (groups,
+   barrier, random words), 6 the moves and the look ahead to the next pass's
+   vertices; 7 (a count, not cycles) the times the first warp went round its
+   waiting moves, block-wide rounds where a thread holds several worms;
    n >= 8 entries,
    cleared after reading.  No paper counterpart: measurement plumbing. */
 int pmwa_profile_phases(pmwa_handle* h, uint64_t* cycles, int32_t n);

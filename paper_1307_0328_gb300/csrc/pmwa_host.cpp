@@ -42,7 +42,7 @@ namespace {
 struct Derived {
   int N, ndx, ndy, ndom, dom_x, dom_y, cap, capb, wcap, poolcap;
   int ntau;  // temporal domains (1: none)
-  double legs_want, mb;  // legs wanted in a domain table; mean Step-3 candidates per bond
+  double legs_want;  // legs wanted in a domain table
   double d[4], D, tkink, SV, SW, XW;
   GridScale SVs, SWs, XQ;
   uint64_t TV[4], SWI;
@@ -188,7 +188,6 @@ void derive(const pmwa_params* p, Derived* g) {
   int cap = p->cap_site ? p->cap_site : int(mean + 8.0 * std::sqrt(mean) + 24.0);
   g->cap = (cap + 7) & ~7;
   const double mb = p->beta * g->D;
-  g->mb = mb;
   g->capb = (int(mb + 8.0 * std::sqrt(mb) + 16.0) + 7) & ~7;
   // shared-memory tile of one domain: legs (<= 4 bonds x beta (D + t) per
   // site), Step-3 candidates (mean beta D per bond), worms (<= beta eta per site)
@@ -456,7 +455,7 @@ int pmwa_create(const pmwa_params* p, void* arena, size_t bytes, void* stream, p
   h->err = d.err;
   h->phase = reinterpret_cast<unsigned long long*>(base + L.phase);
   d.phase_cycles = nullptr;
-  if (!plan_tile_smem(&d, g.legs_want, g.mb)) {  // a domain too large for shared memory
+  if (!plan_tile_smem(&d, g.legs_want)) {  // a domain too large for shared memory
     delete h;
     return PMWA_EINVAL;
   }
@@ -523,8 +522,8 @@ int pmwa_tile_plan(const pmwa_params* p, int32_t* smem, int32_t* legcap, int32_t
   d.sub_block = p->sub_block; d.wcap = g.wcap; d.poolcap = g.poolcap;
   d.ntau = g.ntau;
   d.win_half = (p->vertex_window >= 0.5) ? kTwo59 : uint64_t(p->vertex_window * 0x1p59);
-  if (!plan_tile_smem(&d, g.legs_want, g.mb)) return PMWA_EINVAL;
-  if (smem) *smem = d.sm_total;
+  if (!plan_tile_smem(&d, g.legs_want)) return PMWA_EINVAL;
+  if (smem) *smem = d.sm_plan;
   if (legcap) *legcap = d.legcap;
   if (oldcap) *oldcap = d.oldcap;
   return PMWA_OK;
@@ -1030,7 +1029,7 @@ bool batch_layout(const pmwa_params* p, int n, BatchLayout* L) {
 // whose plans allow different residencies go to different launches: a few
 // large plans then do not cut the residency of all the others.
 int batch_group(const Dev& d) {
-  const int c = tile_class(d.dom_x * d.dom_y, d.sm_total);
+  const int c = tile_class(d);
   // (1 KB the hardware reserves a CTA, up to 1 KB of static shared memory)
   const int per_sm = int((228LL * 1024) / (static_cast<long long>(d.sm_total) + 2048));
   const int r = per_sm >= 8 ? 5 : per_sm >= 6 ? 4 : per_sm >= 4 ? 3 : per_sm >= 3 ? 2 : per_sm >= 2 ? 1 : 0;

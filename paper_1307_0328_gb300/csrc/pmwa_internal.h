@@ -44,10 +44,14 @@ struct Dev {
   int poolcap;  // Step-3 candidates per domain in shared memory
   // shared-memory carve-up of the tile kernel (byte offsets)
   int sm_th, sm_zig, sm_off, sm_base, sm_bcnt, sm_boff, sm_misc, sm_nbr, sm_sub, sm_tinfo, sm_leg, sm_wcnt, sm_pool,
-      sm_worm, sm_idx, sm_ord, sm_wsb, sm_wrk, sm_rw, sm_bkt, sm_cnt, sm_fill, sm_total;
+      sm_worm, sm_idx, sm_ord, sm_dn, sm_nxt, sm_fp, sm_cell, sm_gcnt, sm_hash, sm_bkt, sm_fill,
+      sm_total;
+  int sm_plan;          // bytes of the plan as reported (pmwa_tile_plan); sm_total <= sm_plan are used
   int sm_soff, sm_old;  // staged current configuration of the domain (phases 1-2)
   int sm_part;          // [legcap] u16: index of each vertex leg's partner leg (Step 5)
   int use_part;         // 1: the partner table is planned; 0: Step 5 searches for partners
+  int gtab;             // 1: Step 5 holds tables of its groups' members; 0: lists only
+  int ghash;            // heads of Step 5's chains of worms by leg (a power of two; 0: none)
   int oldcap;           // events it can hold; 0 = read the configuration from HBM
   unsigned long long* phase_cycles;  // 8 counters when profiling, else null
   // random numbers
@@ -136,7 +140,7 @@ int launch_temporal_batch(const Dev* devs, const BatchBase* base, const int2* wo
 int temporal_sites_per_block();
 int prepare_temporal(int cap);
 int launch_tile(const Dev& d, int stop, void* stream);
-int tile_class(int domain_sites, int smem);
+int tile_class(const Dev& d);
 // batch launch groups: 3 CTA-size classes x residency levels by shared memory
 constexpr int kResidencyLevels = 6;
 constexpr int kBatchGroups = 4 * kResidencyLevels;
@@ -171,8 +175,9 @@ int launch_green(int Lx, int Ly, int K, int rmax, const double* rho, double* sum
 // rho slices through the library's own static device scratch (no allocation)
 int rho_slices_static(const Dev& d, int K, double* host_out, void* stream);
 // shared-memory plan of the tile kernel for this instance (fills the sm_*
-// offsets); returns false if a domain cannot fit in shared memory.
-bool plan_tile_smem(Dev* d, double legs_want, double cands_per_bond);
+// offsets) for legs_want legs; returns false if a domain cannot fit in
+// shared memory.
+bool plan_tile_smem(Dev* d, double legs_want);
 
 // Step-5 sub-block count along one axis (host copy of the device rule).
 inline int sb_slots_host(int D, int B, int nd) {

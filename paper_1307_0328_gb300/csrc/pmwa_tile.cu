@@ -9,12 +9,19 @@
 //   phase 3  Step 4, one thread per site: worms of every interval (Eq. 1)
 //            into the shared worm table; each worm records its site and the
 //            index of the vertex leg just below it (its interval)
-//   phase 4  Step 5, N_cycle passes of the shifted sub-block schedule: worms
-//            grouped by sub-block, each group's worms moved in label order
-//            (Eq. 2) by rounds of moves whose intervals do not meet, which
+//   phase 4  Step 5, N_cycle passes of the shifted sub-block schedule: the
+//            worms of a sub-block move in label order (Eq. 2); a move waits
+//            only for the earlier ones whose intervals meet its own, which
 //            gives the moves made one by one; vertex legs never move in
 //            Step 5, so a move is a handful of shared-memory reads and two
-//            bit flips
+//            bit flips.  What bounds it is the length of one move's dependent
+//            chain times the few moves that follow one another in a pass
+//            (3 to 12 of a CTA's warps have work, 0.3 instructions a cycle),
+//            so a pass has one barrier, lengths are 32-bit differences where
+//            these decide, and a worm looks for its next vertex while others
+//            still move.  One 16x16-site domain, cycles a pass: 10.1k -> 6.4k
+//            at beta t = 4 (95 worms), 19.6k -> 10.9k at beta t = 16 (381
+//            worms); an 8x8 domain of one group (22 worms): 19.0k -> 5.4k
 //   phase 5  legs and worms merged per site into the next configuration in
 //            HBM, with the Step-6 counters and the Supplement S-I estimator
 //
@@ -40,11 +47,11 @@ constexpr int kSmemLimit = 232448;  // opt-in shared memory per block on sm_103a
 
 struct WormRec {
   uint64_t key;
-  uint64_t lab;   // label (Step 4); in a Step-5 pass the move's intervals, then its wait mask
+  uint64_t lab;   // label (Step 4)
   uint16_t site;  // local site index
   uint16_t leg;   // leg array index of the delimiter just below (kNone: site without legs)
   uint16_t slab;  // temporal slab (0 without temporal domains); fixed through Step 5
-  uint16_t xr;    // in a Step-5 pass: rank in the sub-block, then the round of the move
+  uint16_t pad;
 };
 
 struct Misc {
@@ -103,27 +110,35 @@ __device__ int block_scan(int* a, int n, int* wsum) {
 
 struct Tile {
   const Dev* d;
-  uint64_t* th;
+  uint32_t* th;    // [256] directed-loop thresholds, 2^32 held as 2^32 - 1
   int* off;        // [nds + 1] start of each site's legs in leg[]
   uint8_t* base;   // [nds] state of a site without legs
   int* bcnt;       // [2 nds] candidates per bond of the domain
+  uint32_t* rng;   // [nds] (bcnt, once the legs are merged) first leg | end << 16 of each site
   int* boff;       // [2 nds] their start in pool[]
+  int* perr;       // [2] (boff, once the legs are merged) a status found in an even / odd pass of Step 5
   Misc* misc;
   uint64_t* leg;   // [legcap]
   uint8_t* wcnt;   // [legcap] worms in the interval just above each leg
   uint16_t* part;  // [legcap] index of the partner leg of each leg's vertex (kNone: none in the domain)
   uint64_t* pool;  // [poolcap] (aliases the worm table)
   WormRec* W;      // [wcap]
-  uint16_t* idx;   // [wcap] worms grouped by sub-block (a pass) or by site (output)
+  uint16_t* idx;   // [wcap] (nxt) worms by label bucket before Step 5, by site after it
   uint16_t* ord;   // [wcap] worm indices in label order (lab, site, key)
-  uint16_t* wsb;   // [wcap] sub-block of the k-th worm in label order (a pass)
-  uint16_t* wrk;   // [wcap] rank of the k-th worm inside its sub-block (a pass)
-  uint64_t* rw;    // [2 wcap] Philox words of each grouped position (a pass)
+  uint16_t* dn;    // [wcap] stamp of the last pass in which the k-th worm in label order has moved
+  // (two buffers each, for even and odd passes)
+  uint16_t* nxt;   // [2 wcap] the worm after the k-th one in its group's list
+  uint32_t* fp;    // [2 wcap] the vertex the k-th worm's move reaches
+  uint32_t* hd;    // [hstride + groups] (bkt, fill) head of each group's list: pass stamp << 16 | worm
+  int hstride;     // from the even passes' heads to the odd ones'
+  uint16_t* cell;  // [2 groups x 8] the first members of each group
+  uint32_t* hash;  // [2 ghash] heads of the chains of worms by leg: pass stamp << 16 | entry
+  int* gcnt;       // [3 groups] members of each group (three passes in turn)
   int* bkt;        // [max(nsub, nds) + 1]
-  uint16_t* cnt;   // [warps x groups] per 32-worm chunk: pass stamp << 8 | worms of group u
   int* fill;       // [max(nsub, nds)]
-  int16_t* nbr;    // [6 nds] per leg tag: partner site << 1 | lower-site bit, -1 off-domain
-  uint8_t* tinfo;  // [6 nds] per leg tag: 1 = lower site of the bond, 2 = bond leaves the domain
+  uint16_t* nbr;   // [6 nds] per leg tag: the bond's other site (0 when it leaves the domain)
+  uint8_t* tinfo;  // [6 nds] per leg tag: 1 = lower site of the bond, 2 = bond leaves the domain,
+                   // 4 << q = both sites in one sub-block in pass pattern q
   uint16_t* sub;   // [4 nds] sub-block of each site for offset pattern pass & 3
   int* soff;       // [nds + 1] start of each site's events in old[] (when staged)
   uint64_t* old;   // [oldcap] the domain's current configuration (when staged)
@@ -213,7 +228,7 @@ __device__ __forceinline__ bool kept_leg(const Tile& T, int li, uint64_t k) {
   if (T.tinfo[li * 6 + ktag(k)] & 2) return true;
   if (OTF) {
     const uint64_t pos = kpk(k) >> 3;
-    return !(in_win(T, li, pos) || in_win(T, T.nbr[li * 6 + ktag(k)] >> 1, pos));
+    return !(in_win(T, li, pos) || in_win(T, T.nbr[li * 6 + ktag(k)], pos));
   }
   return false;
 }
@@ -231,148 +246,199 @@ __device__ __forceinline__ void site_bonds(const Tile& T, int li, int lb[4]) {
 }
 
 // ---------------------------------------------------------------------------
-// phase 4: one Step-5 move of worm seg[r] (its sub-block's worms are seg[0..n),
-// and only they can sit on the sub-block's sites).
-__device__ int leg_index(const Tile& T, int x, uint64_t pv) {
-  const int st = T.off[x], en = T.off[x + 1];
-  int lo = st, hi = en;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (kpk(T.leg[mid]) < pv) lo = mid + 1; else hi = mid;
+// phase 4: Step-5 moves.
+//
+// index of the leg at time point pv on site x (-1: none).  A step tells apart
+// four parts by three loads that do not wait for one another: half the
+// dependent steps of a bisection.
+__device__ __forceinline__ int leg_index(const Tile& T, int x, uint64_t pv) {
+  const int en = T.off[x + 1];
+  const uint64_t key = pv << 2;  // (kpk(k) < pv exactly when k < pv << 2)
+  int lo = T.off[x], n = en - lo;
+  while (n > 3) {
+    const int q = n >> 2;
+    const uint64_t k1 = T.leg[lo + q], k2 = T.leg[lo + 2 * q], k3 = T.leg[lo + 3 * q];
+    // the first leg not below pv lies behind the last of the three that is below it, and not
+    // behind the next one
+    const int j = int(k1 < key) + int(k2 < key) + int(k3 < key);
+    n = (j == 0) ? q : (j == 3) ? n - 3 * q - 1 : q - 1;
+    lo += j * q + (j ? 1 : 0);
   }
+  while (n > 0 && T.leg[lo] < key) { ++lo; --n; }
   return (lo < en && kpk(T.leg[lo]) == pv) ? lo : -1;
 }
 
-constexpr uint64_t kFpTurn = ~0ull;  // descriptor of a worm that turns round whatever the others do
+// A worm's vertex as the two legs of it, iv | ip << 16, or kTurn | its own
+// interval when it turns round whatever the others do (no leg has index 2^16 - 1)
+constexpr uint32_t kTurn = 0xffff0000u;
+__device__ __forceinline__ bool turns(uint32_t fp) { return fp >= kTurn; }
 
-// The vertex that a Step-5 move of worm w (rank r in its sub-block) in pass
-// pattern q reaches, as two words.  d0: the four intervals round the vertex,
-// each named by the leg index of its lower delimiter -- ia_dn, ia on the
-// bond's lower site a and ib_dn, ib on its upper site b (ia, ib: the vertex's
-// legs); d1: the legs ia_up, ib_up above the vertex, the bond's other site
-// (not w's) and r, 16 bits each.  d0 = kFpTurn: the worm turns round whatever
+// What a Step-5 move reaches: the vertex v ahead of the worm, on the worm's
+// own site and on the bond's other site.  Legs never move in Step 5, so all
+// of it but the vertex's states can be formed before the moves the worm waits
+// for have run.
+//
+// Lengths here are differences of the high words of the keys, in units of
+// 2^-32 of the circle (they wrap as the circle does): within one unit of the
+// true length unless they come out as 0 (which is a length below one unit, or
+// the whole circle but less than one unit).
+struct Ahead {
+  uint32_t fp;        // v's legs on the own and the other site, iv | ip << 16 (kTurn: none)
+  uint32_t dns, ups;  // the legs below and above v on both sites: i_dn | p_dn << 16, i_up | p_up << 16
+                      // (an interval is named by its lower leg: the four round v are dns and fp)
+  uint64_t kv;        // v's leg on the own site
+  uint32_t id, iu, pd, pu;      // lengths of v's legs down and up, own and other site, with no worm on them
+  uint32_t lid, liu, lpd, lpu;  // low words of the keys that end them
+  int pl, b;                    // the other site; 1 when the worm's site is the upper one of the bond
+};
+
+// The vertex that the Step-5 move of a worm (key, local site li, interval
+// L) reaches in pass pattern q.  fp >= kTurn: the worm turns round whatever
 // the other worms do (a site without legs, a temporal boundary, a bond to
 // another domain or sub-block).  Returns PMWA_EINVARIANT when the vertex has
 // no partner leg on the other site.
-__device__ int move_desc(const Tile& T, const WormRec& w, int q, int r, uint64_t& d0, uint64_t& d1) {
-  d0 = kFpTurn;
-  d1 = 0;
-  const int li = w.site;
-  const int st = T.off[li], en = T.off[li + 1];
+__device__ __forceinline__ int look_ahead(const Tile& T, uint64_t key, int li, int L, int q, Ahead& o) {
+  o.fp = kTurn | uint32_t(L);
+  const uint32_t rs = T.rng[li];
+  const int st = rs & 0xffff, en = rs >> 16;
   if (st == en) return PMWA_OK;
-  const int L = w.leg;
-  const int iv = kdir(w.key) ? ((L + 1 == en) ? st : L + 1) : L;
+  const int iv = kdir(key) ? ((L + 1 == en) ? st : L + 1) : L;
   const uint64_t kv = T.leg[iv];
-  if (ktag(kv) == 6) return PMWA_OK;
-  const int nb = T.nbr[li * 6 + ktag(kv)];
-  if (nb < 0) return PMWA_OK;
-  const int pl = nb >> 1;
-  if (T.sub[li * 4 + q] != T.sub[pl * 4 + q]) return PMWA_OK;
+  const int tag = ktag(kv);
+  if (tag == 6) return PMWA_OK;
+  const int info = T.tinfo[li * 6 + tag], pl = T.nbr[li * 6 + tag];
+  if (!((info >> (q + 2)) & 1)) return PMWA_OK;
+  const uint32_t rp = T.rng[pl];
   const int ip = T.d->use_part ? (T.part[iv] == kNone ? -1 : int(T.part[iv])) : leg_index(T, pl, kpk(kv));
   if (ip < 0) return PMWA_EINVARIANT;
-  const bool li_a = nb & 1;  // li is the bond's lower site
-  const int al = li_a ? li : pl, bl = li_a ? pl : li;
-  const int ia = li_a ? iv : ip, ib = li_a ? ip : iv;
-  const int sa = T.off[al], ea = T.off[al + 1], sb = T.off[bl], eb = T.off[bl + 1];
-  const int ia_dn = (ia == sa) ? ea - 1 : ia - 1, ib_dn = (ib == sb) ? eb - 1 : ib - 1;
-  const int ia_up = (ia + 1 == ea) ? sa : ia + 1, ib_up = (ib + 1 == eb) ? sb : ib + 1;
-  d0 = uint64_t(ia_dn) | (uint64_t(ia) << 16) | (uint64_t(ib_dn) << 32) | (uint64_t(ib) << 48);
-  d1 = uint64_t(ia_up) | (uint64_t(ib_up) << 16) | (uint64_t(pl) << 32) | (uint64_t(r) << 48);
+  const int sp = rp & 0xffff, ep = rp >> 16;
+  const int i_dn = (iv == st ? en : iv) - 1, i_up = (iv + 1 == en) ? st : iv + 1;
+  const int p_dn = (ip == sp ? ep : ip) - 1, p_up = (ip + 1 == ep) ? sp : ip + 1;
+  const uint64_t kid = T.leg[i_dn], kiu = T.leg[i_up], kpd = T.leg[p_dn], kpu = T.leg[p_up];
+  const uint32_t hv = uint32_t(kv >> 32);
+  const bool i1 = i_dn == iv, p1 = p_dn == ip;  // v alone on its site: its legs are the whole circle
+  o.id = i1 ? ~0u : hv - uint32_t(kid >> 32);
+  o.iu = i1 ? ~0u : uint32_t(kiu >> 32) - hv;
+  o.pd = p1 ? ~0u : hv - uint32_t(kpd >> 32);
+  o.pu = p1 ? ~0u : uint32_t(kpu >> 32) - hv;
+  o.lid = uint32_t(kid);
+  o.liu = uint32_t(kiu);
+  o.lpd = uint32_t(kpd);
+  o.lpu = uint32_t(kpu);
+  o.fp = uint32_t(iv) | (uint32_t(ip) << 16);
+  o.kv = kv;
+  o.dns = uint32_t(i_dn) | (uint32_t(p_dn) << 16);
+  o.ups = uint32_t(i_up) | (uint32_t(p_up) << 16);
+  o.pl = pl;
+  o.b = (info & 1) ^ 1;
   return PMWA_OK;
 }
 
-// A Step-5 move of worm w = T.W[seg[r]] (key, local site li and leg L as
-// read at the start of the pass: only its own move changes them) that
-// reaches the vertex of its descriptor (d0 != kFpTurn); seg[0..n) are the
-// worms of its sub-block, the only ones that can sit on the sub-block's
-// sites.  The worm reverses at another worm ahead of it in its interval;
-// otherwise it enters the vertex v with probability L_min / L_i (word0 >> 32
-// against the exact ratio), leaves by leg j (threshold table, low half of
-// word0) and lands on a uniform worm grid point of leg j (mulhi of word1)
-// heading away from v.  Leg l of v runs from v to the nearest event on its
-// site and side (another vertex leg or worm, the moving worm excluded; the
-// whole circle if none).  Legs are unique to their sites, so a worm's
-// interval is named by its leg alone.  The legs and worm counts the move
-// reads are loaded together up front; the vertex's two legs are updated in
-// registers and stored once.
-__device__ int tile_move_d(const Tile& T, WormRec& w, uint64_t key, int li, int L, uint64_t d0, uint64_t d1,
-                           const uint16_t* seg, int n, int r, uint64_t w0, uint64_t w1) {
+// The Step-5 move of a worm (key, site li, interval L; updated here) to the
+// vertex v of `o`.  each(f) calls f(leg, key) for (at least) every other
+// worm in v's four intervals; it is used only when there is one.  The worm
+// reverses at another worm ahead of it in its interval; otherwise it enters v
+// with probability L_min / L_i (w0 >> 32 against the exact ratio), leaves by
+// leg j (threshold table, low half of w0) and lands on a uniform worm grid
+// point of leg j (mulhi of w1) heading away from v.  Leg l of v runs from v
+// to the nearest event on its site and side (another vertex leg or worm, the
+// moving worm excluded; the whole circle if none).
+//
+// The order of the worms, L_min and the enter test are decided on the 32-bit
+// lengths wherever these leave no doubt (each within one unit of the exact
+// one); a doubt -- two times with one high word, a test within three units
+// -- costs the 64-bit computation (about 1 move in 10^8).  Only the landing
+// point needs the exact length, of leg j alone.  A domain's passes keep few
+// warps busy, so a move is one dependent chain and its cost is latency: the
+// branches are the rare cases only, the loads stand together up front.
+template <class Each>
+__device__ __forceinline__ void make_move(const Tile& T, const Ahead& o, uint64_t& key, int& li, int& L, uint64_t w0,
+                                          uint64_t w1, Each each) {
+  const int iv = int(o.fp & 0xffff), ip = int(o.fp >> 16), i_dn = int(o.dns & 0xffff), p_dn = int(o.dns >> 16);
+  const uint64_t vi = T.leg[iv], vp = T.leg[ip];
+  const int c0 = T.wcnt[i_dn], c1 = T.wcnt[p_dn], c2 = T.wcnt[iv], c3 = T.wcnt[ip];
   const bool up = kdir(key);
-  const int ia_dn = int(d0 & 0xffff), ia = int((d0 >> 16) & 0xffff);
-  const int ib_dn = int((d0 >> 32) & 0xffff), ib = int(d0 >> 48);
-  const int ia_up = int(d1 & 0xffff), ib_up = int((d1 >> 16) & 0xffff), pl = int((d1 >> 32) & 0xffff);
-  const bool li_a = (L == ia || L == ia_dn);  // the worm sits on the bond's lower site
-  const uint64_t kL = T.leg[L], va = T.leg[ia], vb = T.leg[ib];
-  const uint64_t kad = T.leg[ia_dn], kbd = T.leg[ib_dn], kau = T.leg[ia_up], kbu = T.leg[ib_up];
-  const int cL = T.wcnt[L], cia = T.wcnt[ia], cib = T.wcnt[ib], ciad = T.wcnt[ia_dn], cibd = T.wcnt[ib_dn];
-  const uint64_t pL = kpk(kL);
-  const uint64_t my = (kpk(key) - pL) & kMask62;
-  if (cL > 1) {  // other worms share the interval: is one of them ahead?
-    for (int k = 0; k < n; ++k) {
-      const WormRec& o = T.W[seg[k]];
-      if (k == r || int(o.leg) != L) continue;
-      const uint64_t off = (kpk(o.key) - pL) & kMask62;
-      if (up ? off > my : off < my) { w.key = key ^ 2u; return PMWA_OK; }
-    }
+  const uint32_t hv = uint32_t(o.kv >> 32);
+  uint32_t id = o.id, iu = o.iu, pd = o.pd, pu = o.pu;
+  uint32_t lid = o.lid, liu = o.liu, lpd = o.lpd, lpu = o.lpu;
+  int ends = 0;  // legs ended by a worm: 1 own down, 2 own up, 4 other down, 8 other up
+  bool blocked = false, doubt = false;
+  // legs by number: 0 / 1 the lower / upper site below v, 2 / 3 above
+  const int i = o.b | (up ? 0 : 2);
+  const uint32_t sa = uint32_t(o.b ? vp : vi), sb = uint32_t(o.b ? vi : vp);
+  const int S = int((sa >> 1) & 1) | int(sb & 2) | (int(sa & 1) << 2) | (int(sb & 1) << 3);
+  const uint4 th = reinterpret_cast<const uint4*>(T.th)[S * 4 + i];
+  const bool others = c2 + c3 + (i_dn != iv ? c0 : 0) + (p_dn != ip ? c1 : 0) > 1;
+  if (others) {
+    const uint32_t my = up ? hv - uint32_t(key >> 32) : uint32_t(key >> 32) - hv;  // from the worm to v
+    doubt = my == 0;
+    each([&](int lg, uint64_t ko) {
+      const uint32_t x = uint32_t(ko >> 32) - hv, y = 0u - x, lo = uint32_t(ko);  // from v up and down to the worm
+      const uint32_t z = up ? y : x;
+      blocked |= lg == L && z < my;
+      doubt |= lg == L && z == my;
+      if (lg == iv && x <= iu) { doubt |= x == iu; iu = x; liu = lo; ends |= 2; }
+      if (lg == ip && x <= pu) { doubt |= x == pu; pu = x; lpu = lo; ends |= 8; }
+      if (lg == i_dn && y <= id) { doubt |= y == id; id = y; lid = lo; ends |= 1; }
+      if (lg == p_dn && y <= pd) { doubt |= y == pd; pd = y; lpd = lo; ends |= 4; }
+    });
   }
-  const uint64_t pv = kpk(va);
-  const int al = li_a ? li : pl, bl = li_a ? pl : li;
-  const uint64_t pa_dn = kpk(kad), pb_dn = kpk(kbd);
-  // offsets from v up to the nearest object above, and from the lower leg up
-  // to the highest worm of the interval below v
-  uint64_t ua = (ia_up == ia) ? kTwo62 : ((kpk(kau) - pv) & kMask62);
-  uint64_t ub = (ib_up == ib) ? kTwo62 : ((kpk(kbu) - pv) & kMask62);
-  uint64_t da = 0, db = 0;
-  bool fa = false, fb = false;
-  // worms (other than this one) in the four intervals around v?
-  int others = cia + cib + (ia_dn != ia ? ciad : 0) + (ib_dn != ib ? cibd : 0) - 1;
-  for (int k = 0; k < n && others > 0; ++k) {
-    if (k == r) continue;
-    const WormRec& o = T.W[seg[k]];
-    const int lg = o.leg;
-    if (lg != ia && lg != ib && lg != ia_dn && lg != ib_dn) continue;
-    --others;
-    const uint64_t po = kpk(o.key);
-    if (lg == ia) { const uint64_t x = (po - pv) & kMask62; if (x < ua) ua = x; }
-    if (lg == ib) { const uint64_t x = (po - pv) & kMask62; if (x < ub) ub = x; }
-    if (lg == ia_dn) { const uint64_t x = (po - pa_dn) & kMask62; if (!fa || x > da) { da = x; fa = true; } }
-    if (lg == ib_dn) { const uint64_t x = (po - pb_dn) & kMask62; if (!fb || x > db) { db = x; fb = true; } }
+  const uint32_t z1 = uint32_t(w0 >> 32), z0 = uint32_t(w0);
+  const uint32_t lmin = min(min(id, iu), min(pd, pu));
+  // z1 L_i / 2^32 against L_min, each side within 2 units below or above
+  const long long slack = (long long)lmin - (long long)__umulhi(z1, up ? id : iu);
+  bool enter = slack >= 3;
+  doubt |= lmin < 4 || (slack < 3 && slack > -2);
+  int j = int(z0 >= th.x) + int(z0 >= th.y) + int(z0 >= th.z);
+  if (z0 == ~0u) {  // (the table holds thresholds up to 2^32 - 1: a 2^32 counts from the full one)
+    const uint64_t* t = T.d->TH + (S * 4 + i) * 4;
+    j = int(z0 >= t[0]) + int(z0 >= t[1]) + int(z0 >= t[2]);
   }
-  const uint64_t L2 = wpts(pv, (pv + ua) & kMask62);
-  const uint64_t L3 = wpts(pv, (pv + ub) & kMask62);
-  const uint64_t L0 = wpts(fa ? ((pa_dn + da) & kMask62) : pa_dn, pv);
-  const uint64_t L1 = wpts(fb ? ((pb_dn + db) & kMask62) : pb_dn, pv);
-  const int i = li_a ? (up ? 0 : 2) : (up ? 1 : 3);
-  const uint64_t Li = (i == 0) ? L0 : (i == 1) ? L1 : (i == 2) ? L2 : L3;
-  const uint64_t Lmin = min(min(L0, L1), min(L2, L3));
-  // enter iff z1 * L_i < L_min * 2^32 (96-bit comparison)
-  const uint64_t z1 = w0 >> 32, z0 = w0 & 0xffffffffull;
-  const uint64_t ph = __umul64hi(z1, Li), plo = z1 * Li;
-  const uint64_t qh = Lmin >> 32, ql = Lmin << 32;
-  if (!(ph < qh || (ph == qh && plo < ql))) { w.key = key ^ 2u; return PMWA_OK; }
-  const int S = kbl(va) | (kbl(vb) << 1) | (kab(va) << 2) | (kab(vb) << 3);
-  const uint64_t* th = T.th + (S * 4 + i) * 4;
-  const uint64_t t0 = th[0], t1 = th[1], t2 = th[2];
-  const int j = (z0 < t0) ? 0 : (z0 < t1) ? 1 : (z0 < t2) ? 2 : 3;
+  const bool ju = j >= 2, jo = ((j ^ o.b) & 1) == 0;  // leg j goes up; lies on the worm's own site
+  const int dn = jo ? i_dn : p_dn, x = jo ? iv : ip;
+  const int wj = (ends >> ((jo ? 0 : 2) + (ju ? 1 : 0))) & 1;
+  // exact length of leg j: the high-word difference and the low words, grid points times 32
+  const uint32_t hj = jo ? (ju ? iu : id) : (ju ? pu : pd), lj = (jo ? (ju ? liu : lid) : (ju ? lpu : lpd)) & ~31u;
+  const uint32_t lv = uint32_t(o.kv) & ~31u;
+  const uint64_t dj = (uint64_t(hj) << 32) + (ju ? uint64_t(lj) - lv : uint64_t(lv) - lj);
+  uint64_t Lj = (dj >> 5) - (ju ? 0 : wj);
+  if (dn == x && !wj) Lj = kTwo59;
+  if (doubt) {
+    const uint64_t pv = kpk(o.kv), my = up ? (pv - kpk(key)) & kMask62 : (kpk(key) - pv) & kMask62;
+    uint64_t E0 = wpts(kpk(T.leg[i_dn]), pv), E1 = wpts(kpk(T.leg[p_dn]), pv);
+    uint64_t E2 = wpts(pv, kpk(T.leg[o.ups & 0xffff])), E3 = wpts(pv, kpk(T.leg[o.ups >> 16]));
+    blocked = false;
+    if (others)
+      each([&](int lg, uint64_t ko) {
+        const uint64_t po = kpk(ko);
+        if (lg == L && (up ? ((pv - po) & kMask62) < my : ((po - pv) & kMask62) < my)) blocked = true;
+        if (lg == iv) E2 = min(E2, wpts(pv, po));
+        if (lg == ip) E3 = min(E3, wpts(pv, po));
+        if (lg == i_dn) E0 = min(E0, wpts(po, pv));
+        if (lg == p_dn) E1 = min(E1, wpts(po, pv));
+      });
+    // enter iff z1 * L_i < L_min * 2^32 (96-bit comparison)
+    const uint64_t Li = up ? E0 : E2, lo = uint64_t(z1) * (Li & 0xffffffffull);
+    enter = uint64_t(z1) * (Li >> 32) + (lo >> 32) < min(min(E0, E1), min(E2, E3));
+    Lj = jo ? (ju ? E2 : E0) : (ju ? E3 : E1);
+  }
+  const uint64_t at = __umul64hi(w1, Lj);
   // the worm leaves leg i and takes leg j: flip their states
-  uint64_t na = va, nb = vb;
-  if (i & 1) nb ^= (i < 2) ? 2u : 1u; else na ^= (i < 2) ? 2u : 1u;
-  if (j & 1) nb ^= (j < 2) ? 2u : 1u; else na ^= (j < 2) ? 2u : 1u;
-  T.leg[ia] = na;
-  T.leg[ib] = nb;
-  const int ix = (j & 1) ? ib : ia;
-  const uint64_t vx = (j & 1) ? nb : na;
-  const uint64_t Lj = (j == 0) ? L0 : (j == 1) ? L1 : (j == 2) ? L2 : L3;
-  const uint64_t o = __umul64hi(w1, Lj);
-  const int nl = (j >= 2) ? ix : ((j & 1) ? ib_dn : ia_dn);
-  w.key = (j >= 2) ? wkey((wm_above(pv) + o) & (kTwo59 - 1), 1, kab(vx) ^ 1)
-                   : wkey((wm_below(pv) + kTwo59 - o) & (kTwo59 - 1), 0, kbl(vx));
-  T.wcnt[L] -= 1;
-  T.wcnt[nl] += 1;
-  // site and leg in one store: a move of the same pass that runs beside this
-  // one reads either the old or the new pair
-  *reinterpret_cast<uint32_t*>(&w.site) = uint32_t((j & 1) ? bl : al) | (uint32_t(nl) << 16);
-  return PMWA_OK;
+  const uint64_t ni = vi ^ (up ? 2u : 1u) ^ (jo ? (ju ? 1u : 2u) : 0u), np = vp ^ (jo ? 0u : (ju ? 1u : 2u));
+  const uint32_t vx = uint32_t(jo ? ni : np);
+  const uint64_t tv = o.kv & ~31ull;  // (sums of grid points times 32 wrap round the circle by themselves)
+  const uint64_t to = ju ? ((tv + (at << 5)) | 30u | ((vx & 1u) ^ 1u)) : ((tv - ((at + 1) << 5)) | 28u | ((vx >> 1) & 1u));
+  if (blocked || !enter) { key ^= 2u; return; }
+  key = to;
+  T.leg[iv] = ni;
+  T.leg[ip] = np;
+  const int nl = ju ? x : dn;
+  if (nl != L) {
+    T.wcnt[L] = uint8_t((L == iv ? c2 : c0) - 1);
+    T.wcnt[nl] = uint8_t((ju ? (jo ? c2 : c3) : (jo ? c0 : c1)) + 1);
+    L = nl;
+  }
+  li = jo ? li : o.pl;
 }
 
 // per-phase cycle counters (profiling only): thread 0 adds the cycles since
@@ -388,96 +454,38 @@ __device__ __forceinline__ void phase_tick(const Dev& d, int k, long long& t) {
 // Step-5 chain of a worm in pass pattern q: its sub-block times N_beta plus
 // its temporal slab (a worm never leaves its slab: it turns round at the
 // boundaries and every leg ends there)
-__device__ __forceinline__ int worm_group(const Tile& T, const WormRec& w, int q) {
-  return int(T.sub[w.site * 4 + q]) * T.d->ntau + int(w.slab);
+__device__ __forceinline__ int worm_group(const Tile& T, int site, int slab, int q) {
+  return int(T.sub[site * 4 + q]) * T.d->ntau + slab;
 }
 
 // ---------------------------------------------------------------------------
-// Rounds of independent moves.  In a pass the worms of one sub-block move one
+// Independent moves.  In a pass the worms of one sub-block move one
 // after another in label order, and a move reads and writes nothing but its
 // own worm and the four intervals round the vertex it reaches: their worm
 // counts, the worms in them and the states of the vertex's two legs.  A worm
 // that turns round whatever the others do changes nothing another move
 // reads.  So a move need wait only for the earlier moves of its sub-block
-// whose intervals meet its own: rounds that run every move whose such
-// predecessors have run give exactly the configuration of the moves made one
-// by one.
-constexpr int kNear = 47;  // predecessors a wait mask names one by one
-constexpr uint64_t kNearMask = (1ull << kNear) - 1;
-constexpr uint16_t kPending = 0xFFFF;
-
-// do two sets of four intervals (16-bit leg indices) share one?
-__device__ __forceinline__ bool fp_meet(uint64_t a, uint64_t b) {
-  const uint32_t a0 = uint32_t(a), a1 = uint32_t(a >> 32), b0 = uint32_t(b), b1 = uint32_t(b >> 32);
-  const uint32_t c0 = __byte_perm(b0, 0, 0x1032), c1 = __byte_perm(b1, 0, 0x1032);  // halves swapped
-  return (__vcmpeq2(a0, b0) | __vcmpeq2(a0, c0) | __vcmpeq2(a0, b1) | __vcmpeq2(a0, c1) | __vcmpeq2(a1, b0) |
-          __vcmpeq2(a1, c0) | __vcmpeq2(a1, b1) | __vcmpeq2(a1, c1)) != 0;
-}
-
-// The moves of one pass (all threads).  On entry the grouped order idx[]
-// (position p = fill[u] + r holds the r-th worm of group u), each position's
-// move descriptor in rw[2p], rw[2p + 1], each worm's group in lab and
-// kPending in xr are in place.  First each worm's wait mask goes to lab:
-// bit i (i < kNear) = wait for position p - 1 - i, bits kNear.. = the group,
-// bit 63 = also wait for every position of the group more than kNear before
-// it.  Then rounds until every worm has moved, each move drawing Philox
-// block r of stream (domain * groups + u, c2) and recording its round in
-// xr.  Ends with a barrier.
-__device__ void pass_rounds(const Tile& T, int dom, int nw, uint32_t c2) {
-  const Dev& d = *T.d;
-  const int tid = threadIdx.x, NT = blockDim.x;
-  for (int p = tid; p < nw; p += NT) {
-    WormRec& w = T.W[T.idx[p]];
-    const uint64_t f = T.rw[2 * p];
-    uint64_t m = w.lab << kNear;
-    if (f != kFpTurn) {
-      const int r = int(T.rw[2 * p + 1] >> 48);
-      for (int i = 0; i < r; ++i) {
-        const uint64_t g = T.rw[2 * (p - 1 - i)];
-        if (g != kFpTurn && fp_meet(f, g)) m |= (i < kNear) ? (1ull << i) : (1ull << 63);
-      }
-    }
-    w.lab = m;
+// whose intervals meet its own: running every move as soon as its such
+// predecessors have run gives exactly the configuration of the moves made
+// one by one.
+// Do the intervals round another worm's vertex meet those round this one's?
+// On a site they share one iff the other vertex is this one or one of its
+// two neighbours there, so both legs of the other (either half of g) are held
+// against the legs below, at and above this vertex on both sites, two at a
+// time: some half word of x is zero iff (x - 0x00010001) & ~x has a half
+// word's top bit set.  For a worm that turns round, g holds its own interval
+// and the answer covers every case where that is one of the four.
+struct Meet {
+  uint32_t a0, a1, a2, c0, c1, c2;
+  __device__ __forceinline__ explicit Meet(const Ahead& o) {
+    a0 = o.dns; a1 = o.fp; a2 = o.ups;
+    c0 = (a0 << 16) | (a0 >> 16); c1 = (a1 << 16) | (a1 >> 16); c2 = (a2 << 16) | (a2 >> 16);  // halves swapped
   }
-  __syncthreads();
-  for (int round = 0;; ++round) {
-    int pending = 0;
-    for (int p = tid; p < nw; p += NT) {
-      WormRec& w = T.W[T.idx[p]];
-      if (w.xr != kPending) continue;
-      const uint64_t d0 = T.rw[2 * p];
-      if (d0 == kFpTurn) {
-        w.key ^= 2u;
-        w.xr = uint16_t(round);
-        continue;
-      }
-      const uint64_t d1 = T.rw[2 * p + 1], m = w.lab;
-      const int r = int(d1 >> 48), u = int((m >> kNear) & 0xffff);
-      bool ready = true;
-      for (uint64_t b = m & kNearMask; b && ready; b &= b - 1)
-        ready = T.W[T.idx[p - __ffsll((long long)b)]].xr < round;
-      if (ready && (m >> 63))
-        for (int j = p - r; j < p - kNear && ready; ++j) ready = T.W[T.idx[j]].xr < round;
-      if (!ready) {
-        pending = 1;
-        continue;
-      }
-      const P4 b = philox(uint32_t(r), uint32_t(dom * T.ngrp + u), c2, d.sweep, d.key0, d.key1);
-      const int rc = tile_move_d(T, w, w.key, w.site, w.leg, d0, d1, T.idx + (p - r), T.fill[u + 1] - T.fill[u], r,
-                                 uint64_t(b.x) | (uint64_t(b.y) << 32), uint64_t(b.z) | (uint64_t(b.w) << 32));
-      if (rc) tile_fail(T.misc, rc, 5);
-      w.xr = uint16_t(round);
-    }
-    if (!__syncthreads_or(pending)) {
-      if (d.phase_cycles && tid == 0) atomicAdd(d.phase_cycles + 7, (unsigned long long)(round + 1));
-      break;
-    }
-    if (round >= nw) {  // (each round moves the first waiting worm of every group: never taken)
-      if (tid == 0) tile_fail(T.misc, PMWA_EINVARIANT, 7);
-      break;
-    }
+  __device__ __forceinline__ bool operator()(uint32_t g) const {
+    auto z = [](uint32_t x) { return (x - 0x00010001u) & ~x; };
+    return ((z(a0 ^ g) | z(a1 ^ g) | z(a2 ^ g) | z(c0 ^ g) | z(c1 ^ g) | z(c2 ^ g)) & 0x80008000u) != 0;
   }
-}
+};
 
 __device__ __forceinline__ bool worm_less(const WormRec& a, const WormRec& b) {
   if (a.lab != b.lab) return a.lab < b.lab;
@@ -521,266 +529,377 @@ __device__ void label_order(const Tile& T, int nw, int* wsum) {
   __syncthreads();
 }
 
-// One warp (lane = threadIdx.x < 32) groups the nw worms of pass pattern q
-// by sub-block, keeping label order inside each group: for the worms in
-// label order, 32 at a time, the sub-block u of each (wsb), its rank among
-// the worms of u met so far (wrk; equal sub-blocks in a chunk found with
-// __match_any_sync, running counts in bkt[]), then fill[u] = first slot of
-// sub-block u (exclusive scan of the counts) and bkt[] cleared.
-__device__ void rank_pass(const Tile& T, int nw, int q, int lane) {
-  const unsigned lt = (1u << lane) - 1u;
-  for (int k0 = 0; k0 < nw; k0 += 32) {
-    const int k = k0 + lane;
-    const int u = (k < nw) ? worm_group(T, T.W[T.ord[k]], q) : -1;
-    const unsigned peers = __match_any_sync(0xffffffffu, u);
-    const int base = (u >= 0) ? T.bkt[u] : 0;
-    __syncwarp();
-    if (u >= 0) {
-      T.wsb[k] = uint16_t(u);
-      T.wrk[k] = uint16_t(base + __popc(peers & lt));
-      if ((peers & lt) == 0) T.bkt[u] = base + __popc(peers);
-    }
-    __syncwarp();
-  }
-  const int n = T.ngrp;
-  const int chunk = (n + 31) / 32;
-  const int lo = min(n, lane * chunk), hi = min(n, lo + chunk);
-  int sum = 0;
-  for (int i = lo; i < hi; ++i) sum += T.bkt[i];
-  int v = sum;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int x = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v += x;
-  }
-  int run = v - sum;
-  for (int i = lo; i < hi; ++i) {
-    const int x = T.bkt[i];
-    T.fill[i] = run;
-    run += x;
-    T.bkt[i] = 0;
-  }
-  if (lane == 31) T.fill[n] = v;
+// The groups of a pass.  A worm that looks ahead for pass p joins its group u:
+// it takes the next place of the group's table of kGroupSlots worm numbers
+// (numbers in label order), or, when those are taken, puts itself at the head
+// of the group's linked list (hd[u] = stamp << 16 | k, the stamp being p + 1,
+// so that the heads need no clearing; nxt[k] the worm it found there).
+// Two-by-two sub-blocks hold one to five worms: the table brings a group's
+// members in one go, where a list is one dependent load after the other.
+// Tables and lists alternate between two buffers, the counts between three
+// (a pass clears the one that the pass after the next fills).
+__device__ __forceinline__ void join_list(const Tile& T, int k, int u, int pass) {
+  const uint32_t stamp = uint32_t(pass + 1);
+  const uint32_t was = atomicExch(T.hd + (pass & 1) * T.hstride + u, (stamp << 16) | uint32_t(k));
+  T.nxt[(pass & 1) * T.d->wcap + k] = (was >> 16) == stamp ? uint16_t(was) : kNone;
 }
 
-// The grouping of rank_pass by the whole block, for nw <= blockDim.x worms,
-// in two halves around a block barrier (called by every thread).  Warp c ranks the
-// 32 worms of chunk c of the label order among themselves (__match_any_sync)
-// and its group leaders record the chunk's count of each sub-block in
-// cnt[c][u], stamped with pass_stamp(pass) (an entry with another stamp
-// counts 0; the table is cleared every 255 passes, so a stale stamp never
-// matches).
-// After the barrier every worm adds the counts of the earlier chunks to its
-// rank, while one warp forms fill[] from the totals: the last warp when it
-// holds no worms, else warp 0 (whose worms add nothing).  The worm of thread
-// k = threadIdx.x gets its sub-block u (-1: no worm) and rank r; fill comes
-// out as rank_pass makes it (after a barrier); bkt[] is scratch.
-__device__ __forceinline__ int pass_stamp(int pass) { return ((pass % 255) + 1) << 8; }
-
-// (before the barrier: the chunk ranks and counts)
-__device__ void rank_chunk(const Tile& T, int nw, int q, int pass, int& u, int& r) {
-  const int tid = threadIdx.x, c = tid >> 5, lane = tid & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  const int W = (nw + 31) >> 5, n = T.ngrp;
-  const int stamp = pass_stamp(pass);
-  u = -1;
-  r = 0;
-  if (c < W) {  // warp-uniform
-    u = (tid < nw) ? worm_group(T, T.W[T.ord[tid]], q) : -1;
-    const unsigned peers = __match_any_sync(0xffffffffu, u);
-    r = __popc(peers & lt);
-    if (u >= 0 && (peers & lt) == 0) T.cnt[c * n + u] = uint16_t(stamp | __popc(peers));
-  }
+// a worm's site and interval in one store: a move that runs beside this
+// one's reads either the old or the new pair
+__device__ __forceinline__ void store_place(WormRec& w, int li, int L) {
+  *reinterpret_cast<uint32_t*>(&w.site) = uint32_t(li) | (uint32_t(L) << 16);
 }
 
-// (after the barrier: the earlier chunks' counts, and fill[])
-__device__ void rank_finish(const Tile& T, int nw, int pass, int u, int& r) {
-  const int tid = threadIdx.x, c = tid >> 5, lane = tid & 31;
-  const int W = (nw + 31) >> 5, n = T.ngrp;
-  const int stamp = pass_stamp(pass);
-  if (c > 0 && u >= 0) {
-    for (int c2 = 0; c2 < c; ++c2) {
-      const int v = T.cnt[c2 * n + u];
-      if ((v & ~0xff) == stamp) r += v & 0xff;
-    }
-  }
-  const int nwarps = int(blockDim.x) >> 5;
-  if (c == (W < nwarps ? nwarps - 1 : 0)) {
-    const int chunk = (n + 31) / 32;
-    const int lo = min(n, lane * chunk), hi = min(n, lo + chunk);
-    int sum = 0;
-    for (int i = lo; i < hi; ++i) {
-      int tot = 0;
-      for (int c2 = 0; c2 < W; ++c2) {
-        const int v = T.cnt[c2 * n + i];
-        if ((v & ~0xff) == stamp) tot += v & 0xff;
-      }
-      T.bkt[i] = tot;
-      sum += tot;
-    }
-    int v = sum;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += x;
-    }
-    int run = v - sum;
-    for (int i = lo; i < hi; ++i) {
-      T.fill[i] = run;
-      run += T.bkt[i];
-      T.bkt[i] = 0;
-    }
-    if (lane == 31) T.fill[n] = v;
-  }
-}
+constexpr int kSpinLimit = 1 << 20;  // polls of a predecessor before the pass gives up (never reached)
+constexpr int kGroupSlots = 8;       // worms of a group's table (16 bits each)
 
-// One pass when every worm has a thread (32 < nw <= blockDim.x; called by
-// every thread, ends with a barrier).  Thread k holds the k-th worm of the
-// label order from its grouping to its move: the worm's key, site and leg,
-// its move descriptor, its rank r in its group u, its wait mask and its
-// Philox block r of stream (domain * groups + u, c2) stay in registers.
-// Other threads read only the descriptor's intervals (rw[at], for the wait
-// masks) and the round of each position's move (wsb[at], kPending until it
-// has moved), at its grouped position at = fill[u] + r.  The wait mask:
-// bit i < 63 = wait for position at - 1 - i; bit 63 = also wait for every
-// position of the group at least 64 before.  tclk: the phase clock (set-up
-// to counter 5, moves to counter 6).
-__device__ void pass_fast(const Tile& T, int dom, int nw, int q, int pass, uint32_t c2, long long& tclk) {
+// All N_cycle passes of a domain whose 32 < nw <= blockDim.x worms have a
+// thread each (called by all threads); W[] is in label order and a thread
+// keeps its worm k in registers throughout.  The worms are spread over the
+// warps, at least 16 a warp: a warp's loops run as long as its slowest lane's,
+// but more warps issue more instructions.
+//
+// A pass has one barrier.  Behind it every worm goes through its group once,
+// for its rank r (the members with a smaller k) and for the members whose
+// intervals meet its own (nn of them, the first four in `mem`, 16 bits each),
+// draws its Philox block and moves as soon as the earlier ones of those (bits
+// of `deps`) have set their flag dn[] -- no round waits for the slowest worm
+// of the domain.  What it reaches in the next pass depends on its own place
+// and on leg times alone, so it looks ahead and joins its next group right
+// after its move, while other worms still move.
+//
+// A worm with more than four such neighbours goes through the members again
+// at each use.  In a domain with few large groups (sub_block 0: one) going
+// through a group costs more than the moves; there the worms enter their
+// vertex's two legs (one that turns: its interval) in a hash table of chains,
+// entry 2 k + side with its successors in W[k].lab, and a worm looks up the
+// six legs whose owners' intervals can meet its own.  Its rank is k with one
+// group, else counted over the group numbers in nxt[].
+__device__ void block_passes(const Tile& T, int dom, int nw, long long& tclk) {
   const Dev& d = *T.d;
-  const int tid = threadIdx.x, NT = blockDim.x;
-  if (pass > 0 && pass % 255 == 0) {  // the stamps start over: no entry may carry one
-    for (int i = tid; i < (NT >> 5) * T.ngrp; i += NT) T.cnt[i] = 0;
-    __syncthreads();
-  }
-  int u, r;
-  rank_chunk(T, nw, q, pass, u, r);
-  const bool act = u >= 0;
-  int wi = 0, li = 0, L = 0, rc = PMWA_OK;
-  uint64_t key = 0, d0 = kFpTurn, d1 = 0;
+  const int nwarps = int(blockDim.x) >> 5, per = max(16, (nw + nwarps - 1) / nwarps), lane = threadIdx.x & 31;
+  const int k = (int(threadIdx.x) >> 5) * per + lane;
+  const bool act = lane < per && k < nw, scan = nw > 12 * T.ngrp, table = d.gtab && !scan, hash = scan && d.ghash;
+  uint64_t key = 0;
+  int li = 0, L = 0, slab = 0, u = 0, u_old = 0;
+  Ahead o;
+  o.fp = kTurn;
+  // (a status found while pass p is prepared or run is read after the next
+  // barrier by all threads alike: two flags in turn)
+  auto fail = [&](int pass, int rc) { T.perr[pass & 1] = rc; };
+  auto prepare = [&](int pass, int b3) {
+    u = worm_group(T, li, slab, pass & 3);
+    const int at = table ? atomicAdd(T.gcnt + b3 * T.ngrp + u, 1) : kGroupSlots;
+    const int rc = look_ahead(T, key, li, L, pass & 3, o);
+    if (rc) fail(pass, rc);
+    T.fp[(pass & 1) * d.wcap + k] = o.fp;
+    if (hash) {
+      const uint32_t stamp = uint32_t(pass + 1);
+      uint32_t* hh = T.hash + (pass & 1) * d.ghash;
+      uint16_t* next = reinterpret_cast<uint16_t*>(&T.W[k].lab) + 2 * (pass & 1);
+      for (int e = 0; e < (turns(o.fp) ? 1 : 2); ++e) {
+        const uint32_t leg = (e ? o.fp >> 16 : o.fp) & 0xffffu;
+        const uint32_t was = atomicExch(hh + (leg & (d.ghash - 1)), (stamp << 16) | uint32_t(2 * k + e));
+        next[e] = (was >> 16) == stamp ? uint16_t(was) : kNone;
+      }
+    }
+    if (at < kGroupSlots) T.cell[((pass & 1) * T.ngrp + u) * kGroupSlots + at] = uint16_t(k);
+    else if (scan) T.nxt[(pass & 1) * d.wcap + k] = uint16_t(u);
+    else join_list(T, k, u, pass);
+  };
   if (act) {
-    wi = T.ord[tid];
-    const WormRec& w = T.W[wi];
+    const WormRec& w = T.W[k];
     key = w.key;
     li = w.site;
     L = w.leg;
-    rc = move_desc(T, w, q, 0, d0, d1);
+    slab = w.slab;
+    prepare(0, 0);
   }
-  __syncthreads();
-  rank_finish(T, nw, pass, u, r);
-  __syncthreads();
-  int at = 0, lo = 0, n = 0;
-  uint64_t w0 = 0, w1 = 0;
-  if (act) {
-    lo = T.fill[u];
-    n = T.fill[u + 1] - lo;
-    at = lo + r;
-    T.idx[at] = uint16_t(wi);
-    T.rw[at] = d0;
-    T.wsb[at] = kPending;
-    if (rc) tile_fail(T.misc, rc, 5);
-    if (d0 != kFpTurn) {
-      const P4 b = philox(uint32_t(r), uint32_t(dom * T.ngrp + u), c2, d.sweep, d.key0, d.key1);
+  volatile uint16_t* dn = T.dn;
+  int b3 = 0;  // pass % 3
+  for (int pass = 0; pass < d.n_cycle; ++pass) {
+    __syncthreads();
+    if (const int rc = T.perr[pass & 1]) {
+      tile_fail(T.misc, rc, 5);
+      return;
+    }
+    const int stamp = pass + 1;
+    const uint32_t* fp = T.fp + (pass & 1) * d.wcap;
+    const uint16_t* nxt = T.nxt + (pass & 1) * d.wcap;
+    const uint16_t* cell = T.cell + ((pass & 1) * T.ngrp + u) * kGroupSlots;
+    const Meet meet(o);
+    bool moved = !act;
+    int r = 0, nn = 0, n = 0;  // n: members in the table
+    bool list = false;         // some members are in the list
+    uint32_t deps = 0;
+    uint64_t mem = 0, w0 = 0, w1 = 0;
+    const int b3n = b3 == 2 ? 0 : b3 + 1, b3p = b3 == 0 ? 2 : b3 - 1;
+    if (act && turns(o.fp)) {
+      key ^= 2u;
+      moved = true;
+    }
+    auto look_at = [&](int j, uint32_t g) {
+      const bool m = meet(g) && j != k;
+      r += j < k ? 1 : 0;
+      nn += m ? 1 : 0;
+      mem = m ? (mem << 16) | uint64_t(j) : mem;
+      deps = m ? (deps << 1) | (j < k && !turns(g) ? 1u : 0u) : deps;
+    };
+    // every member again, for a worm with more than four neighbours
+    auto again = [&](auto f) {
+      if (scan) {
+        for (int j = 0; j < nw; ++j)
+          if (nxt[j] == u) f(j);
+      }
+      for (int e = 0; e < n; ++e) f(int(cell[e]));
+      if (list)
+        for (int j = int(T.hd[(pass & 1) * T.hstride + u] & 0xffff); j != kNone; j = nxt[j]) f(j);
+    };
+    if (!moved) {
+      if (table) {
+        const int c = T.gcnt[b3 * T.ngrp + u];
+        n = min(c, kGroupSlots);
+        list = c > kGroupSlots;
+      } else {
+        list = !scan;
+      }
+      for (int e0 = 0; e0 < n; e0 += 4) {
+        const uint2 four = *reinterpret_cast<const uint2*>(cell + e0);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int j = int(((e < 2 ? four.x : four.y) >> (16 * (e & 1))) & 0xffff);
+          if (e0 + e < n) look_at(j, fp[j]);
+        }
+      }
+      if (list)
+        for (int j = int(T.hd[(pass & 1) * T.hstride + u] & 0xffff); j != kNone; j = nxt[j]) look_at(j, fp[j]);
+      if (hash) {
+        const uint32_t* hh = T.hash + (pass & 1) * d.ghash;
+        r = k;
+        if (T.ngrp > 1) {
+          r = 0;
+          for (int j = 0; j < k; ++j) r += nxt[j] == u ? 1 : 0;
+        }
+        mem = ~0ull;
+        for (int s = 0; s < 6; ++s) {
+          const uint32_t pair = s < 2 ? o.dns : s < 4 ? o.fp : o.ups, leg = (s & 1) ? pair >> 16 : pair & 0xffffu;
+          const uint32_t h = hh[leg & (d.ghash - 1)];
+          int e = (h >> 16) == uint32_t(stamp) ? int(h & 0xffff) : kNone;
+          while (e != kNone) {
+            const int j = e >> 1;
+            const uint32_t g = fp[j];
+            if (((e & 1) ? g >> 16 : g & 0xffffu) == leg && j != k) {
+              // (a worm can be found by both of its legs)
+              const uint64_t x = mem ^ (uint64_t(j) * 0x0001000100010001ull);
+              if (!((x - 0x0001000100010001ull) & ~x & 0x8000800080008000ull)) {
+                mem = (mem << 16) | uint64_t(j);
+                deps = (deps << 1) | (j < k && !turns(g) ? 1u : 0u);
+                ++nn;
+              }
+            }
+            e = reinterpret_cast<const uint16_t*>(&T.W[j].lab)[2 * (pass & 1) + (e & 1)];
+          }
+        }
+      } else if (scan) {
+        for (int j = 0; j < nw; ++j)
+          if (nxt[j] == u) look_at(j, fp[j]);
+      }
+      const P4 b = philox(uint32_t(r), uint32_t(dom * T.ngrp + u), c2_word(kScatter, uint32_t(pass), d.replica),
+                          d.sweep, d.key0, d.key1);
       w0 = uint64_t(b.x) | (uint64_t(b.y) << 32);
       w1 = uint64_t(b.z) | (uint64_t(b.w) << 32);
     }
+    if (act && table && pass > 0) T.gcnt[b3p * T.ngrp + u_old] = 0;
+    u_old = u;
+    phase_tick(d, 5, tclk);
+    int spin = 0;
+    while (!__all_sync(0xffffffffu, moved)) {
+      if (!moved) {
+        bool ready = true;
+        if (nn <= 4) {
+          for (uint32_t m = deps; m; m &= m - 1)
+            ready = ready && dn[(mem >> (16 * (__ffs(int(m)) - 1))) & 0xffff] == stamp;
+        } else {
+          again([&](int j) {
+            if (j < k && !turns(fp[j]) && meet(fp[j])) ready = ready && dn[j] == stamp;
+          });
+        }
+        if (ready) {
+          __threadfence_block();
+          make_move(T, o, key, li, L, w0, w1, [&](auto f) {
+            if (nn <= 4) {
+              for (int e = 0; e < nn; ++e) {
+                const WormRec& w = T.W[(mem >> (16 * e)) & 0xffff];
+                f(int(w.leg), w.key);
+              }
+            } else {
+              again([&](int j) {
+                if (j != k) f(int(T.W[j].leg), T.W[j].key);
+              });
+            }
+          });
+          WormRec& w = T.W[k];
+          w.key = key;
+          store_place(w, li, L);
+          __threadfence_block();
+          dn[k] = uint16_t(stamp);
+          moved = true;
+        }
+      }
+      if (++spin > kSpinLimit) { fail(pass + 1, PMWA_ETIMEOUT); break; }
+    }
+    if (d.phase_cycles && threadIdx.x == 0) atomicAdd(d.phase_cycles + 7, (unsigned long long)spin);
+    phase_tick(d, 6, tclk);
+    if (act && pass + 1 < d.n_cycle) prepare(pass + 1, b3n);
+    b3 = b3n;
   }
   __syncthreads();
-  phase_tick(d, 5, tclk);
-  uint64_t m = 0;
-  if (act && d0 != kFpTurn)
-    for (int i = 0; i < r; ++i) {
-      const uint64_t g = T.rw[at - 1 - i];
-      if (g != kFpTurn && fp_meet(d0, g)) m |= (i < 63) ? (1ull << i) : (1ull << 63);
+  if (const int rc = T.perr[d.n_cycle & 1]) tile_fail(T.misc, rc, 5);
+  if (act) T.W[k].key = key;
+}
+
+// All N_cycle passes of a domain with more worms than threads (all threads).
+// As block_passes, with the worms of a thread taken in turn, their state in
+// W[ord[k]] and rounds ended by a block barrier: every round moves the worms
+// whose predecessors have moved.
+__device__ void many_passes(const Tile& T, int dom, int nw, long long& tclk) {
+  const Dev& d = *T.d;
+  const int tid = threadIdx.x, NT = blockDim.x;
+  volatile uint16_t* dn = T.dn;
+  for (int pass = 0; pass < d.n_cycle; ++pass) {
+    const int q = pass & 3, stamp = pass + 1;
+    uint32_t* fp = T.fp + (pass & 1) * d.wcap;
+    const uint16_t* nxt = T.nxt + (pass & 1) * d.wcap;
+    for (int k = tid; k < nw; k += NT) {
+      WormRec& w = T.W[T.ord[k]];
+      join_list(T, k, worm_group(T, w.site, w.slab, q), pass);
+      Ahead o;
+      const int rc = look_ahead(T, w.key, w.site, w.leg, q, o);
+      fp[k] = o.fp;
+      if (rc) tile_fail(T.misc, rc, 5);
+      if (turns(o.fp)) w.key ^= 2u;
     }
-  bool done = !act;
-  for (int round = 0;; ++round) {
-    int pending = 0;
-    if (!done) {
-      bool ready = true;
-      for (uint64_t b = m & ~(1ull << 63); b && ready; b &= b - 1) ready = T.wsb[at - __ffsll((long long)b)] < round;
-      if (ready && (m >> 63))
-        for (int j = lo; j < at - 63 && ready; ++j) ready = T.wsb[j] < round;
-      if (ready) {
-        WormRec& w = T.W[wi];
-        if (d0 == kFpTurn) {
-          w.key = key ^ 2u;
-        } else {
-          const int rc2 = tile_move_d(T, w, key, li, L, d0, d1, T.idx + lo, n, r, w0, w1);
-          if (rc2) tile_fail(T.misc, rc2, 5);
+    __syncthreads();
+    phase_tick(d, 5, tclk);
+    for (int round = 0;; ++round) {
+      int pending = 0;
+      for (int k = tid; k < nw; k += NT) {
+        if (turns(fp[k]) || dn[k] == stamp) continue;
+        WormRec& w = T.W[T.ord[k]];
+        const int u = worm_group(T, w.site, w.slab, q), head = int(T.hd[(pass & 1) * T.hstride + u] & 0xffff);
+        uint64_t key = w.key;
+        int li = w.site, L = w.leg;
+        Ahead o;
+        look_ahead(T, key, li, L, q, o);
+        const Meet meet(o);
+        bool ready = true;
+        int r = 0;
+        for (int j = head; j != kNone; j = nxt[j]) {
+          if (j >= k) continue;
+          ++r;
+          if (!turns(fp[j]) && meet(fp[j])) ready = ready && dn[j] == stamp;
         }
-        T.wsb[at] = uint16_t(round);
-        done = true;
-      } else {
-        pending = 1;
+        if (!ready) { pending = 1; continue; }
+        __threadfence_block();
+        const P4 b = philox(uint32_t(r), uint32_t(dom * T.ngrp + u), c2_word(kScatter, uint32_t(pass), d.replica),
+                            d.sweep, d.key0, d.key1);
+        make_move(T, o, key, li, L, uint64_t(b.x) | (uint64_t(b.y) << 32), uint64_t(b.z) | (uint64_t(b.w) << 32),
+                  [&](auto f) {
+                    for (int j = head; j != kNone; j = nxt[j])
+                      if (j != k) f(int(T.W[T.ord[j]].leg), T.W[T.ord[j]].key);
+                  });
+        w.key = key;
+        store_place(w, li, L);
+        __threadfence_block();
+        dn[k] = uint16_t(stamp);
+      }
+      if (!__syncthreads_or(pending)) {
+        if (d.phase_cycles && tid == 0) atomicAdd(d.phase_cycles + 7, (unsigned long long)(round + 1));
+        break;
+      }
+      if (round >= nw) {  // (each round moves the first waiting worm of every group: never taken)
+        if (tid == 0) tile_fail(T.misc, PMWA_EINVARIANT, 7);
+        break;
       }
     }
-    if (!__syncthreads_or(pending)) {
-      if (d.phase_cycles && tid == 0) atomicAdd(d.phase_cycles + 7, (unsigned long long)(round + 1));
-      break;
-    }
-    if (round >= nw) {  // (each round moves the first waiting worm of every group: never taken)
-      if (tid == 0) tile_fail(T.misc, PMWA_EINVARIANT, 7);
-      break;
-    }
+    phase_tick(d, 6, tclk);
+    __syncthreads();
+    if (T.misc->err) return;
   }
-  phase_tick(d, 6, tclk);
 }
 
 // All N_cycle passes of a domain holding nw <= 32 worms, run by one warp
-// (lane = threadIdx.x < 32) with no block barrier.  Lane k holds the k-th
-// worm in label order; __match_any_sync over the groups gives each worm its
-// rank r in its group, and the r-th move of a group draws Philox block r,
-// as in the block-wide passes.  Each lane forms its move's descriptor (the
-// intervals go through rw[lane]); a lane waits for the lanes of its group of
-// lower rank whose intervals meet its own, and rounds move every lane whose
-// waits are over (at most 32 rounds: the first waiting lane of each group
-// waits for nobody), which gives each group's moves made one by one in rank
-// order.  Returns a status (the same for all lanes).
+// (lane = threadIdx.x < 32) with no block barrier.  Lane k holds worm k of the
+// label order (W[] is in that order).  __match_any_sync over the groups gives
+// the lanes of its group and its rank r (the r-th move of a group draws Philox
+// block r, as in the block-wide passes); the vertices go through fp[lane] and
+// tell a lane which of them meet its own intervals.  It waits for those of
+// lower rank, and rounds move every lane whose waits are over (at most 32
+// rounds: the first waiting lane of each group waits for nobody), which gives
+// each group's moves made one by one in rank order.  Returns a status (the
+// same for all lanes).
 __device__ int small_passes(const Tile& T, int dom, int nw, int lane) {
   const Dev& d = *T.d;
   const unsigned lt = (1u << lane) - 1u;
   const bool act = lane < nw;
-  const int w = act ? T.ord[lane] : 0;
+  uint64_t key = 0;
+  int li = 0, L = 0, slab = 0, rc = PMWA_OK;
+  if (act) {
+    const WormRec& w = T.W[lane];
+    key = w.key;
+    li = w.site;
+    L = w.leg;
+    slab = w.slab;
+  }
   for (int pass = 0; pass < d.n_cycle; ++pass) {
     const int q = pass & 3;
-    const int u = act ? worm_group(T, T.W[w], q) : 0x7fffffff;
-    const unsigned peers = __match_any_sync(0xffffffffu, u);
-    const int r = __popc(peers & lt), n = __popc(peers);
-    int less = 0;  // worms of groups numbered below u: the start of u's group
-    for (int j = 0; j < 32; ++j) less += (__shfl_sync(0xffffffffu, u, j) < u) ? 1 : 0;
-    int rc = PMWA_OK, li = 0, L = 0;
-    uint64_t key = 0, d0 = kFpTurn, d1 = 0, w0 = 0, w1 = 0;
+    int u = -1 - lane;
+    Ahead o;
+    o.fp = kTurn;
     if (act) {
-      T.idx[less + r] = uint16_t(w);
-      const WormRec& wr = T.W[w];
-      key = wr.key;
-      li = wr.site;
-      L = wr.leg;
-      rc = move_desc(T, wr, q, r, d0, d1);
-      if (d0 != kFpTurn) {
-        const P4 b = philox(uint32_t(r), uint32_t(dom * T.ngrp + u), c2_word(kScatter, uint32_t(pass), d.replica),
-                            d.sweep, d.key0, d.key1);
-        w0 = uint64_t(b.x) | (uint64_t(b.y) << 32);
-        w1 = uint64_t(b.z) | (uint64_t(b.w) << 32);
-      }
-      T.rw[lane] = d0;
+      u = worm_group(T, li, slab, q);
+      rc = look_ahead(T, key, li, L, q, o);
     }
+    const unsigned peers = __match_any_sync(0xffffffffu, u);
+    uint32_t* fp = T.fp + (pass & 1) * d.wcap;  // (two buffers: a slow lane may still read the last pass's)
+    if (act) fp[lane] = o.fp;
+    const bool turn = turns(o.fp);
+    const Meet meet(o);
+    const unsigned turning = __ballot_sync(0xffffffffu, turn);
     __syncwarp();
-    unsigned wait = 0;  // lanes this move waits for
-    if (act && d0 != kFpTurn)
-      for (unsigned m = peers & lt; m; m &= m - 1) {
+    unsigned near = 0;  // lanes whose intervals meet this one's, two at a time
+    if (!turn)
+      for (unsigned m = peers & ~(1u << lane); m;) {
         const int j = __ffs(int(m)) - 1;
-        const uint64_t g = T.rw[j];
-        if (g != kFpTurn && fp_meet(d0, g)) wait |= 1u << j;
+        m &= m - 1;
+        const int i = m ? __ffs(int(m)) - 1 : j;
+        m &= m - 1;
+        const uint32_t gj = fp[j], gi = fp[i];
+        near |= (meet(gj) ? 1u : 0u) << j | (meet(gi) ? 1u : 0u) << i;
       }
-    bool moved = !act;
-    unsigned done = __ballot_sync(0xffffffffu, moved);
+    bool moved = turn;
+    uint64_t w0 = 0, w1 = 0;
+    if (!turn) {
+      const P4 b = philox(uint32_t(__popc(peers & lt)), uint32_t(dom * T.ngrp + u),
+                          c2_word(kScatter, uint32_t(pass), d.replica), d.sweep, d.key0, d.key1);
+      w0 = uint64_t(b.x) | (uint64_t(b.y) << 32);
+      w1 = uint64_t(b.z) | (uint64_t(b.w) << 32);
+    } else {
+      key ^= 2u;
+    }
+    const unsigned wait = near & lt & ~turning;
+    unsigned done = turning;
     while (done != 0xffffffffu) {
       if (!moved && (wait & ~done) == 0) {
-        WormRec& wr = T.W[w];
-        if (d0 == kFpTurn) {
-          wr.key = key ^ 2u;
-        } else if (rc == PMWA_OK) {
-          rc = tile_move_d(T, wr, key, li, L, d0, d1, T.idx + less, n, r, w0, w1);
-        }
+        make_move(T, o, key, li, L, w0, w1, [&](auto f) {
+          for (unsigned m = near; m; m &= m - 1) {
+            const int j = __ffs(int(m)) - 1;
+            f(int(T.W[j].leg), T.W[j].key);
+          }
+        });
+        WormRec& w = T.W[lane];
+        w.key = key;
+        store_place(w, li, L);
         moved = true;
       }
       __syncwarp();
@@ -788,8 +907,8 @@ __device__ int small_passes(const Tile& T, int dom, int nw, int lane) {
     }
     const unsigned bad = __ballot_sync(0xffffffffu, rc != PMWA_OK);
     if (bad) return __shfl_sync(0xffffffffu, rc, __ffs(int(bad)) - 1);
-    __syncwarp();
   }
+  if (act) T.W[lane].key = key;
   return PMWA_OK;
 }
 
@@ -880,11 +999,13 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
                                           int* wsum) {
   Tile T;
   T.d = &d;
-  T.th = reinterpret_cast<uint64_t*>(sm + d.sm_th);
+  T.th = reinterpret_cast<uint32_t*>(sm + d.sm_th);
   T.off = reinterpret_cast<int*>(sm + d.sm_off);
   T.base = reinterpret_cast<uint8_t*>(sm + d.sm_base);
   T.bcnt = reinterpret_cast<int*>(sm + d.sm_bcnt);
+  T.rng = reinterpret_cast<uint32_t*>(T.bcnt);
   T.boff = reinterpret_cast<int*>(sm + d.sm_boff);
+  T.perr = T.boff;
   T.misc = reinterpret_cast<Misc*>(sm + d.sm_misc);
   T.leg = reinterpret_cast<uint64_t*>(sm + d.sm_leg);
   T.wcnt = reinterpret_cast<uint8_t*>(sm + d.sm_wcnt);
@@ -893,13 +1014,17 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
   T.W = reinterpret_cast<WormRec*>(sm + d.sm_worm);
   T.idx = reinterpret_cast<uint16_t*>(sm + d.sm_idx);
   T.ord = reinterpret_cast<uint16_t*>(sm + d.sm_ord);
-  T.wsb = reinterpret_cast<uint16_t*>(sm + d.sm_wsb);
-  T.wrk = reinterpret_cast<uint16_t*>(sm + d.sm_wrk);
-  T.rw = reinterpret_cast<uint64_t*>(sm + d.sm_rw);
+  T.dn = reinterpret_cast<uint16_t*>(sm + d.sm_dn);
+  T.nxt = reinterpret_cast<uint16_t*>(sm + d.sm_nxt);
+  T.fp = reinterpret_cast<uint32_t*>(sm + d.sm_fp);
   T.bkt = reinterpret_cast<int*>(sm + d.sm_bkt);
-  T.cnt = reinterpret_cast<uint16_t*>(sm + d.sm_cnt);
   T.fill = reinterpret_cast<int*>(sm + d.sm_fill);
-  T.nbr = reinterpret_cast<int16_t*>(sm + d.sm_nbr);
+  T.gcnt = reinterpret_cast<int*>(sm + d.sm_gcnt);
+  T.hash = reinterpret_cast<uint32_t*>(sm + d.sm_hash);
+  T.cell = reinterpret_cast<uint16_t*>(sm + d.sm_cell);
+  T.hd = reinterpret_cast<uint32_t*>(T.bkt);
+  T.hstride = (d.sm_fill - d.sm_bkt) / int(sizeof(int));
+  T.nbr = reinterpret_cast<uint16_t*>(sm + d.sm_nbr);
   T.tinfo = reinterpret_cast<uint8_t*>(sm + d.sm_tinfo);
   T.sub = reinterpret_cast<uint16_t*>(sm + d.sm_sub);
   T.soff = reinterpret_cast<int*>(sm + d.sm_soff);
@@ -923,24 +1048,29 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
     if (n) prefetch_l2(d.keyA + size_t(s) * d.cap, uint32_t((n * 8 + 15) & ~15));
   }
   const ZigTab Z = zig_stage(sm + d.sm_zig, d.zig_cap, d.worm_tries);
-  for (int k = tid; k < 256; k += NT) T.th[k] = d.TH[k];
+  for (int k = tid; k < 256; k += NT) T.th[k] = d.TH[k] >> 32 ? ~0u : uint32_t(d.TH[k]);
   if (tid == 0) { misc->pool_used = 0; misc->nworms = 0; misc->err = 0; misc->where = 0; }
   for (int k = tid; k < d.ntau; k += NT) misc->wslab[k] = 0;
   // per-site tables: bond partners by leg tag, sub-blocks by offset pattern
+  for (int li = tid; li < nds; li += NT)
+    for (int q = 0; q < 4; ++q) T.sub[li * 4 + q] = uint16_t(T.sub_of(li, q));
+  __syncthreads();
   for (int li = tid; li < nds; li += NT) {
-    for (int t = 0; t < 6; ++t) { T.nbr[li * 6 + t] = -1; T.tinfo[li * 6 + t] = 0; }
+    for (int t = 0; t < 6; ++t) { T.nbr[li * 6 + t] = 0; T.tinfo[li * 6 + t] = 0; }
     const int s = T.gsite(li);
     for (int j = 0; j < 4; ++j) {
       const int dir = j & 1;
       const int a = (j < 2) ? s : site_step(d, s, dir, -1);
       const int tg = bond_tag(d, a, dir);
       const bool out = boundary_bond(d, a, dir);
-      T.tinfo[li * 6 + tg] = uint8_t((j < 2 ? 1 : 0) | (out ? 2 : 0));
-      if (out) continue;
-      const int other = (j < 2) ? site_step(d, s, dir, +1) : a;
-      T.nbr[li * 6 + tg] = int16_t((T.lsite(other) << 1) | (j < 2 ? 1 : 0));
+      int info = (j < 2 ? 1 : 0) | (out ? 2 : 0);
+      if (!out) {
+        const int lo = T.lsite((j < 2) ? site_step(d, s, dir, +1) : a);
+        T.nbr[li * 6 + tg] = uint16_t(lo);
+        for (int q = 0; q < 4; ++q) info |= T.sub[li * 4 + q] == T.sub[lo * 4 + q] ? 4 << q : 0;
+      }
+      T.tinfo[li * 6 + tg] = uint8_t(info);
     }
-    for (int q = 0; q < 4; ++q) T.sub[li * 4 + q] = uint16_t(T.sub_of(li, q));
   }
   __syncthreads();
 
@@ -1077,9 +1207,8 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
         while (T.off[li + 1] <= j) ++li;
         const uint64_t key = T.leg[j];
         if (ktag(key) == 6) continue;  // a temporal boundary
-        const int nb = T.nbr[li * 6 + ktag(key)];
-        if (nb < 0 || (nb & 1) == 0) continue;
-        const int ip = leg_index(T, nb >> 1, kpk(key));
+        if ((T.tinfo[li * 6 + ktag(key)] & 3) != 1) continue;  // (inside the domain, seen from its lower site)
+        const int ip = leg_index(T, T.nbr[li * 6 + ktag(key)], kpk(key));
         if (ip < 0) { tile_fail(misc, PMWA_EINVARIANT, 34); continue; }
         T.part[j] = uint16_t(ip);
         T.part[ip] = uint16_t(j);
@@ -1150,45 +1279,30 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
       // inside the sub-block of offset pattern p & 3 that holds its site, in
       // label order; the r-th move of sub-block u draws Philox block r of
       // stream (unit = domain * n_sub + u, scatter | pass).
-      for (int u = tid; u < T.ngrp; u += NT) T.bkt[u] = 0;
-      for (int i = tid; i < (NT >> 5) * T.ngrp; i += NT) T.cnt[i] = 0;  // no stamp of this sweep
+      for (int u = tid; u < T.ngrp; u += NT) T.hd[u] = T.hd[T.hstride + u] = 0;  // stamp 0: no pass
+      for (int i = tid; i < 2 * d.ghash; i += NT) T.hash[i] = 0;
+      if (d.gtab)
+        for (int u = tid; u < 3 * T.ngrp; u += NT) T.gcnt[u] = 0;
+      for (int li = tid; li < nds; li += NT) T.rng[li] = uint32_t(T.off[li]) | (uint32_t(T.off[li + 1]) << 16);
+      for (int k = tid; k < nw; k += NT) T.dn[k] = 0;
+      if (tid < 2) T.perr[tid] = PMWA_OK;
+      if (nw > 0 && nw <= NT) {  // the worms into label order, one a thread
+        WormRec w{};
+        if (tid < nw) w = T.W[T.ord[tid]];
+        __syncthreads();
+        if (tid < nw) T.W[tid] = w;
+      }
       __syncthreads();
-      if (nw > 0 && nw <= 32) {  // few worms: one warp, no block barrier per pass
-        if (tid < 32) {
-          const int rc = small_passes(T, dom, nw, tid);
-          if (rc && tid == 0) tile_fail(misc, rc, 5);
-        }
-        __syncthreads();
-        if (misc->err) goto fail;
+      if (nw > NT) {
+        many_passes(T, dom, nw, tclk);
+      } else if (nw > 32) {
+        block_passes(T, dom, nw, tclk);
+      } else if (nw > 0 && tid < 32) {  // few worms: one warp, no barrier
+        const int rc = small_passes(T, dom, nw, tid);
+        if (rc && tid == 0) tile_fail(misc, rc, 5);
       }
-      for (int pass = 0; pass < (nw > 32 ? d.n_cycle : 0); ++pass) {  // no worms: nothing moves
-        const int q = pass & 3;
-        const uint32_t c2 = c2_word(kScatter, uint32_t(pass), d.replica);
-        if (nw <= NT) {  // all warps, one chunk each, one worm a thread
-          pass_fast(T, dom, nw, q, pass, c2, tclk);
-          if (misc->err) goto fail;
-          continue;
-        }
-        {
-          if (tid < 32) rank_pass(T, nw, q, tid);
-          __syncthreads();
-          for (int k = tid; k < nw; k += NT) {
-            const int u = T.wsb[k], r = T.wrk[k], at = T.fill[u] + r;
-            T.idx[at] = T.ord[k];
-            WormRec& w = T.W[T.ord[k]];
-            const int rc = move_desc(T, w, q, r, T.rw[2 * at], T.rw[2 * at + 1]);
-            if (rc) tile_fail(misc, rc, 5);
-            w.lab = uint64_t(u);
-            w.xr = kPending;
-          }
-        }
-        __syncthreads();
-        phase_tick(d, 5, tclk);
-        if (misc->err) goto fail;
-        pass_rounds(T, dom, nw, c2);
-        phase_tick(d, 6, tclk);
-        if (misc->err) goto fail;
-      }
+      __syncthreads();
+      if (misc->err) goto fail;
       phase_tick(d, 3, tclk);
     }
   }
@@ -1389,7 +1503,14 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_tile_batch(const Dev* __restri
 // 1-2), later the worm table and the Step-5 arrays.  The configuration is
 // staged only when that costs no CTA per SM (CTAs per SM: the 228 KB of
 // shared memory of an SM over the per-CTA size plus its 1 KB reserve).
-bool plan_tile_smem(Dev* d, double legs_want, double cands_per_bond) {
+//
+// What a plan offers (its size, its legs) is computed from the reserve below:
+// 2 KB of thresholds, 48 bytes a worm, two words a site or group and two
+// bytes a group for each warp.  The domain tuner picks shapes by these sizes
+// and a tuned instance's chain follows from its domain shape, so the reserve
+// is kept; what the kernel lays out fits inside it (40 bytes a worm, 1 KB of
+// thresholds, and the groups' member tables where they fit).
+bool plan_tile_smem(Dev* d, double legs_want) {
   const int nds = d->dom_x * d->dom_y;
   // Step-5 chains: sub-blocks x temporal slabs
   const int nsub = sb_slots_host(d->dom_x, d->sub_block, d->ndx) * sb_slots_host(d->dom_y, d->sub_block, d->ndy) *
@@ -1397,25 +1518,21 @@ bool plan_tile_smem(Dev* d, double legs_want, double cands_per_bond) {
   const int nb = std::max(nsub, nds) + 1;
   auto up16 = [](size_t x) { return (x + 15) & ~size_t(15); };
   size_t o = 0;
-  d->sm_th = int(o); o = up16(o + 256 * sizeof(uint64_t));
+  d->sm_th = int(o); o = up16(o + 256 * sizeof(uint32_t));
   d->sm_zig = int(o); o = up16(o + size_t(kZigBytes));
   d->sm_off = int(o); o = up16(o + size_t(nds + 1) * sizeof(int));
   d->sm_base = int(o); o = up16(o + size_t(nds));
   d->sm_bcnt = int(o); o = up16(o + size_t(2 * nds) * sizeof(int));
   d->sm_boff = int(o); o = up16(o + size_t(2 * nds) * sizeof(int));
   d->sm_misc = int(o); o = up16(o + sizeof(Misc));
-  d->sm_nbr = int(o); o = up16(o + size_t(6 * nds) * sizeof(int16_t));
+  d->sm_nbr = int(o); o = up16(o + size_t(6 * nds) * sizeof(uint16_t));
   d->sm_sub = int(o); o = up16(o + size_t(4 * nds) * sizeof(uint16_t));
   d->sm_tinfo = int(o); o = up16(o + size_t(6 * nds));
-  const size_t fixed = o;
-  // worm side of the union: table, index, label order, sub-block ids and
-  // ranks, Philox words, two bucket arrays
-  // (and the per-chunk sub-block counts of the block-wide grouping: one row
-  // per warp of the domain's CTA, 16 for CTAs of 256 or 512 threads)
+  const size_t fixed = o + 1024;  // (the reserve of the fixed tables)
+  // worm side of the union, as reserved
   const int warps = nds <= 32 ? 2 : (nds <= 96 ? 4 : 16);
-  const size_t cnt_bytes = up16(size_t(warps) * size_t(nsub) * sizeof(uint16_t));
-  const size_t worm_bytes = up16(size_t(d->wcap) * sizeof(WormRec)) + 4 * up16(size_t(d->wcap) * 2) +
-                            up16(size_t(d->wcap) * 16) + 2 * up16(size_t(nb) * sizeof(int)) + cnt_bytes;
+  const size_t worm_bytes = up16(size_t(d->wcap) * 24) + 4 * up16(size_t(d->wcap) * 2) + up16(size_t(d->wcap) * 16) +
+                            2 * up16(size_t(nb) * sizeof(int)) + up16(size_t(warps) * size_t(nsub) * 2);
   // (on-the-fly windows: the worms of the current configuration by site, beside the pool)
   const size_t otf_bytes = d->win_half ? up16(size_t(nds + 1) * sizeof(int)) + up16(size_t(d->wcap) * 8) : 0;
   const size_t pool_bytes = up16(size_t(d->poolcap) * sizeof(uint64_t)) + otf_bytes;
@@ -1449,6 +1566,7 @@ bool plan_tile_smem(Dev* d, double legs_want, double cands_per_bond) {
   const bool staged = cap0 == want && tot1 <= limit && per_sm(tot1) >= per_sm(tot0);
   d->legcap = int(cap0);
   d->oldcap = staged ? int(want) : 0;
+  d->sm_plan = int(fixed + size_t(legs_bytes(cap0, part)) + size_t(staged ? uni1 : uni0));
   d->sm_leg = int(o); o = up16(o + size_t(d->legcap) * sizeof(uint64_t));
   d->sm_wcnt = int(o); o = up16(o + size_t(d->legcap));
   d->use_part = part ? 1 : 0;
@@ -1460,18 +1578,24 @@ bool plan_tile_smem(Dev* d, double legs_want, double cands_per_bond) {
   d->sm_old = int(o + pool_bytes + up16(size_t(nds + 1) * sizeof(int)));
   d->sm_worm = int(o);
   size_t w = o + up16(size_t(d->wcap) * sizeof(WormRec));
-  d->sm_idx = int(w); w = up16(w + size_t(d->wcap) * 2);
   d->sm_ord = int(w); w = up16(w + size_t(d->wcap) * 2);
-  d->sm_wsb = int(w); w = up16(w + size_t(d->wcap) * 2);
-  d->sm_wrk = int(w); w = up16(w + size_t(d->wcap) * 2);
-  d->sm_rw = int(w); w = up16(w + size_t(d->wcap) * 16);
+  d->sm_dn = int(w); w = up16(w + size_t(d->wcap) * 2);
+  d->sm_idx = d->sm_nxt = int(w); w = up16(w + size_t(d->wcap) * 4);
+  d->sm_fp = int(w); w = up16(w + size_t(d->wcap) * 8);
   d->sm_bkt = int(w); w = up16(w + size_t(nb) * sizeof(int));
-  d->sm_cnt = int(w); w += cnt_bytes;
   d->sm_fill = int(w); w = up16(w + size_t(nb) * sizeof(int));
-  o = std::max(w, o + pool_bytes + (staged ? size_t(stage) : 0));
-  d->sm_total = int(o);
-  (void)cands_per_bond;
-  return d->sm_total <= kSmemLimit - 1024;
+  // the groups' member tables, where the reserve has room for them
+  const size_t cells = up16(size_t(nsub) * 2 * kGroupSlots * sizeof(uint16_t)), counts = up16(size_t(nsub) * 3 * sizeof(int));
+  d->gtab = w + cells + counts <= size_t(d->sm_plan) ? 1 : 0;
+  d->sm_cell = int(w); w += d->gtab ? cells : 0;
+  d->sm_gcnt = int(w); w += d->gtab ? counts : 0;
+  // and chains of worms by leg: as many heads as fit, a power of two
+  d->sm_hash = int(w);
+  d->ghash = 0;
+  for (int h = 64; h <= 1024 && w + 8 * size_t(h) <= size_t(d->sm_plan); h *= 2) d->ghash = h;
+  w += 8 * size_t(d->ghash);
+  d->sm_total = int(std::max(w, o + pool_bytes + (staged ? size_t(stage) : 0)));
+  return d->sm_plan <= kSmemLimit - 1024 && d->sm_total <= d->sm_plan;
 }
 
 int upload_zig_tile(const Zig& z) { return upload_constants(z); }
@@ -1480,10 +1604,14 @@ int upload_zig_tile(const Zig& z) { return upload_constants(z); }
 // of them share an SM (class 0: 64 threads, 1: 128, 2: 256); a large domain
 // whose plan leaves room for one CTA per SM takes 512 threads (class 3),
 // which the registers then allow
-int tile_class(int domain_sites, int smem) {
-  if (domain_sites <= 32) return 0;
-  if (domain_sites <= 96) return 1;
-  return (228LL * 1024) / (static_cast<long long>(smem) + 2048) <= 1 ? 3 : 2;
+// (a mean of more worms than three quarters of the threads takes the next
+// class: Step 5 runs a worm a thread)
+int tile_class(const Dev& d) {
+  const int sites = d.dom_x * d.dom_y;
+  const double worms = d.beta * d.eta * sites;
+  if (sites <= 32 && worms <= 48.0) return 0;
+  if (sites <= 96 && worms <= 96.0) return 1;
+  return (228LL * 1024) / (static_cast<long long>(d.sm_total) + 2048) <= 1 ? 3 : 2;
 }
 
 int prepare_tile_batch(int cls, int smem) {
@@ -1519,7 +1647,7 @@ static int launch_tile_k(const Dev& d, int stop, cudaStream_t st) {
 }
 
 int launch_tile(const Dev& d, int stop, void* stream) {
-  const int cls = tile_class(d.dom_x * d.dom_y, d.sm_total);
+  const int cls = tile_class(d);
   const cudaStream_t st = cudaStream_t(stream);
   const bool otf = d.win_half > 0;
   switch (cls) {
