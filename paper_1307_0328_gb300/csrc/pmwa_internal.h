@@ -152,6 +152,13 @@ int boundary_bonds_per_block(int cap);
 int prepare_boundary(int cap);
 int prepare_tile_batch(int cls, int smem);
 int launch_advance(BatchBase* base, int n, int S, void* stream);
+// log2 of the threads that share a site's K slices: K rounded up to a power of
+// two, at most a warp
+inline int slice_lanes(int K) {
+  int sh = 0;
+  while (sh < 5 && (1 << sh) < K) ++sh;
+  return sh;
+}
 int launch_rho(const Dev& d, int K, double* out, void* stream);
 // n Philox4x32-10 blocks: in[6 j ..] = c0..c3, k0, k1; out[4 j ..] = output
 int launch_philox(const uint32_t* in, uint32_t* out, int64_t n, void* stream);

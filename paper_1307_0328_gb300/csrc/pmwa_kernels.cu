@@ -11,6 +11,7 @@
 // of 64-bit event keys sorted in time, and cnt[i] = count | base << 31.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "pmwa_device.cuh"
@@ -27,31 +28,64 @@ __device__ __forceinline__ int cnt_base(uint32_t c) { return int(c >> 31); }
 __device__ __forceinline__ uint32_t cnt_make(int n, int base) { return uint32_t(n) | (uint32_t(base) << 31); }
 
 // Supplement S-I worm density at K equal-time slices tau_k = k beta / K:
-// eta g_sigma(x) of the interval between vertex legs holding tau_k.
-__global__ void k_rho(const __grid_constant__ Dev d, int K, double* out) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= d.N) return;
+// eta g_sigma(x) of the interval between vertex legs holding tau_k.  2^sh
+// threads a site (slice_lanes: the power of two from K up to a warp), one a
+// slice: each finds its slice by bisection in the site's list (which its
+// neighbours' loads keep in L1) and writes next to them.  The binary64 pipe bounds it,
+// so the polynomials of this estimator are fused multiply-adds (the decisions
+// of Steps 1 and 2 keep their separately rounded ones).  256x256 sites, K = 16:
+// RHO_FIG.
+__device__ __forceinline__ double g_sigma_fused(int sigma, double x) {
+  const double y = -2.0 * x;
+  const int h = __double2hiint(y) & 0x7fffffff;  // |y| compared on the integer pipe: 2^-6, 2^-4, 2^-2, 1
+  double e;
+  if (h < 0x3ff00000) {
+    const int d = h < 0x3f900000 ? 7 : h < 0x3fb00000 ? 9 : h < 0x3fd00000 ? 13 : 19;
+    double p = c_inv_fact[d];
+    for (int n = d - 1; n >= 1; --n) p = fma(p, y, c_inv_fact[n]);
+    e = p * y;
+  } else {
+    e = exp_det(y) - 1.0;
+  }
+  return sigma ? (2.0 + e) / -e : -e / (2.0 + e);
+}
+
+__global__ void k_rho(const __grid_constant__ Dev d, int K, int sh, double* out) {
+  const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if ((t >> sh) >= d.N) return;
+  const int s = int(t >> sh), step = 1 << sh;
   const uint64_t* Kk = d.keyA + size_t(s) * d.cap;
   const int n = cnt_n(d.cntA[s]);
-  int nl = 0, lastleg = -1;
-  for (int k = 0; k < n; ++k) if (!kworm(Kk[k])) { ++nl; lastleg = k; }
+  int lastleg = n - 1;
+  while (lastleg >= 0 && kworm(Kk[lastleg])) --lastleg;
   const uint64_t q62 = kTwo62 / uint64_t(K), r62 = kTwo62 % uint64_t(K);
-  for (int k = 0; k < K; ++k) {
+  for (int k = int(t) & (step - 1); k < K; k += step) {
     const uint64_t pt = uint64_t(k) * q62 + (uint64_t(k) * r62) / uint64_t(K);
     double r;
-    if (nl == 0) {
+    if (lastleg < 0) {
       const double x = __dmul_rn(double(kTwo59), d.XW);
-      r = __dmul_rn(d.eta, g_sigma(0, x));
+      r = __dmul_rn(d.eta, g_sigma_fused(0, x));
     } else {
-      int j = lastleg;   // last leg with pk <= pt, cyclic
-      for (int i = 0; i < n; ++i) if (!kworm(Kk[i]) && kpk(Kk[i]) <= pt) j = i;
-      int h = j;         // next leg after j, cyclic
-      for (int i = 1; i <= n; ++i) { h = (j + i) % n; if (!kworm(Kk[h])) break; }
+      int lo = 0, hi = n;  // the first event above pt
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (kpk(Kk[mid]) <= pt) lo = mid + 1; else hi = mid;
+      }
+      int h = lo, j = lo - 1;  // last leg with pk <= pt and the next leg after it, cyclic
+      while (h < n && kworm(Kk[h])) ++h;
+      if (h == n) { h = 0; while (kworm(Kk[h])) ++h; }
+      while (j >= 0 && kworm(Kk[j])) --j;
+      if (j < 0) j = lastleg;
       const double x = __dmul_rn(__ull2double_rn(wpts(kpk(Kk[j]), kpk(Kk[h]))), d.XW);
-      r = __dmul_rn(d.eta, g_sigma(kab(Kk[j]) ^ kbl(Kk[h]), x));
+      r = __dmul_rn(d.eta, g_sigma_fused(kab(Kk[j]) ^ kbl(Kk[h]), x));
     }
     out[size_t(s) * K + k] = r;
   }
+}
+
+static void run_rho(const Dev& d, int K, double* out, cudaStream_t st) {
+  const int sh = slice_lanes(K);
+  k_rho<<<blocks_for((long long)d.N << sh, 128), 128, 0, st>>>(d, K, sh, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -715,7 +749,7 @@ int rho_slices_static(const Dev& d, int K, double* host_out, void* stream) {
   int st = PMWA_OK;
   double* scratch = rho_scratch_address(&st);
   if (!scratch) return st;
-  k_rho<<<blocks_for(d.N, 128), 128, 0, cudaStream_t(stream)>>>(d, K, scratch);
+  run_rho(d, K, scratch, cudaStream_t(stream));
   if (cudaGetLastError() != cudaSuccess) return PMWA_ECUDA;
   if (cudaMemcpyAsync(host_out, scratch, size_t(d.N) * size_t(K) * sizeof(double), cudaMemcpyDeviceToHost,
                       cudaStream_t(stream)) != cudaSuccess)
@@ -725,42 +759,71 @@ int rho_slices_static(const Dev& d, int K, double* host_out, void* stream) {
 }
 
 // Supplement S-I equal-time correlators from the worm densities rho[i*K+k]:
-// blockIdx.y = r - 1 (r = 1..rmax) accumulates sum_{i,k} rho_i rho_{i+r x}
-// into sums[r-1] and rho_i rho_{i+r y} into sums[rmax + r - 1]; blockIdx.y =
-// rmax accumulates the plaquette product rho_i rho_{i+x} rho_{i+y}
-// rho_{i+x+y} into sums[2 rmax].  Sites strided over blockIdx.x.
-__global__ void k_green(int Lx, int Ly, int K, int rmax, const double* __restrict__ rho, double* sums) {
-  const int N = Lx * Ly;
-  const int r = int(blockIdx.y) + 1;
-  double ax = 0.0, ay = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-    const int x = i % Lx, y = i / Lx;
-    const double* ri = rho + size_t(i) * K;
-    if (r <= rmax) {
-      const double* rx = rho + size_t((x + r) % Lx + Lx * y) * K;
-      const double* ry = rho + size_t(x + Lx * ((y + r) % Ly)) * K;
-      for (int k = 0; k < K; ++k) { ax = fma(ri[k], rx[k], ax); ay = fma(ri[k], ry[k], ay); }
+// sum_{i,k} rho_i rho_{i+r x} into sums[r-1], rho_i rho_{i+r y} into
+// sums[rmax + r - 1] (r = 1..rmax), and the plaquette product rho_i rho_{i+x}
+// rho_{i+y} rho_{i+x+y} into sums[2 rmax].  A row of the lattice is Lx K
+// consecutive doubles and a shift by r sites is a cyclic shift by r K of it,
+// so every load is coalesced; a block takes rows blockIdx.x, + gridDim.x, ...
+// and kGreenR values of r (blockIdx.y; the last one the plaquette), which
+// share the row's own densities.  256x256 sites, K = 16, rmax = 64: 0.69 ms
+// with a thread a site (a line a lane and load), now 0.32 ms; two fused
+// multiply-adds a site, slice and r are 0.21 ms of the binary64 pipe (two
+// lanes a cycle and SM).
+constexpr int kGreenR = 4;
+__global__ void __launch_bounds__(256) k_green(int Lx, int Ly, int K, int rmax, const double* __restrict__ rho,
+                                               double* sums) {
+  const int groups = int(gridDim.y) - 1, g = int(blockIdx.y);
+  const long long W = static_cast<long long>(Lx) * K;
+  double ax[kGreenR] = {}, ay[kGreenR] = {};
+  for (int y = blockIdx.x; y < Ly; y += gridDim.x) {
+    const double* row = rho + size_t(y) * W;
+    if (g < groups) {
+      const double* far[kGreenR];
+#pragma unroll
+      for (int e = 0; e < kGreenR; ++e) far[e] = rho + size_t((y + min(g * kGreenR + e + 1, rmax)) % Ly) * W;
+      for (long long f = threadIdx.x; f < W; f += blockDim.x) {
+        const double c = row[f];
+#pragma unroll
+        for (int e = 0; e < kGreenR; ++e) {
+          long long fx = f + static_cast<long long>(min(g * kGreenR + e + 1, rmax)) * K;
+          if (fx >= W) fx -= W;
+          ax[e] = fma(c, row[fx], ax[e]);
+          ay[e] = fma(c, far[e][f], ay[e]);
+        }
+      }
     } else {
-      const double* r1 = rho + size_t((x + 1) % Lx + Lx * y) * K;
-      const double* r2 = rho + size_t(x + Lx * ((y + 1) % Ly)) * K;
-      const double* r3 = rho + size_t((x + 1) % Lx + Lx * ((y + 1) % Ly)) * K;
-      for (int k = 0; k < K; ++k) ax = fma(ri[k] * r1[k], r2[k] * r3[k], ax);
+      const double* up = rho + size_t((y + 1) % Ly) * W;
+      for (long long f = threadIdx.x; f < W; f += blockDim.x) {
+        const long long fx = f + K >= W ? f + K - W : f + K;
+        ax[0] = fma(row[f] * row[fx], up[f] * up[fx], ax[0]);
+      }
     }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    ax += __shfl_down_sync(0xffffffffu, ax, o);
-    ay += __shfl_down_sync(0xffffffffu, ay, o);
+  // one sum a block and r: the order of few additions is left to the atomics
+  __shared__ double red[8][2 * kGreenR];
+#pragma unroll
+  for (int e = 0; e < kGreenR; ++e) {
+    for (int o = 16; o > 0; o >>= 1) {
+      ax[e] += __shfl_down_sync(0xffffffffu, ax[e], o);
+      ay[e] += __shfl_down_sync(0xffffffffu, ay[e], o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      red[threadIdx.x >> 5][e] = ax[e];
+      red[threadIdx.x >> 5][kGreenR + e] = ay[e];
+    }
   }
-  if ((threadIdx.x & 31) == 0) {
-    if (r <= rmax) { atomicAdd(sums + (r - 1), ax); atomicAdd(sums + rmax + r - 1, ay); }
-    else atomicAdd(sums + 2 * rmax, ax);
-  }
+  __syncthreads();
+  if (threadIdx.x >= 2 * kGreenR) return;
+  const int e = int(threadIdx.x) % kGreenR, r = g * kGreenR + e + 1;
+  double v = 0.0;
+  for (int w = 0; w < 8; ++w) v += red[w][threadIdx.x];
+  if (g < groups && r <= rmax) atomicAdd(sums + (threadIdx.x < kGreenR ? r - 1 : rmax + r - 1), v);
+  if (g == groups && threadIdx.x == 0) atomicAdd(sums + 2 * rmax, v);
 }
 
 int launch_green(int Lx, int Ly, int K, int rmax, const double* rho, double* sums, void* stream) {
-  const int N = Lx * Ly;
-  const int bx = N < 256 * 152 ? blocks_for(N, 256) : 152;
-  k_green<<<dim3(bx, rmax + 1), 256, 0, cudaStream_t(stream)>>>(Lx, Ly, K, rmax, rho, sums);
+  const int groups = (rmax + kGreenR - 1) / kGreenR;
+  k_green<<<dim3(std::min(Ly, 304), groups + 1), 256, 0, cudaStream_t(stream)>>>(Lx, Ly, K, rmax, rho, sums);
   return int(cudaGetLastError());
 }
 
@@ -784,7 +847,7 @@ int launch_philox(const uint32_t* in, uint32_t* out, int64_t n, void* stream) {
 }
 
 int launch_rho(const Dev& d, int K, double* out, void* stream) {
-  k_rho<<<blocks_for(d.N, 128), 128, 0, cudaStream_t(stream)>>>(d, K, out);
+  run_rho(d, K, out, cudaStream_t(stream));
   return int(cudaGetLastError());
 }
 
