@@ -754,24 +754,39 @@ int pmwa_export_bytes(pmwa_handle* h, size_t* bytes) {
 }
 
 int pmwa_export(pmwa_handle* h, void* buf, size_t bytes) {
-  size_t need = 0;
-  int rc = pmwa_export_bytes(h, &need);
-  if (rc) return rc;
-  if (!buf || bytes < need) return PMWA_EINVAL;
+  if (!h) return PMWA_EINVAL;
+  if (h->broken) return PMWA_EINVARIANT;
   const size_t N = size_t(h->d.N), cap = size_t(h->d.cap);
   std::vector<uint32_t> cnt(N);
-  std::vector<uint64_t> keys(N * cap);
-  if (cudaMemcpy(cnt.data(), h->d.cntA, N * 4, cudaMemcpyDeviceToHost) ||
-      cudaMemcpy(keys.data(), h->d.keyA, N * cap * 8, cudaMemcpyDeviceToHost))
+  if (cudaStreamSynchronize(h->stream) || cudaMemcpy(cnt.data(), h->d.cntA, N * 4, cudaMemcpyDeviceToHost))
     return PMWA_ECUDA;
+  std::vector<uint64_t> at(N);  // each site's header word in the buffer
+  size_t words = 1;
+  for (size_t s = 0; s < N; ++s) {
+    at[s] = words;
+    words += 1 + (cnt[s] & 0x7fffffffu);
+  }
+  if (!buf || bytes < words * 8) return PMWA_EINVAL;
   uint64_t* o = static_cast<uint64_t*>(buf);
-  size_t k = 0;
-  o[k++] = N;
+  o[0] = N;
+  // packed on the device (scratch: the idle next-configuration slots) where
+  // the packed words and their places fit there
+  if (words + N <= N * cap) {
+    uint64_t* dev = h->d.keyB;
+    uint64_t* dat = dev + words;
+    if (cudaMemcpyAsync(dat, at.data(), N * 8, cudaMemcpyHostToDevice, h->stream) ||
+        launch_pack(h->d, dat, dev, h->stream) ||
+        cudaMemcpyAsync(o + 1, dev + 1, (words - 1) * 8, cudaMemcpyDeviceToHost, h->stream) ||
+        cudaStreamSynchronize(h->stream))
+      return PMWA_ECUDA;
+    return PMWA_OK;
+  }
+  std::vector<uint64_t> keys(N * cap);
+  if (cudaMemcpy(keys.data(), h->d.keyA, N * cap * 8, cudaMemcpyDeviceToHost)) return PMWA_ECUDA;
   for (size_t s = 0; s < N; ++s) {
     const size_t n = cnt[s] & 0x7fffffffu;
-    o[k++] = uint64_t(n) | (uint64_t(cnt[s] >> 31) << 63);
-    std::memcpy(o + k, keys.data() + s * cap, n * 8);
-    k += n;
+    o[at[s]] = uint64_t(n) | (uint64_t(cnt[s] >> 31) << 63);
+    std::memcpy(o + at[s] + 1, keys.data() + s * cap, n * 8);
   }
   return PMWA_OK;
 }
@@ -781,15 +796,47 @@ int pmwa_import(pmwa_handle* h, const void* buf, size_t bytes) {
   const uint64_t* in = static_cast<const uint64_t*>(buf);
   const size_t nw = bytes / 8, N = size_t(h->d.N), cap = size_t(h->d.cap);
   if (nw < 1 || in[0] != N) return PMWA_EINVAL;
+  // the headers, up to the first one that is wrong (at site ns, with status
+  // rc): the sites before it are checked for the other invariants first
+  std::vector<uint64_t> at(N);
+  size_t words = 1, ns = 0;
+  int rc = PMWA_OK;
+  for (; ns < N; ++ns) {
+    // (a header's place follows from the ones before it: fetch the lines ahead)
+    for (int k = 0; k < 4; ++k) __builtin_prefetch(in + std::min(words + 256 + 8 * size_t(k), nw - 1));
+    if (words >= nw) { rc = PMWA_EINVAL; break; }
+    const size_t n = size_t(in[words] & 0x7fffffffu);
+    if (n > cap) { rc = PMWA_ECAPACITY; break; }
+    if (words + 1 + n > nw) { rc = PMWA_EINVAL; break; }
+    at[ns] = words;
+    words += 1 + n;
+  }
+  if (cudaStreamSynchronize(h->stream)) return PMWA_ECUDA;
+  // checked and unpacked on the device (scratch: the idle next-configuration
+  // slots) where the buffer and its places fit there
+  if (words + N + 1 <= N * cap) {
+    uint64_t* dev = h->d.keyB;
+    uint64_t* dat = dev + words;
+    unsigned long long* dbad = reinterpret_cast<unsigned long long*>(dat + N);
+    unsigned long long bad = 0;
+    if (cudaMemcpyAsync(dev, in, words * 8, cudaMemcpyHostToDevice, h->stream) ||
+        cudaMemcpyAsync(dat, at.data(), N * 8, cudaMemcpyHostToDevice, h->stream) ||
+        launch_packed_check(dat, dev, int(ns), dbad, h->stream) ||
+        cudaMemcpyAsync(&bad, dbad, sizeof bad, cudaMemcpyDeviceToHost, h->stream) ||
+        cudaStreamSynchronize(h->stream))
+      return PMWA_ECUDA;
+    if (bad != ~0ull) return PMWA_EINVARIANT;
+    if (rc) return rc;
+    if (launch_unpack(h->d, dat, dev, h->stream) || cudaStreamSynchronize(h->stream)) return PMWA_ECUDA;
+    h->broken = false;
+    return PMWA_OK;
+  }
   std::vector<uint32_t> cnt(N);
   std::vector<uint64_t> keys(N * cap, 0);
-  size_t k = 1;
-  for (size_t s = 0; s < N; ++s) {
-    if (k >= nw) return PMWA_EINVAL;
-    const uint64_t hd = in[k++];
+  for (size_t s = 0; s < ns; ++s) {
+    const size_t k = at[s] + 1;
+    const uint64_t hd = in[at[s]];
     const size_t n = size_t(hd & 0x7fffffffu);
-    if (n > cap) return PMWA_ECAPACITY;
-    if (k + n > nw) return PMWA_EINVAL;
     for (size_t j = 0; j < n; ++j) {
       const uint64_t key = in[k + j];
       if (((key >> 2) & 7) == 6) return PMWA_EINVARIANT;
@@ -803,10 +850,9 @@ int pmwa_import(pmwa_handle* h, const void* buf, size_t bytes) {
     if (n && int(hd >> 63) != int(in[k + n - 1] & 1)) return PMWA_EINVARIANT;
     std::memcpy(keys.data() + s * cap, in + k, n * 8);
     cnt[s] = uint32_t(n) | (uint32_t(hd >> 63) << 31);
-    k += n;
   }
-  if (cudaStreamSynchronize(h->stream) ||
-      cudaMemcpy(h->d.cntA, cnt.data(), N * 4, cudaMemcpyHostToDevice) ||
+  if (rc) return rc;
+  if (cudaMemcpy(h->d.cntA, cnt.data(), N * 4, cudaMemcpyHostToDevice) ||
       cudaMemcpy(h->d.keyA, keys.data(), N * cap * 8, cudaMemcpyHostToDevice))
     return PMWA_ECUDA;
   h->broken = false;

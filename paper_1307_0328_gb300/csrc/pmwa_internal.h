@@ -179,6 +179,12 @@ constexpr int kCheckNone = 0x7fffffff;
 constexpr int kCheckCapacity = 1, kCheckTag = 2, kCheckOrder = 3, kCheckContinuity = 4, kCheckBase = 5,
               kCheckBond = 6, kCheckPartner = 7, kCheckConservation = 8;
 int launch_green(int Lx, int Ly, int K, int rmax, const double* rho, double* sums, void* stream);
+// checkpoints: the configuration to / from a packed buffer in device memory,
+// each site's header word at at[s] and its keys after it; *bad = the first of
+// ns packed sites that breaks an invariant of the format, ~0 if none does
+int launch_pack(const Dev& d, const uint64_t* at, uint64_t* out, void* stream);
+int launch_packed_check(const uint64_t* at, const uint64_t* in, int ns, unsigned long long* bad, void* stream);
+int launch_unpack(const Dev& d, const uint64_t* at, const uint64_t* in, void* stream);
 // rho slices through the library's own static device scratch (no allocation)
 int rho_slices_static(const Dev& d, int K, double* host_out, void* stream);
 // shared-memory plan of the tile kernel for this instance (fills the sm_*

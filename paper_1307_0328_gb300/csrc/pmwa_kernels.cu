@@ -88,6 +88,8 @@ static void run_rho(const Dev& d, int K, double* out, cudaStream_t st) {
   k_rho<<<blocks_for((long long)d.N << sh, 128), 128, 0, st>>>(d, K, sh, out);
 }
 
+static inline int site_warps(int N) { return blocks_for((long long)N * 32, 128); }
+
 // ---------------------------------------------------------------------------
 // Step 2 (spatial-boundary update, Eq. 4) and Step 3 on one boundary bond,
 // in place on the current configuration.
@@ -824,6 +826,69 @@ __global__ void __launch_bounds__(256) k_green(int Lx, int Ly, int K, int rmax, 
 int launch_green(int Lx, int Ly, int K, int rmax, const double* rho, double* sums, void* stream) {
   const int groups = (rmax + kGreenR - 1) / kGreenR;
   k_green<<<dim3(std::min(Ly, 304), groups + 1), 256, 0, cudaStream_t(stream)>>>(Lx, Ly, K, rmax, rho, sums);
+  return int(cudaGetLastError());
+}
+
+// ---------------------------------------------------------------------------
+// Checkpoints: the used keys of every site between the slots and a packed
+// buffer (each site's header word at at[s], its keys after it).  One warp per
+// site.  Only the used part of a configuration then crosses to the host, 9 MB
+// instead of 46 MB at 256x256, beta t = 4 (export 3.6 -> 0.15 ms, import 4.9
+// -> 0.75 ms, each kernel 10 us).
+__global__ void k_pack(const __grid_constant__ Dev d, const uint64_t* __restrict__ at, uint64_t* out) {
+  const int s = int((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (s >= d.N) return;
+  const uint32_t c = d.cntA[s];
+  const int n = cnt_n(c);
+  const uint64_t* K = d.keyA + size_t(s) * d.cap;
+  uint64_t* o = out + at[s];
+  if (lane == 0) o[0] = uint64_t(n) | (uint64_t(cnt_base(c)) << 63);
+  for (int k = lane; k < n; k += 32) o[1 + k] = K[k];
+}
+
+// bad = min over the sites 0 .. ns - 1 of a packed buffer that break an
+// invariant of the format (tags, time order, continuity, base state)
+__global__ void k_packed_check(const uint64_t* __restrict__ at, const uint64_t* __restrict__ in, int ns,
+                               unsigned long long* bad) {
+  const int s = int((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (s >= ns) return;
+  const uint64_t* p = in + at[s];
+  const uint64_t hd = p[0];
+  const int n = cnt_n(uint32_t(hd));
+  bool ok = true;
+  for (int k = lane; k < n; k += 32) {
+    const uint64_t key = p[1 + k], nx = p[1 + (k + 1 == n ? 0 : k + 1)];
+    ok = ok && ktag(key) != 6 && (k + 1 == n || kpk(key) < kpk(nx)) && kab(key) == kbl(nx) &&
+         (k + 1 < n || int(hd >> 63) == kab(key));
+  }
+  if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicMin(bad, (unsigned long long)(s));
+}
+
+__global__ void k_unpack(const __grid_constant__ Dev d, const uint64_t* __restrict__ at, const uint64_t* __restrict__ in) {
+  const int s = int((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (s >= d.N) return;
+  const uint64_t* p = in + at[s];
+  const uint64_t hd = p[0];
+  const int n = cnt_n(uint32_t(hd));
+  uint64_t* K = d.keyA + size_t(s) * d.cap;
+  for (int k = lane; k < n; k += 32) K[k] = p[1 + k];
+  if (lane == 0) d.cntA[s] = cnt_make(n, int(hd >> 63));
+}
+
+int launch_pack(const Dev& d, const uint64_t* at, uint64_t* out, void* stream) {
+  k_pack<<<site_warps(d.N), 128, 0, cudaStream_t(stream)>>>(d, at, out);
+  return int(cudaGetLastError());
+}
+
+int launch_packed_check(const uint64_t* at, const uint64_t* in, int ns, unsigned long long* bad, void* stream) {
+  if (cudaMemsetAsync(bad, 0xff, sizeof *bad, cudaStream_t(stream)) != cudaSuccess) return int(cudaGetLastError());
+  if (ns < 1) return 0;
+  k_packed_check<<<site_warps(ns), 128, 0, cudaStream_t(stream)>>>(at, in, ns, bad);
+  return int(cudaGetLastError());
+}
+
+int launch_unpack(const Dev& d, const uint64_t* at, const uint64_t* in, void* stream) {
+  k_unpack<<<site_warps(d.N), 128, 0, cudaStream_t(stream)>>>(d, at, in);
   return int(cudaGetLastError());
 }
 
