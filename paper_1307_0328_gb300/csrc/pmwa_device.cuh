@@ -187,23 +187,38 @@ __device__ inline double xg_sigma(int sigma, double x) {
 }
 
 // The same two series in fixed point, for the per-interval terms of the
-// estimator: coefficients a_n 2^62 and b_n 2^62 rounded to nearest (exact
-// rationals from the Bernoulli numbers), Horner's rule on signed 64-bit
-// words with y 2^64 = (x 2^64)^2 / 2^64.  The terms kept (5, 8 or 19 for
-// tanh and 5, 7 or 13 for coth as x < 2^-5, 2^-3, 2^-1) leave a truncation
-// below 2^-63; each product is floored, so a term is within (n + 1) 2^-62
-// of x g_sigma(x).  No floating point is used, so the sum of the terms of a
-// site is exact and independent of the order of summation.
-__constant__ long long c_xtanh_fx[19] = {
-    4611686018427387904ll, -1537228672809129301ll, 614891469123651721ll, -248884642264335220ll,
-    100855214512344991ll, -40874459371278820ll, 16565766642662335ll, -6713851087910371ll,
-    2721021299897250ll, -1102788392755917ll, 446943300930299ll, -181139297079955ll,
-    73412991936897ll, -29753164951077ll, 12058503559795ll, -4887127414535ll,
-    1980678137006ll, -802738613024ll, 325337705708ll};
-__constant__ long long c_xcoth_fx[13] = {
-    4611686018427387904ll, 1537228672809129301ll, -102481911520608620ll, 9760182049581773ll,
-    -976018204958177ll, 98587697470523ll, -9981552960019ll, 1011155871493ll,
-    -102446800762ll, 10379912109ll, -1051701970ll, 106559612ll, -10796744ll};
+// estimator: the magnitudes of a_n 2^62 and b_n 2^62 rounded to nearest (exact
+// rationals from the Bernoulli numbers), Horner's rule on 64-bit words with
+// y 2^64 = (x 2^64)^2 / 2^64.  The signs alternate (for coth from b_1 on), so
+// every step is a difference of positive numbers.  The terms kept (8 for
+// x < 2^-3, 19 for x < 1/2; the b_n from 13 on are below 2^-63 there) leave a
+// truncation below 2^-63; each product is floored, so a term is within
+// (n + 1) 2^-62 of x g_sigma(x).  No floating point is used, so the sum of the
+// terms of a site is exact and independent of the order of summation.
+__constant__ unsigned long long c_xg_fx[2][19] = {
+    {4611686018427387904ull, 1537228672809129301ull, 614891469123651721ull, 248884642264335220ull,
+     100855214512344991ull, 40874459371278820ull, 16565766642662335ull, 6713851087910371ull,
+     2721021299897250ull, 1102788392755917ull, 446943300930299ull, 181139297079955ull,
+     73412991936897ull, 29753164951077ull, 12058503559795ull, 4887127414535ull,
+     1980678137006ull, 802738613024ull, 325337705708ull},
+    {4611686018427387904ull, 1537228672809129301ull, 102481911520608620ull, 9760182049581773ull,
+     976018204958177ull, 98587697470523ull, 9981552960019ull, 1011155871493ull,
+     102446800762ull, 10379912109ull, 1051701970ull, 106559612ull, 10796744ull, 0, 0, 0, 0, 0, 0}};
+
+// N terms of the series of sigma at y = Y 2^-64, times 2^62.  Unrolled with
+// the coefficients of both sigmas read at uniform addresses and one selected:
+// a loop whose length and table differ from lane to lane reads its constants
+// one lane after the other (output and measurement of a 16x16 domain at beta
+// t = 4: 73k -> 60k cycles a sweep, at beta t = 16 145k -> 112k).
+template <int N>
+__device__ __forceinline__ uint64_t xg_series(int sigma, uint64_t Y) {
+  auto c = [&](int k) { return sigma ? c_xg_fx[1][k] : c_xg_fx[0][k]; };
+  uint64_t p = c(N - 1);
+#pragma unroll
+  for (int k = N - 2; k >= 1; --k) p = c(k) - __umul64hi(p, Y);
+  p = __umul64hi(p, Y);
+  return sigma ? c_xg_fx[1][0] + p : __umul64hi(c_xg_fx[0][0] - p, Y);
+}
 
 // x g_sigma(x) 2^62 for x = I beta eta / 2^59 (XQ: beta eta 2^5 as a grid
 // scale, so that x 2^64 = (I m) >> sh); false when x >= 1/2, where the
@@ -218,20 +233,8 @@ __device__ __forceinline__ bool xg_fix(int sigma, uint64_t I, GridScale XQ, uint
     X = (hi << (64 - XQ.sh)) | (lo >> XQ.sh);
   }
   if (X >= (1ull << 63)) return false;
-  const long long Y = (long long)__umul64hi(X, X);
-  const int band = (X < (1ull << 59)) ? 0 : (X < (1ull << 61)) ? 1 : 2;
-  long long p;
-  if (sigma) {
-    const int n = band == 0 ? 5 : band == 1 ? 7 : 13;
-    p = c_xcoth_fx[n - 1];
-    for (int k = n - 2; k >= 0; --k) p = c_xcoth_fx[k] + __mul64hi(p, Y);
-    out = uint64_t(p);
-  } else {
-    const int n = band == 0 ? 5 : band == 1 ? 8 : 19;
-    p = c_xtanh_fx[n - 1];
-    for (int k = n - 2; k >= 0; --k) p = c_xtanh_fx[k] + __mul64hi(p, Y);
-    out = uint64_t(__mul64hi(p, Y));
-  }
+  const uint64_t Y = __umul64hi(X, X);
+  out = X < (1ull << 61) ? xg_series<8>(sigma, Y) : xg_series<19>(sigma, Y);
   return true;
 }
 

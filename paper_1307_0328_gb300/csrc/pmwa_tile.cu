@@ -1307,9 +1307,26 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
     }
   }
 
-  // ---- phase 5: next configuration + Step 6
+  // ---- phase 5: next configuration + Step 6.  An event's place in its site's
+  // list follows from counts alone: a leg's from its index and the site's
+  // worms below it, a worm's from its interval and the site's worms below it.
+  // So legs and worms are laid over the threads, not sites (a site's merge is
+  // one chain, and sites are half or an eighth of the threads in the larger
+  // and smaller CTAs), and consecutive lanes write consecutive keys.  The
+  // occupied time of a site is 2^62 when its state at the origin is 1, plus
+  // the times where the state falls and minus those where it rises.  Cycles a
+  // sweep, with xg_series: 16x16 sites 75k -> 60k at beta t = 4, 153k -> 113k
+  // at beta t = 16; 4x4 sites with 188 legs each 165k -> 92k.
   {
     const int nw = (stop >= 4) ? misc->nworms : 0;
+    const int NB = d.ntau > 1 ? d.ntau : 0;  // temporal boundaries in the leg table: no events
+    uint64_t nv = 0, nk = 0, nwc = 0, olo = 0, ohi = 0, qlo = 0, qhi = 0;
+    double q = 0.0;
+    // +t at a fall, -t at a rise of the state (128-bit two's complement)
+    auto flip = [&](uint64_t pk, int above) {
+      if (above) add128(olo, ohi, ~pk + 1, pk ? ~0ull : 0);
+      else add128(olo, ohi, pk, 0);
+    };
     if (stop >= 4) {
       for (int li = tid; li <= nds; li += NT) T.bkt[li] = 0;
       __syncthreads();
@@ -1320,97 +1337,57 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
       __syncthreads();
       for (int w = tid; w < nw; w += NT) T.idx[atomicAdd(&T.fill[T.W[w].site], 1)] = uint16_t(w);
       __syncthreads();
-    }
-    uint64_t nv = 0, nk = 0, nwc = 0, olo = 0, ohi = 0, qlo = 0, qhi = 0;
-    double q = 0.0;
-    for (int li = tid; li < nds; li += NT) {
-      const int s = T.gsite(li);
-      const int st = T.off[li], nl = T.off[li + 1] - st;
-      uint64_t* OUT = d.keyB + size_t(s) * d.cap;
-      const uint64_t* KO = d.keyA + size_t(s) * d.cap;
-      const int nO = cnt_n(d.cntA[s]);
-      uint16_t* seg = nullptr;
-      int nws = 0;
-      if (stop >= 4) {
-        seg = T.idx + T.bkt[li];
-        nws = T.bkt[li + 1] - T.bkt[li];
-        for (int p = 1; p < nws; ++p) {  // worms of the site in time order
-          const uint16_t v = seg[p];
-          int r = p - 1;
-          while (r >= 0 && T.W[v].key < T.W[seg[r]].key) { seg[r + 1] = seg[r]; --r; }
-          seg[r + 1] = v;
-        }
+      // worms of site li below `key`
+      auto below = [&](int li, uint64_t key) {
+        int r = 0;
+        for (int p = T.bkt[li]; p < T.bkt[li + 1]; ++p) r += T.W[T.idx[p]].key < key ? 1 : 0;
+        return r;
+      };
+      for (int w = tid; w < nw; w += NT) {
+        const uint64_t key = T.W[w].key;
+        const int li = T.W[w].site, L = T.W[w].leg;
+        int at = below(li, key);
+        // (a worm of the interval round the origin may lie before the first leg)
+        if (L != kNone && key > T.leg[L]) at += L - T.off[li] + 1 - (NB ? slab_of_m(d, key >> 5) + 1 : 0);
+        if (at >= d.cap) { tile_fail(misc, PMWA_ECAPACITY, 6); continue; }
+        d.keyB[size_t(T.gsite(li)) * d.cap + at] = key;
+        flip(kpk(key), kab(key));
+        ++nwc;
       }
-      // merge legs with worms (stop 3: the old worms); the occupied time of
-      // the intervals between consecutive events is summed as they are
-      // written (Step 6), the interval round the circle after the last one
-      int il = 0, iw = 0, io = 0, no = 0, nww = 0;
-      bool bad = false;
-      uint64_t occ = 0, first_pk = 0, prev = 0;
-      for (;;) {
-        uint64_t wk = ~0ull;
-        if (stop >= 4) { if (iw < nws) wk = T.W[seg[iw]].key; }
-        else {
-          while (io < nO && !kworm(KO[io])) ++io;
-          if (io < nO) wk = KO[io];
-        }
-        const uint64_t lk = il < nl ? T.leg[st + il] : ~0ull;
-        if (lk == ~0ull && wk == ~0ull) break;
-        uint64_t key;
-        if (kpk(lk) < kpk(wk) || wk == ~0ull) {
-          key = lk;
-          ++il;
-          if (ktag(key) == 6) continue;  // a temporal boundary is no event
-        } else {
-          key = wk;
-          ++nww;
-          if (stop >= 4) ++iw; else ++io;
-        }
-        if (no >= d.cap) { bad = true; break; }
-        if (no == 0) first_pk = kpk(key);
-        else if (kab(prev)) occ += (kpk(key) - kpk(prev)) & kMask62;
-        prev = key;
-        OUT[no++] = key;
-      }
-      if (bad) { tile_fail(misc, PMWA_ECAPACITY, 6); continue; }
-      int base;
-      if (no) base = kab(OUT[no - 1]);
-      else base = (stop >= 4) ? T.base[li] : cnt_base(d.cntA[s]);
-      d.cntB[s] = uint32_t(no) | (uint32_t(base) << 31);
-      if (stop < 6) continue;
-      // Step 6, per site: occupied time (at most 2^62 a site, summed in 128
-      // bits), worms; a site without legs is one interval of sigma = 0
-      if (no == 0) occ = base ? kTwo62 : 0;
-      else if (no == 1) occ = kab(prev) ? kTwo62 : 0;
-      else if (kab(prev)) occ += (first_pk - kpk(prev)) & kMask62;
-      add128(olo, ohi, occ, 0);
-      nwc += uint64_t(nww);
-      if (nl == 0) {
-        uint64_t v;
-        if (xg_fix(0, kTwo59, d.XQ, v)) add128(qlo, qhi, v, 0);
-        else q += xg_sigma(0, double(kTwo59) * d.XW);
-      }
-    }
-    if (stop >= 6) {
-      // Step 6, per interval (legs split evenly over the threads): vertex
-      // and kink counts, and the improved <Q> sum of x g_sigma(x), in fixed
-      // point (exact sum) where x < 1/2, else in binary64
-      const int total = T.off[nds];
-      const int chunk = (total + NT - 1) / NT;
-      int j = tid * chunk;
-      const int jend = min(total, j + chunk);
+      const int total = T.off[nds], warps = NT >> 5;
+      const int chunk = ((total + warps - 1) / warps + 31) & ~31;  // legs a warp
+      int j = (tid >> 5) * chunk + (tid & 31);
+      const int jend = min(total, (tid >> 5) * chunk + chunk);
       if (j < jend) {
         int a = 0, b = nds;  // the site of leg j: off[a] <= j < off[a + 1]
         while (a + 1 < b) {
           const int m = (a + b) >> 1;
           if (T.off[m] <= j) a = m; else b = m;
         }
-        int li = a;
-        for (; j < jend; ++j) {
-          while (T.off[li + 1] <= j) ++li;
+        int li = a, en = T.off[a + 1];
+        size_t slot = size_t(T.gsite(li)) * d.cap;
+        for (; j < jend; j += 32) {
+          if (en <= j) {
+            do en = T.off[++li + 1]; while (en <= j);
+            slot = size_t(T.gsite(li)) * d.cap;
+          }
+          const int st = T.off[li];
           const uint64_t lo = T.leg[j];
-          const uint64_t hi = T.leg[(j + 1 == T.off[li + 1]) ? T.off[li] : j + 1];
-          if (ktag(lo) < 6 && (T.tinfo[li * 6 + ktag(lo)] & 1)) { ++nv; if (kab(lo) != kbl(lo)) ++nk; }
+          const int tag = ktag(lo);
+          if (tag < 6) {
+            const uint64_t m = lo >> 5;
+            const int at = j - st + below(li, lo) - (NB && m ? slab_of_m(d, m - 1) + 1 : 0);
+            if (at >= d.cap) tile_fail(misc, PMWA_ECAPACITY, 6);
+            else d.keyB[slot + at] = lo;
+          }
+          if (stop < 6) continue;
+          // Step 6, per interval: vertex and kink counts, and the improved <Q>
+          // sum of x g_sigma(x), in fixed point (exact sum) where x < 1/2,
+          // else in binary64
+          const bool kink = tag < 6 && kab(lo) != kbl(lo);
+          if (kink) flip(kpk(lo), kab(lo));
+          if (tag < 6 && (T.tinfo[li * 6 + tag] & 1)) { ++nv; if (kink) ++nk; }
+          const uint64_t hi = T.leg[j + 1 == en ? st : j + 1];
           const uint64_t I = wpts(kpk(lo), kpk(hi));
           const int sg = kab(lo) ^ kbl(hi);
           uint64_t v;
@@ -1418,8 +1395,49 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
           else q += xg_sigma(sg, __ull2double_rn(I) * d.XW);
         }
       }
-      q += __ull2double_rn(qhi) * 4.0 + __ull2double_rn(qlo) * 0x1p-62;
     }
+    for (int li = tid; li < nds; li += NT) {
+      const int s = T.gsite(li);
+      const int st = T.off[li], nl = T.off[li + 1] - st;
+      int no, base;
+      if (stop >= 4) {
+        no = nl - (nl ? NB : 0) + T.bkt[li + 1] - T.bkt[li];
+        base = T.base[li];
+        if (nl) {  // the state at the origin: above the last leg, and past the worms behind it
+          const uint64_t top = T.leg[st + nl - 1];
+          base = kab(top);
+          for (int p = T.bkt[li]; p < T.bkt[li + 1]; ++p) base ^= T.W[T.idx[p]].key > top ? 1 : 0;
+        }
+        if (no > d.cap) continue;  // (reported above)
+      } else {
+        // Step 3 alone: the legs merged with the current configuration's worms
+        uint64_t* OUT = d.keyB + size_t(s) * d.cap;
+        const uint64_t* KO = d.keyA + size_t(s) * d.cap;
+        const int nO = cnt_n(d.cntA[s]);
+        int il = 0, io = 0;
+        no = 0;
+        bool bad = false;
+        for (;;) {
+          while (io < nO && !kworm(KO[io])) ++io;
+          while (il < nl && ktag(T.leg[st + il]) == 6) ++il;  // a temporal boundary is no event
+          const uint64_t wk = io < nO ? KO[io] : ~0ull, lk = il < nl ? T.leg[st + il] : ~0ull;
+          if (lk == ~0ull && wk == ~0ull) break;
+          if (no >= d.cap) { bad = true; break; }
+          if (lk < wk) { OUT[no++] = lk; ++il; } else { OUT[no++] = wk; ++io; }
+        }
+        if (bad) { tile_fail(misc, PMWA_ECAPACITY, 6); continue; }
+        base = no ? kab(OUT[no - 1]) : cnt_base(d.cntA[s]);
+      }
+      d.cntB[s] = uint32_t(no) | (uint32_t(base) << 31);
+      if (stop < 6) continue;
+      if (base) add128(olo, ohi, kTwo62, 0);
+      if (nl == 0) {  // a site without legs is one interval of sigma = 0
+        uint64_t v;
+        if (xg_fix(0, kTwo59, d.XQ, v)) add128(qlo, qhi, v, 0);
+        else q += xg_sigma(0, double(kTwo59) * d.XW);
+      }
+    }
+    q += __ull2double_rn(qhi) * 4.0 + __ull2double_rn(qlo) * 0x1p-62;
     if (stop >= 6) {
       for (int o = 16; o > 0; o >>= 1) {
         nv += __shfl_down_sync(0xffffffffu, nv, o);
