@@ -13,12 +13,16 @@
 
 namespace pmwa {
 
-__constant__ double c_zX[257];
-__constant__ double c_zF[257];
-__constant__ double c_zW[256];
-__constant__ double c_zS[256];
-__constant__ unsigned long long c_zK[256];
-__constant__ unsigned long long c_zXF[256];
+// (the strip index differs from lane to lane, and a constant bank serves one
+// address at a time: these tables are in global memory, where a warp's reads go
+// out together)
+__device__ float4 c_zw32[256];
+__device__ double c_zX[257];
+__device__ double c_zF[257];
+__device__ double c_zW[256];
+__device__ double c_zS[256];
+__device__ unsigned long long c_zK[256];
+__device__ unsigned long long c_zXF[256];
 __constant__ unsigned long long c_zRF;
 __constant__ double c_zR;
 // Taylor coefficients 1/n!, n = 0..24: the correctly rounded quotients
@@ -35,6 +39,7 @@ static int upload_constants(const Zig& z) {
   if ((e = cudaMemcpyToSymbol(c_zW, z.W, sizeof z.W))) return int(e);
   if ((e = cudaMemcpyToSymbol(c_zS, z.S, sizeof z.S))) return int(e);
   if ((e = cudaMemcpyToSymbol(c_zK, z.K, sizeof z.K))) return int(e);
+  if ((e = cudaMemcpyToSymbol(c_zw32, z.w32, sizeof z.w32))) return int(e);
   if ((e = cudaMemcpyToSymbol(c_zR, &z.R, sizeof z.R))) return int(e);
   if ((e = cudaMemcpyToSymbol(c_zXF, z.XF, sizeof z.XF))) return int(e);
   if ((e = cudaMemcpyToSymbol(c_zRF, &z.RF, sizeof z.RF))) return int(e);
@@ -272,6 +277,47 @@ __device__ __forceinline__ uint64_t zfix_add(uint64_t a, uint64_t b) { return (a
 // product (u XF[i]) >> 53; accept when u < K[i]; strip 0 past R restarts at
 // R + new deviate; else a binary64 wedge test y < e^-x with a second word.
 // <= z.zcap (64) words.
+
+// The wedge test of strip i > 0 at u, with the second word w2: y < exp_det(-x)
+// for x = u W[i], y = F[i] + t1 (F[i+1] - F[i]), t1 = (w2 >> 11) 2^-53.
+//
+// On the strip's wedge [a, b] = [X[i+1], X[i]] the tangent at a bounds e^-x
+// below, e^-x >= e^-a (1 - (x - a)), and the chord above (e^-x is convex).  With
+// s = 1 - t1 and dl = x - a, y lies below the tangent when s (F[i+1] - F[i]) >
+// F[i+1] dl and above the chord when s (F[i+1] - F[i]) < |slope| dl: products of
+// positive numbers, so binary32 gives each within a relative 2^-21 (dl from the
+// integer u - K[i], exact to its last place; below 2^20 of these the table's
+// rounding counts and the test is left to binary64).  A margin of 2^-16 decides
+// the tests outside the strip between chord and tangent, 98 % of them; the
+// others take the binary64 form.  Binary64 is a long chain of slow operations
+// here: one test cost a warp 3k cycles, and a third of a warp's steps have one
+// (worm creation of a 16x16 domain at beta t = 4: 79k -> 66k cycles a sweep).
+static __device__ __noinline__ bool zig_wedge64(unsigned i, uint64_t u, uint64_t w2) {
+  const double x = __dmul_rn(__ull2double_rn(u), c_zW[i]);
+  const double t1 = __dmul_rn(__ull2double_rn(w2 >> 11), 0x1p-53);
+  const double t2 = __dsub_rn(c_zF[i + 1], c_zF[i]);
+  const double y = __dadd_rn(c_zF[i], __dmul_rn(t1, t2));
+  // (away from the curve by more than eps = F[i+1] 2^-40, far beyond the
+  // rounding of the bounds, of the tables and of exp_det, the bounds give the
+  // exact test's answer)
+  const double fa = c_zF[i + 1], dl = __dsub_rn(x, c_zX[i + 1]), eps = __dmul_rn(fa, 0x1p-40);
+  if (y < __dsub_rn(__dmul_rn(fa, __dsub_rn(1.0, dl)), eps)) return true;
+  if (y > __dadd_rn(__dadd_rn(fa, __dmul_rn(dl, c_zS[i])), eps)) return false;
+  return y < exp_det(-x);
+}
+
+__device__ __forceinline__ bool zig_wedge(const ZigTab& z, unsigned i, uint64_t u, uint64_t w2) {
+  const float4 t = c_zw32[i];  // F[i+1] - F[i], F[i+1], |slope|, W[i]
+  const uint64_t over = u - z.K[i];
+  const float lhs = __ull2float_rn((1ull << 53) - (w2 >> 11)) * 0x1p-53f * t.x;
+  const float dl = __ull2float_rn(over) * t.w;
+  if (over >= (1ull << 20)) {
+    if (lhs > t.y * dl * (1.0f + 0x1p-16f)) return true;
+    if (lhs < t.z * dl * (1.0f - 0x1p-16f)) return false;
+  }
+  return zig_wedge64(i, u, w2);
+}
+
 template <class St>
 __device__ inline uint64_t zig_exp(const ZigTab& z, St& s, int* bad) {
   uint64_t acc = 0;
@@ -283,26 +329,44 @@ __device__ inline uint64_t zig_exp(const ZigTab& z, St& s, int* bad) {
     const uint64_t xf = (__umul64hi(u, xf0) << 11) | ((u * xf0) >> 53);
     if (u < z.K[i]) return zfix_add(acc, xf);
     if (i == 0) { acc = zfix_add(acc, c_zRF); continue; }
-    const double x = __dmul_rn(__ull2double_rn(u), c_zW[i]);
-    const uint64_t w2 = s.word();
-    const double t1 = __dmul_rn(__ull2double_rn(w2 >> 11), 0x1p-53);
-    const double t2 = __dsub_rn(c_zF[i + 1], c_zF[i]);
-    const double y = __dadd_rn(c_zF[i], __dmul_rn(t1, t2));
-    // The test y < exp_det(-x), decided first by bounds of e^-x on the
-    // strip's wedge [a, b] = [X[i+1], X[i]]: the tangent at a below
-    // (e^-x >= e^-a (1 - (x - a))) and the chord above (e^-x is convex).
-    // Away from the curve by more than eps = F[i+1] 2^-40 -- far beyond the
-    // rounding of the bounds, of the tables and of exp_det (a few units in
-    // the last place) -- the bounds give the same answer as the exact test,
-    // which runs only inside that margin.
-    const double fa = c_zF[i + 1], dl = __dsub_rn(x, c_zX[i + 1]), eps = __dmul_rn(fa, 0x1p-40);
-    if (y < __dsub_rn(__dmul_rn(fa, __dsub_rn(1.0, dl)), eps)) return zfix_add(acc, xf);
-    if (y > __dadd_rn(__dadd_rn(fa, __dmul_rn(dl, c_zS[i])), eps)) continue;
-    if (y < exp_det(-x)) return zfix_add(acc, xf);
+    if (zig_wedge(z, i, u, s.word())) return zfix_add(acc, xf);
   }
   *bad = PMWA_ETIMEOUT;
   return 0;
 }
+
+// The same draw one word at a time, for a warp whose lanes each run a chain of
+// their own: every step takes the next word of the lane's stream, so that the
+// lanes stay together (two steps a Philox block) whatever the state of each.
+struct ZigDraw {
+  uint64_t acc, u;   // deviate so far; the wedge's point
+  int i, tries;      // strip of a pending wedge test (0: none); words of this deviate
+  __device__ __forceinline__ void start() { acc = 0; i = 0; tries = 0; }
+  // one word: true when the deviate is complete (in E); *bad when it needs
+  // more than z.zcap tries
+  __device__ __forceinline__ bool step(const ZigTab& z, uint64_t w, uint64_t& E, int* bad) {
+    if (i) {  // the wedge test's word
+      const unsigned k = unsigned(i);
+      i = 0;
+      if (!zig_wedge(z, k, u, w)) { if (tries >= z.zcap) *bad = PMWA_ETIMEOUT; return false; }
+      const uint64_t xf0 = z.XF[k];
+      E = zfix_add(acc, (__umul64hi(u, xf0) << 11) | ((u * xf0) >> 53));
+      return true;
+    }
+    ++tries;
+    const unsigned k = unsigned(w & 255u);
+    u = w >> 11;
+    const uint64_t xf0 = z.XF[k];
+    if (u < z.K[k]) {
+      E = zfix_add(acc, (__umul64hi(u, xf0) << 11) | ((u * xf0) >> 53));
+      return true;
+    }
+    if (k == 0) acc = zfix_add(acc, c_zRF);
+    else i = int(k);
+    if (!i && tries >= z.zcap) *bad = PMWA_ETIMEOUT;
+    return false;
+  }
+};
 
 // Gap of a Bernoulli process of mean spacing S on an integer grid:
 // 1 + floor(E S) from the exact 128-bit product (E 2^58) m, shifted right

@@ -323,6 +323,7 @@ static int lay_strips(double R, Zig* z) {
       z->S[i] = (i == 0) ? 0.0 : (F[i] - F[i + 1]) / (X[i] - X[i + 1]);
       z->K[i] = (uint64_t)std::floor(X[i + 1] / X[i] * 0x1p53);
       z->W[i] = X[i] * 0x1p-53;
+      z->w32[i] = make_float4(float(F[i + 1] - F[i]), float(F[i + 1]), float(-z->S[i]), float(z->W[i]));
       z->XF[i] = (uint64_t)(X[i] * 0x1p58);  // exact: 53-bit X[i] >= 2^-5
     }
     z->RF = (uint64_t)(R * 0x1p58);

@@ -122,6 +122,7 @@ __host__ __device__ inline Dev at_iteration(const Dev& d0, const BatchBase& b, i
 struct Zig {
   double X[257], F[257], W[256];
   double S[256];     // slope (F[i] - F[i+1]) / (X[i] - X[i+1]) of strip i's chord (i >= 1)
+  float4 w32[256];   // binary32 wedge test: F[i+1] - F[i], F[i+1], -S[i], W[i] (i >= 1)
   uint64_t K[256];
   uint64_t XF[256];  // X[i] 2^58 (exact)
   uint64_t RF;       // R 2^58 (exact)

@@ -474,7 +474,7 @@ __device__ void boundary_warp(const Dev& d, int dir, int t, uint64_t* stage, con
 
 constexpr int kBoundaryWarps = 4;  // bonds (warps) per block
 
-__global__ void __launch_bounds__(32 * kBoundaryWarps) k_boundary(const __grid_constant__ Dev d, int dir) {
+__global__ void __launch_bounds__(32 * kBoundaryWarps, 7) k_boundary(const __grid_constant__ Dev d, int dir) {
   extern __shared__ __align__(16) unsigned char bsm[];
   if (instance_failed(d.err)) return;
   const ZigTab Z = zig_stage(bsm, d.zig_cap, d.worm_tries);
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(32 * kBoundaryWarps) k_boundary(const __grid_c
 
 // Batched form: each block serves bonds t0 .. t0 + kBoundaryWarps - 1 of one
 // instance, when that instance's boundary step is due at iteration `it`.
-__global__ void __launch_bounds__(32 * kBoundaryWarps) k_boundary_batch(const Dev* __restrict__ devs,
+__global__ void __launch_bounds__(32 * kBoundaryWarps, 7) k_boundary_batch(const Dev* __restrict__ devs,
                                                                         const BatchBase* __restrict__ base,
                                                                         const int2* __restrict__ work, int it,
                                                                         int dir, int cap) {
@@ -607,7 +607,7 @@ __device__ void temporal_warp(const Dev& d, int s, uint64_t* K, const ZigTab& Z)
   if (lane == 0) d.cntA[s] = cnt_make(n, n ? kab(K[n - 1]) : base);
 }
 
-__global__ void __launch_bounds__(32 * kTemporalWarps) k_temporal(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(32 * kTemporalWarps, 7) k_temporal(const __grid_constant__ Dev d) {
   extern __shared__ __align__(16) unsigned char tsm[];
   if (instance_failed(d.err)) return;
   const ZigTab Z = zig_stage(tsm, d.zig_cap, d.worm_tries);
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(32 * kTemporalWarps) k_temporal(const __grid_c
 // Batched form: each block serves sites t0 .. t0 + kTemporalWarps - 1 of one
 // instance, when that instance has temporal domains and its Step 1 is due at
 // iteration `it`.
-__global__ void __launch_bounds__(32 * kTemporalWarps) k_temporal_batch(const Dev* __restrict__ devs,
+__global__ void __launch_bounds__(32 * kTemporalWarps, 7) k_temporal_batch(const Dev* __restrict__ devs,
                                                                         const BatchBase* __restrict__ base,
                                                                         const int2* __restrict__ work, int it,
                                                                         int cap) {

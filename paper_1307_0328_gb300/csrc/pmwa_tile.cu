@@ -914,6 +914,145 @@ __device__ int small_passes(const Tile& T, int dom, int nw, int lane) {
 
 }  // namespace
 
+// Step 4 (Eq. 1) on every site of the domain (all threads): thread tid takes
+// sites tid, tid + NT, ...  A site's words come from one stream, interval
+// after interval, so a site is one chain; what a word is used for depends on
+// the words before it (a gap of the rate-eta process, its wedge test, the
+// parity sampler's two extra words, a new worm's label).  The lanes of a warp
+// take one word each a step, whatever their state, so that the Philox blocks
+// -- most of the arithmetic -- are evaluated by all lanes together and the
+// common state, a gap longer than its interval, is shared; a loop of draws per
+// interval had the lanes in different places of nested loops.  The sampler
+// and the order of the words are sample_worms'.  Cycles a sweep, loop of draws
+// -> steps -> steps with the binary32 wedge test: 16x16 sites 92k -> 79k -> 66k
+// at beta t = 4, 273k -> 225k -> 188k at beta t = 16; 4x4 sites with 188 legs
+// each 380k -> 337k -> 287k.
+__device__ __forceinline__ void create_worms(const Tile& T, const ZigTab& Z, int tid, int NT) {
+  const Dev& d = *T.d;
+  enum { kDone, kState, kGap, kKeep, kExtra, kLabel };
+  uint64_t offs[kMaxWormsPerInterval];
+  int li = tid, state = kDone, bad = 0;
+  uint32_t unit = 0, block = 0;
+  int st = 0, nl = 0, k = 0;            // the site's legs, its current interval
+  uint64_t lo = 0, M = 0, pos = 0;      // interval: lower leg, worm grid points; last proposal
+  int sigma = 0, p = 0, n = 0, tries = 0, o = 0, j = 0;
+  bool first = true;
+  ZigDraw zd;
+  zd.start();
+  auto attempt = [&] { n = 0; first = true; state = kGap; zd.start(); };
+  auto retry = [&] {
+    if (++tries >= Z.wtries) bad = PMWA_ETIMEOUT;
+    attempt();
+  };
+  // the interval from leg st + k on (or the next one with grid points), else
+  // the end of the site
+  auto enter = [&] {
+    for (;;) {
+      if (k == nl) { state = kDone; li += NT; return; }
+      lo = T.leg[st + k];
+      const uint64_t hi = T.leg[st + (k + 1 == nl ? 0 : k + 1)];
+      M = wpts(kpk(lo), kpk(hi));
+      p = kab(lo);
+      sigma = p ^ kbl(hi);
+      if (M) break;
+      if (sigma) { bad = PMWA_EINVARIANT; return; }
+      T.wcnt[st + k] = 0;
+      ++k;
+    }
+    tries = 0;
+    attempt();
+  };
+  auto begin = [&] {
+    const int s = T.gsite(li);
+    st = T.off[li];
+    nl = T.off[li + 1] - st;
+    unit = uint32_t(s);
+    block = 0;
+    k = 0;
+    if (nl == 0) { state = kState; return; }
+    // (the state of a site whose delimiters are temporal boundaries only and
+    // which keeps no worm: all its boundary states are equal)
+    T.base[li] = uint8_t(kab(T.leg[st]));
+    enter();
+  };
+  // the interval has its n worms
+  auto accept = [&] {
+    if (nl) T.wcnt[st + k] = uint8_t(n);  // (n <= kMaxWormsPerInterval)
+    if (n == 0) { ++k; if (nl) enter(); else { state = kDone; li += NT; } return; }
+    o = atomicAdd(&T.misc->nworms, n);
+    const int sl = nl ? slab_of_m(d, wm_above(kpk(lo))) : 0;  // an interval lies inside one temporal slab
+    atomicAdd(&T.misc->wslab[sl], n);
+    if (o + n > d.wcap) { bad = PMWA_ECAPACITY; return; }
+    j = 0;
+    state = kLabel;
+  };
+  auto step = [&](uint64_t w) {
+    if (state == kGap) {
+      uint64_t E;
+      if (zd.step(Z, w, E, &bad)) {
+        const uint64_t g = grid_gap(E, d.SWs), nxt = first ? g - 1 : pos + g;
+        first = false;
+        zd.start();
+        if (nxt < M) {
+          pos = nxt;
+          if (n >= kMaxWormsPerInterval) bad = PMWA_ECAPACITY; else offs[n++] = pos;
+        } else if (sigma == 1 && M <= d.SWI) {
+          if (n & 1) retry(); else state = kKeep;
+        } else if ((n & 1) == sigma) {
+          accept();
+        } else {
+          retry();
+        }
+      }
+    } else if (state == kKeep) {
+      if (__umul64hi(w, uint64_t(n + 1)) != 0) retry(); else state = kExtra;
+    } else if (state == kExtra) {
+      const uint64_t extra = __umul64hi(w, M);
+      int at = n;
+      bool clash = false;
+      for (int e = 0; e < n; ++e) {
+        if (offs[e] == extra) { clash = true; break; }
+        if (offs[e] > extra) { at = e; break; }
+      }
+      if (clash) {
+        retry();
+      } else if (n >= kMaxWormsPerInterval) {
+        bad = PMWA_ECAPACITY;
+      } else {
+        for (int e = n; e > at; --e) offs[e] = offs[e - 1];
+        offs[at] = extra;
+        ++n;
+        accept();
+      }
+    } else if (state == kLabel) {
+      const uint64_t m0 = nl ? wm_above(kpk(lo)) : 0;
+      T.W[o + j] = WormRec{wkey((m0 + offs[j]) & (kTwo59 - 1), int(w & 1), p ^ 1 ^ (j & 1)), w >> 1, uint16_t(li),
+                           nl ? uint16_t(st + k) : kNone, uint16_t(nl ? slab_of_m(d, m0) : 0), 0};
+      if (++j == n) { ++k; if (nl) enter(); else { state = kDone; li += NT; } }
+    } else if (state == kState) {  // a site without legs: its state, then one interval round the circle
+      p = int(w >> 63);
+      T.base[li] = uint8_t(p);
+      M = kTwo59;
+      sigma = 0;
+      tries = 0;
+      attempt();
+    }
+  };
+  for (;;) {
+    if (state == kDone && li < T.nds && !bad) begin();
+    const bool run = state != kDone && !bad;
+    if (!__any_sync(0xffffffffu, run)) {
+      if (__any_sync(0xffffffffu, state == kDone && li < T.nds && !bad)) continue;
+      break;
+    }
+    const P4 b = philox(block, unit, c2_word(kRegen, 0, d.replica), d.sweep, d.key0, d.key1);
+    ++block;
+    if (run) step(uint64_t(b.x) | (uint64_t(b.y) << 32));
+    if (run && state != kDone && !bad) step(uint64_t(b.z) | (uint64_t(b.w) << 32));
+  }
+  if (bad) tile_fail(T.misc, bad, 4);
+}
+
 // ---------------------------------------------------------------------------
 // Where the sources of a site's Step-3 merge start and end for one part of
 // its circle: the old events [o0, o1), the new legs of its four bonds
@@ -1220,53 +1359,7 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
 
   if (stop >= 4) {
     // ---- phase 3: Step 4, worms of every interval (the pool is dead now)
-    for (int li = tid; li < nds; li += NT) {
-      const int s = T.gsite(li);
-      const int st = T.off[li], nl = T.off[li + 1] - st;
-      Stream rs;
-      rs.init(d.key0, d.key1, uint32_t(s), c2_word(kRegen, 0, d.replica), d.sweep);
-      uint64_t offs[kMaxWormsPerInterval];
-      int bad = 0;
-      if (nl == 0) {
-        const int s0 = int(rs.word() >> 63);
-        T.base[li] = uint8_t(s0);
-        const int n = sample_worms<kMaxWormsPerInterval>(Z, rs, kTwo59, 0, d.SWs, d.SWI, offs, &bad);
-        if (!bad && n > 0) {
-          const int o = atomicAdd(&misc->nworms, n);
-          atomicAdd(&misc->wslab[0], n);
-          if (o + n > d.wcap) bad = PMWA_ECAPACITY;
-          for (int k = 0; k < n && !bad; ++k) {
-            const uint64_t w = rs.word();
-            T.W[o + k] = WormRec{wkey(offs[k], int(w & 1), s0 ^ 1 ^ (k & 1)), w >> 1, uint16_t(li), kNone, 0, 0};
-          }
-        }
-      } else {
-        // (the state of a site whose delimiters are temporal boundaries only
-        // and which keeps no worm: all its boundary states are equal)
-        T.base[li] = uint8_t(kab(T.leg[st]));
-        for (int k = 0; k < nl && !bad; ++k) {
-          const uint64_t lo = T.leg[st + k], hi = T.leg[st + (k + 1 == nl ? 0 : k + 1)];
-          const uint64_t M = wpts(kpk(lo), kpk(hi));
-          const int p = kab(lo), sigma = p ^ kbl(hi);
-          const int n = sample_worms<kMaxWormsPerInterval>(Z, rs, M, sigma, d.SWs, d.SWI, offs, &bad);
-          T.wcnt[st + k] = uint8_t(n > 0 ? min(n, 255) : 0);
-          if (n > 255) bad = PMWA_ECAPACITY;
-          if (bad || n <= 0) continue;
-          const int o = atomicAdd(&misc->nworms, n);
-          if (o + n > d.wcap) { bad = PMWA_ECAPACITY; break; }
-          const uint64_t m0 = wm_above(kpk(lo));
-          // an interval lies inside one temporal slab (boundaries delimit it)
-          const int sl = slab_of_m(d, m0);
-          atomicAdd(&misc->wslab[sl], n);
-          for (int j = 0; j < n; ++j) {
-            const uint64_t w = rs.word();
-            T.W[o + j] = WormRec{wkey((m0 + offs[j]) & (kTwo59 - 1), int(w & 1), p ^ 1 ^ (j & 1)), w >> 1,
-                                 uint16_t(li), uint16_t(st + k), uint16_t(sl), 0};
-          }
-        }
-      }
-      if (bad) tile_fail(misc, bad, 4);
-    }
+    create_worms(T, Z, tid, NT);
     __syncthreads();
     phase_tick(d, 2, tclk);
     if (misc->err) goto fail;
@@ -1315,8 +1408,8 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
   // and smaller CTAs), and consecutive lanes write consecutive keys.  The
   // occupied time of a site is 2^62 when its state at the origin is 1, plus
   // the times where the state falls and minus those where it rises.  Cycles a
-  // sweep, with xg_series: 16x16 sites 75k -> 60k at beta t = 4, 153k -> 113k
-  // at beta t = 16; 4x4 sites with 188 legs each 165k -> 92k.
+  // sweep, with xg_series: 16x16 sites 75k -> 60k at beta t = 4, 153k -> 112k
+  // at beta t = 16; 4x4 sites with 188 legs each 165k -> 91k.
   {
     const int nw = (stop >= 4) ? misc->nworms : 0;
     const int NB = d.ntau > 1 ? d.ntau : 0;  // temporal boundaries in the leg table: no events
@@ -1437,7 +1530,6 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
         else q += xg_sigma(0, double(kTwo59) * d.XW);
       }
     }
-    q += __ull2double_rn(qhi) * 4.0 + __ull2double_rn(qlo) * 0x1p-62;
     if (stop >= 6) {
       for (int o = 16; o > 0; o >>= 1) {
         nv += __shfl_down_sync(0xffffffffu, nv, o);
@@ -1446,8 +1538,13 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
         const uint64_t blo = __shfl_down_sync(0xffffffffu, olo, o);
         const uint64_t bhi = __shfl_down_sync(0xffffffffu, ohi, o);
         add128(olo, ohi, blo, bhi);
-        q += __shfl_down_sync(0xffffffffu, q, o);
+        const uint64_t clo = __shfl_down_sync(0xffffffffu, qlo, o);
+        const uint64_t chi = __shfl_down_sync(0xffffffffu, qhi, o);
+        add128(qlo, qhi, clo, chi);
       }
+      if (__any_sync(0xffffffffu, q != 0.0))  // (binary64 terms are rare)
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_down_sync(0xffffffffu, q, o);
+      q += __ull2double_rn(qhi) * 4.0 + __ull2double_rn(qlo) * 0x1p-62;
       if ((tid & 31) == 0) {
         pmwa_row* r = d.rows + d.row;
         if (nv) atomicAdd(reinterpret_cast<unsigned long long*>(&r->n_v), (unsigned long long)nv);

@@ -126,3 +126,59 @@ def test_binary32_heat_bath_agrees_outside_its_margin(V, mu, beta, eta):
     assert worst < 2.0 ** -16, worst
     assert decided > 40000
     assert agree == decided
+
+
+def _wedge32(F, X, K, i, u, w2):
+    """The binary32 pre-decision of the wedge test (zig_wedge): +1 accept, -1
+    reject, 0 undecided, with the tables and operations in numpy float32."""
+    f = np.float32
+    slope = np.zeros(256)
+    slope[1:] = (F[1:256] - F[2:257]) / (X[1:256] - X[2:257])
+    W = X[:256] * 2.0 ** -53
+    tx, ty, tz, tw = (F[i + 1] - F[i]).astype(f), F[i + 1].astype(f), (-slope[i]).astype(f), W[i].astype(f)
+    over = u - K[i]
+    lhs = (np.uint64(1 << 53) - (w2 >> np.uint64(11))).astype(f) * f(2.0 ** -53) * tx
+    dl = over.astype(f) * tw
+    out = np.zeros(len(u), dtype=np.int8)
+    big = over >= np.uint64(1 << 20)
+    acc = big & (lhs > ty * dl * f(1.0 + 2.0 ** -16))
+    rej = big & (lhs < tz * dl * f(1.0 - 2.0 ** -16))
+    assert not (acc & rej).any()
+    out[acc] = 1
+    out[rej] = -1
+    return out
+
+
+def test_binary32_wedge_decisions_agree_with_the_exact_test():
+    """Random wedge points, and points placed within a few 2^-20 of the
+    tangent, the chord and the curve: no binary32 decision contradicts
+    y < e^-x (by more than binary64 rounding), and few random ones are left."""
+    t = P.pmwa_tables(Lx=4, Ly=4, beta=2.0, eta=0.2)
+    X, F, K = t["X"], t["F"], t["K"]
+    rng = np.random.default_rng(11)
+    n = 2000000
+    i = rng.integers(1, 256, n)
+    span = np.uint64(1 << 53) - K[i]
+    u = K[i] + (rng.random(n) * span.astype(float)).astype(np.uint64)
+    u = np.minimum(u, np.uint64((1 << 53) - 1))
+    w2 = rng.integers(0, 1 << 63, n, dtype=np.uint64) * np.uint64(2)
+    x = u.astype(float) * (X[i] * 2.0 ** -53)
+    # the last three quarters: y set near the tangent, the chord, the curve
+    dl = x - X[i + 1]
+    slope = (F[i] - F[i + 1]) / (X[i] - X[i + 1])
+    q = n // 4
+    for part, y in ((1, F[i + 1] * (1 - dl)), (2, F[i + 1] + dl * slope), (3, np.exp(-x))):
+        s = slice(part * q, (part + 1) * q)
+        t1 = (y[s] - F[i[s]]) / (F[i[s] + 1] - F[i[s]]) * (1 + (rng.random(q) - 0.5) * 2.0 ** -18)
+        w2[s] = (np.clip(t1, 0.0, 1.0 - 2.0 ** -53) * 2.0 ** 53).astype(np.uint64) << np.uint64(11)
+    y = F[i] + (w2 >> np.uint64(11)).astype(float) * 2.0 ** -53 * (F[i + 1] - F[i])
+    got = _wedge32(F, X, K, i, u, w2)
+    e = np.exp(-x)
+    assert not ((got == 1) & (y > e * (1 + 1e-14))).any()
+    assert not ((got == -1) & (y < e * (1 - 1e-14))).any()
+    # undecided: between chord and tangent, whose distance at dl is at most
+    # F[i+1] dl delta / 2 of a strip F[i+1] delta (1 - delta / 2) high (delta
+    # its width), on average over dl a share delta / 4 / (1 - delta / 2), and
+    # the two margins
+    delta = X[i[:q]] - X[i[:q] + 1]
+    assert (got[:q] == 0).mean() < 1.05 * (delta / 4 / (1 - delta / 2)).mean() + 1e-4
