@@ -144,7 +144,8 @@ struct Tile {
   uint64_t* old;   // [oldcap] the domain's current configuration (when staged)
   int* wmo;        // [nds + 1] on-the-fly windows: start of each site's old worms in wm[]
   uint64_t* wm;    // [wcap] grid points of the current configuration's worms, by site
-  bool staged;
+  bool staged;     // the current configuration is in old[]
+  bool early;      // it is in leg[] (from off[li] on for site li) until the merge
   int x0, y0, nds, nsub;
   int ngrp;  // Step-5 chains: sub-blocks x temporal slabs
 
@@ -153,6 +154,8 @@ struct Tile {
   __device__ const uint64_t* okeys(int li, int s) const {
     return staged ? old + soff[li] : d->keyA + size_t(s) * d->cap;
   }
+  // the same before the merge writes legs: the copy in the leg table too
+  __device__ const uint64_t* okeys_early(int li, int s) const { return early ? leg + off[li] : okeys(li, s); }
   __device__ int lsite(int s) const { return (s % d->Lx - x0) + d->dom_x * (s / d->Lx - y0); }
   __device__ int sub_of(int li, int pass) const {
     const int B = d->sub_block;
@@ -1086,50 +1089,72 @@ __device__ __forceinline__ MergeRange merge_range(const Tile& T, const uint64_t*
 
 // The Step-3 merge of one part of site li's circle into the leg table from
 // position o: the kept old events, the new legs of its four bonds and the
-// temporal boundaries (tag-6 delimiters whose state above and below is the
-// worldline's state there in the current configuration; Step 3 changes no
-// state), in time order.  The site is the lower site of bonds 0 and 1 (its
-// state in bit 0 of a candidate) and the upper site of bonds 2 and 3 (bit 1).
+// temporal boundaries (tag-6 delimiters), in time order.  A new leg's and a
+// boundary's states above and below are the worldline's state there, that of
+// the last old event passed (Step 3 changes no state).
+//
+// A chain of as many steps as the site has old events and new legs, one
+// thread a site: each step takes the earliest of the six heads, kept or not,
+// by selects -- no lane waits for another's branch -- and the old list, which
+// is read from L2, is fetched four keys ahead.  Cycles of the whole phase a
+// sweep: 16x16 sites 108k -> 76k at beta t = 4, 175k -> 101k at beta t = 16; 4x4
+// sites with 188 legs each 532k -> 228k.
 template <bool OTF>
 __device__ __forceinline__ void merge_site(const Tile& T, int li, const uint64_t* KO, int nO, int base0,
                                            const int lb[4], const MergeRange& R, int o) {
   const Dev& d = *T.d;
-  // each run's next candidate (h) and how many remain (m)
-  const uint64_t* q0 = T.pool + (lb[0] >= 0 ? T.boff[lb[0]] : 0) + R.s0;
-  const uint64_t* q1 = T.pool + (lb[1] >= 0 ? T.boff[lb[1]] : 0) + R.s1;
-  const uint64_t* q2 = T.pool + (lb[2] >= 0 ? T.boff[lb[2]] : 0) + R.s2;
-  const uint64_t* q3 = T.pool + (lb[3] >= 0 ? T.boff[lb[3]] : 0) + R.s3;
-  int m0 = R.e0 - R.s0, m1 = R.e1 - R.s1, m2 = R.e2 - R.s2, m3 = R.e3 - R.s3;
-  uint64_t h0 = m0 ? q0[0] : 0, h1 = m1 ? q1[0] : 0, h2 = m2 ? q2[0] : 0, h3 = m3 ? q3[0] : 0;
+  unsigned out = 0;  // leg tags of the site whose bonds leave the domain: their legs all stay
+#pragma unroll
+  for (int t = 0; t < 6; ++t) out |= (T.tinfo[li * 6 + t] & 2) ? 1u << t : 0u;
+  // each run's next candidate (h), its place in the pool (i) and the run's end (e)
+  int i0 = (lb[0] >= 0 ? T.boff[lb[0]] : 0), i1 = (lb[1] >= 0 ? T.boff[lb[1]] : 0);
+  int i2 = (lb[2] >= 0 ? T.boff[lb[2]] : 0), i3 = (lb[3] >= 0 ? T.boff[lb[3]] : 0);
+  const int e0 = i0 + R.e0, e1 = i1 + R.e1, e2 = i2 + R.e2, e3 = i3 + R.e3;
+  i0 += R.s0; i1 += R.s1; i2 += R.s2; i3 += R.s3;
+  const uint64_t none = ~0ull;
+  uint64_t h0 = i0 < e0 ? T.pool[i0] : none, h1 = i1 < e1 ? T.pool[i1] : none;
+  uint64_t h2 = i2 < e2 ? T.pool[i2] : none, h3 = i3 < e3 ? T.pool[i3] : none;
   int io = R.o0, ib = R.t0;
-  uint64_t tb = ib < R.t1 ? tb_pk(d, ib) : 0;
+  const int on = R.o1;
+  uint64_t r0 = io < on ? KO[io] : none, r1 = io + 1 < on ? KO[io + 1] : none;
+  uint64_t r2 = io + 2 < on ? KO[io + 2] : none, r3 = io + 3 < on ? KO[io + 3] : none;
+  uint64_t tb = ib < R.t1 ? tb_pk(d, ib) << 2 : none;
+  uint64_t cur = nO ? uint64_t(kab(KO[(io ? io : nO) - 1])) : uint64_t(base0);
   for (;;) {
-    uint64_t ko = 0;
-    while (io < R.o1 && !kept_leg<OTF>(T, li, ko = KO[io])) ++io;
-    uint64_t best = ~0ull;
-    int src = -1;
-    if (io < R.o1) { best = kpk(ko); src = 4; }
-    if (m0 && (h0 >> 2) < best) { best = h0 >> 2; src = 0; }
-    if (m1 && (h1 >> 2) < best) { best = h1 >> 2; src = 1; }
-    if (m2 && (h2 >> 2) < best) { best = h2 >> 2; src = 2; }
-    if (m3 && (h3 >> 2) < best) { best = h3 >> 2; src = 3; }
-    if (ib < R.t1 && tb < best) { best = tb; src = 5; }
-    if (src < 0) break;
-    uint64_t key;
-    switch (src) {
-      case 4: key = ko; ++io; break;
-      case 5: {
-        const uint64_t bst = uint64_t(slot_state(KO, nO, base0, best));
-        key = (best << 2) | (bst << 1) | bst;
-        if (++ib < R.t1) tb = tb_pk(d, ib);
-        break;
+    // (times differ, so whole words compare as times do)
+    const bool s01 = h1 < h0, s23 = h3 < h2;
+    const uint64_t a = s01 ? h1 : h0, b = s23 ? h3 : h2;
+    const bool sb = b < a;
+    const uint64_t c = sb ? b : a, t = min(r0, tb);
+    const bool fresh = c < t, bound = !fresh && tb < r0;
+    const uint64_t best = fresh ? c : t;
+    if (best == none) break;
+    if (fresh || bound) {
+      T.leg[o++] = (best & ~3ull) | (cur * 3);
+    } else {
+      const int tag = ktag(r0);
+      bool keep = tag != 7 && (kab(r0) != kbl(r0) || ((out >> tag) & 1));
+      if (OTF && !keep && tag != 7) {
+        const uint64_t pos = kpk(r0) >> 3;
+        keep = !(in_win(T, li, pos) || in_win(T, T.nbr[li * 6 + tag], pos));
       }
-      case 0: { const uint64_t st = h0 & 1; key = ((h0 >> 2) << 2) | (st << 1) | st; if (--m0) h0 = *++q0; break; }
-      case 1: { const uint64_t st = h1 & 1; key = ((h1 >> 2) << 2) | (st << 1) | st; if (--m1) h1 = *++q1; break; }
-      case 2: { const uint64_t st = (h2 >> 1) & 1; key = ((h2 >> 2) << 2) | (st << 1) | st; if (--m2) h2 = *++q2; break; }
-      default: { const uint64_t st = (h3 >> 1) & 1; key = ((h3 >> 2) << 2) | (st << 1) | st; if (--m3) h3 = *++q3; break; }
+      if (keep) T.leg[o++] = r0;
+      cur = uint64_t(kab(r0));
+      r0 = r1; r1 = r2; r2 = r3;
+      r3 = io + 4 < on ? KO[io + 4] : none;
+      ++io;
     }
-    T.leg[o++] = key;
+    if (bound) tb = ++ib < R.t1 ? tb_pk(d, ib) << 2 : none;
+    if (fresh) {
+      const int run = sb ? (s23 ? 3 : 2) : (s01 ? 1 : 0);
+      const int at = 1 + (run == 0 ? i0 : run == 1 ? i1 : run == 2 ? i2 : i3);
+      const int end = run == 0 ? e0 : run == 1 ? e1 : run == 2 ? e2 : e3;
+      const uint64_t nx = at < end ? T.pool[at] : none;
+      if (run == 0) { h0 = nx; i0 = at; }
+      if (run == 1) { h1 = nx; i1 = at; }
+      if (run == 2) { h2 = nx; i2 = at; }
+      if (run == 3) { h3 = nx; i3 = at; }
+    }
   }
 }
 
@@ -1168,7 +1193,7 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
   T.sub = reinterpret_cast<uint16_t*>(sm + d.sm_sub);
   T.soff = reinterpret_cast<int*>(sm + d.sm_soff);
   T.old = reinterpret_cast<uint64_t*>(sm + d.sm_old);
-  T.staged = false;
+  T.staged = T.early = false;
   T.x0 = (dom % d.ndx) * d.dom_x;
   T.y0 = (dom / d.ndx) * d.dom_y;
   T.nds = d.dom_x * d.dom_y;
@@ -1229,6 +1254,27 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
     }
     __syncthreads();
   }
+  // Else the leg table, empty until the merge, holds the lists for phase 1 and
+  // the merge's counts where they fit: every bond reads two of them key by
+  // key, 29 cycles a key instead of L2's several hundred.  (The counts of the
+  // merge then go through the worm-count bytes: 8 a site.)  Cycles of the
+  // candidate phase a sweep: 254k -> 146k at 16x16 sites and beta t = 16, 598k
+  // -> 340k at 4x4 sites with 188 legs each; 94k -> 97k at beta t = 4, which the
+  // counts win back.
+  if (!T.staged && d.legcap >= 8 * nds) {
+    for (int li = tid; li < nds; li += NT) T.off[li] = cnt_n(d.cntA[T.gsite(li)]);
+    __syncthreads();
+    T.early = block_scan(T.off, nds, wsum) <= d.legcap;
+    if (T.early) {
+      const int lane = tid & 31;
+      for (int li = tid >> 5; li < nds; li += NT >> 5) {
+        const uint64_t* KO = d.keyA + size_t(T.gsite(li)) * d.cap;
+        const int st = T.off[li], n = T.off[li + 1] - st;
+        for (int k = lane; k < n; k += 32) T.leg[st + k] = KO[k];
+      }
+    }
+    __syncthreads();
+  }
 
   if (OTF) {
     // the worms of the current configuration, by site: the windows of the
@@ -1237,7 +1283,7 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
     T.wm = reinterpret_cast<uint64_t*>(sm + d.sm_wm);
     for (int li = tid; li < nds; li += NT) {
       const int s = T.gsite(li), n = cnt_n(d.cntA[s]);
-      const uint64_t* KO = T.okeys(li, s);
+      const uint64_t* KO = T.okeys_early(li, s);
       int c = 0;
       for (int k = 0; k < n; ++k) c += kworm(KO[k]) ? 1 : 0;
       T.wmo[li] = c;
@@ -1248,7 +1294,7 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
     if (misc->err) goto fail;
     for (int li = tid; li < nds; li += NT) {
       const int s = T.gsite(li), n = cnt_n(d.cntA[s]);
-      const uint64_t* KO = T.okeys(li, s);
+      const uint64_t* KO = T.okeys_early(li, s);
       int o = T.wmo[li];
       for (int k = 0; k < n; ++k) if (kworm(KO[k])) T.wm[o++] = kpk(KO[k]) >> 3;
     }
@@ -1263,7 +1309,7 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
     int n = 0, bad = 0;
     if (d.has_vertices && !boundary_bond(d, a, dir)) {
       const int b = site_step(d, a, dir, +1);
-      n = bond_candidates<OTF>(d, Z, a, dir, T.okeys(li, a), T.okeys(T.lsite(b), b), buf,
+      n = bond_candidates<OTF>(d, Z, a, dir, T.okeys_early(li, a), T.okeys_early(T.lsite(b), b), buf,
                                min(d.capb, kMaxCandPerBond), &bad, &T, li, T.lsite(b));
     }
     if (bad) { tile_fail(misc, bad, 31); n = 0; }
@@ -1293,7 +1339,7 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
     for (int un = tid; un < units; un += NT) {
       const int li = two ? un % nds : un, h = two ? un / nds : -1;
       const int s = T.gsite(li);
-      const uint64_t* KO = T.okeys(li, s);
+      const uint64_t* KO = T.okeys_early(li, s);
       const int nO = cnt_n(d.cntA[s]);
       int lb[4];
       site_bonds(T, li, lb);
@@ -1301,12 +1347,12 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
       int c = 0;
       for (int k = R.o0; k < R.o1; ++k) c += kept_leg<OTF>(T, li, KO[k]);
       c += (R.e0 - R.s0) + (R.e1 - R.s1) + (R.e2 - R.s2) + (R.e3 - R.s3) + (R.t1 - R.t0);
-      if (two) hc[h * nds + li] = c;
+      if (two || T.early) hc[(two ? h * nds : 0) + li] = c;
       else T.off[li] = c;
     }
-    if (two) {
+    if (two || T.early) {
       __syncthreads();
-      for (int li = tid; li < nds; li += NT) T.off[li] = hc[li] + hc[nds + li];
+      for (int li = tid; li < nds; li += NT) T.off[li] = hc[li] + (two ? hc[nds + li] : 0);
     }
     __syncthreads();
     if (block_scan(T.off, nds, wsum) > d.legcap) { if (tid == 0) tile_fail(misc, PMWA_ECAPACITY, 33); }
