@@ -76,6 +76,14 @@ __device__ __forceinline__ void tile_fail(Misc* m, int code, int where) {
   if (atomicCAS(&m->err, 0, code) == 0) m->where = where;
 }
 
+// item of thread tid when n <= NT items are spread over the warps (n: none);
+// tid when there are more
+__device__ __forceinline__ int spread(int tid, int NT, int n) {
+  if (n >= NT) return tid;
+  const int warps = NT >> 5, per = (n + warps - 1) / warps, lane = tid & 31;
+  return lane < per ? (tid >> 5) * per + lane : n;
+}
+
 // exclusive scan of a[0..n) in place (a[n] receives the total); all threads
 __device__ int block_scan(int* a, int n, int* wsum) {
   const int t = threadIdx.x, T = blockDim.x, lane = t & 31, wid = t >> 5, nw = T >> 5;
@@ -206,7 +214,9 @@ __device__ int bond_candidates(const Dev& d, const ZigTab& z, int a, int dir, co
     pos = nxt;
     if (OTF && !(in_win(*T, la, pos) || in_win(*T, lb, pos))) continue;
     const uint64_t pk = (pos << 3) | tag;
+    while (ia + 4 <= nA && kpk(KA[ia + 3]) < pk) ia += 4;
     while (ia < nA && kpk(KA[ia]) < pk) ++ia;
+    while (ib + 4 <= nB && kpk(KB[ib + 3]) < pk) ib += 4;
     while (ib < nB && kpk(KB[ib]) < pk) ++ib;
     if (ia < nA && kpk(KA[ia]) == pk && kab(KA[ia]) != kbl(KA[ia])) continue;  // a kink holds the point
     const int na = nA ? kab(KA[ia ? ia - 1 : nA - 1]) : cnt_base(ca);
@@ -934,7 +944,7 @@ __device__ __forceinline__ void create_worms(const Tile& T, const ZigTab& Z, int
   const Dev& d = *T.d;
   enum { kDone, kState, kGap, kKeep, kExtra, kLabel };
   uint64_t offs[kMaxWormsPerInterval];
-  int li = tid, state = kDone, bad = 0;
+  int li = spread(tid, NT, T.nds), state = kDone, bad = 0;
   uint32_t unit = 0, block = 0;
   int st = 0, nl = 0, k = 0;            // the site's legs, its current interval
   uint64_t lo = 0, M = 0, pos = 0;      // interval: lower leg, worm grid points; last proposal
@@ -1059,31 +1069,42 @@ __device__ __forceinline__ void create_worms(const Tile& T, const ZigTab& Z, int
 // ---------------------------------------------------------------------------
 // Where the sources of a site's Step-3 merge start and end for one part of
 // its circle: the old events [o0, o1), the new legs of its four bonds
-// [s_j, e_j) of each run, the temporal boundaries [t0, t1).  h = -1: the
-// whole circle; h = 0 / 1: the time keys below / from 2^61.
+// [s_j, e_j) of each run, the temporal boundaries [t0, t1).  Part h of P (a
+// power of two) holds the time keys from h 2^62 / P up to the next part's.
+// o0 >= 0: the first old event, known from before (else it is looked up).
 struct MergeRange {
   int o0, o1, s0, e0, s1, e1, s2, e2, s3, e3, t0, t1;
 };
 
 __device__ __forceinline__ MergeRange merge_range(const Tile& T, const uint64_t* KO, int nO, const int lb[4],
-                                                  int h) {
+                                                  int h, int P, int o0, int o1) {
   const Dev& d = *T.d;
-  const uint64_t cut = 1ull << 61;
   const int n0 = lb[0] >= 0 ? T.bcnt[lb[0]] : 0, n1 = lb[1] >= 0 ? T.bcnt[lb[1]] : 0;
   const int n2 = lb[2] >= 0 ? T.bcnt[lb[2]] : 0, n3 = lb[3] >= 0 ? T.bcnt[lb[3]] : 0;
   const int NB = d.ntau > 1 ? d.ntau : 0;
   MergeRange R{0, nO, 0, n0, 0, n1, 0, n2, 0, n3, 0, NB};
-  if (h < 0) return R;
+  if (P == 1) return R;
+  const uint64_t part = kTwo62 / uint64_t(P);
   // (a candidate c of the pool has the time key c >> 2 = kpk(c))
-  const int xo = slot_lower(KO, nO, cut);
-  const int x0 = n0 ? slot_lower(T.pool + T.boff[lb[0]], n0, cut) : 0;
-  const int x1 = n1 ? slot_lower(T.pool + T.boff[lb[1]], n1, cut) : 0;
-  const int x2 = n2 ? slot_lower(T.pool + T.boff[lb[2]], n2, cut) : 0;
-  const int x3 = n3 ? slot_lower(T.pool + T.boff[lb[3]], n3, cut) : 0;
-  int xt = 0;
-  while (xt < NB && tb_pk(d, xt) < cut) ++xt;
-  if (h == 0) { R.o1 = xo; R.e0 = x0; R.e1 = x1; R.e2 = x2; R.e3 = x3; R.t1 = xt; }
-  else { R.o0 = xo; R.s0 = x0; R.s1 = x1; R.s2 = x2; R.s3 = x3; R.t0 = xt; }
+  if (h > 0) {
+    const uint64_t cut = part * uint64_t(h);
+    R.o0 = o0 >= 0 ? o0 : slot_lower(KO, nO, cut);
+    R.s0 = n0 ? slot_lower(T.pool + T.boff[lb[0]], n0, cut) : 0;
+    R.s1 = n1 ? slot_lower(T.pool + T.boff[lb[1]], n1, cut) : 0;
+    R.s2 = n2 ? slot_lower(T.pool + T.boff[lb[2]], n2, cut) : 0;
+    R.s3 = n3 ? slot_lower(T.pool + T.boff[lb[3]], n3, cut) : 0;
+    while (R.t0 < NB && tb_pk(d, R.t0) < cut) ++R.t0;
+  }
+  if (h + 1 < P) {
+    const uint64_t cut = part * uint64_t(h + 1);
+    R.o1 = o1 >= 0 ? o1 : slot_lower(KO, nO, cut);
+    R.e0 = n0 ? slot_lower(T.pool + T.boff[lb[0]], n0, cut) : 0;
+    R.e1 = n1 ? slot_lower(T.pool + T.boff[lb[1]], n1, cut) : 0;
+    R.e2 = n2 ? slot_lower(T.pool + T.boff[lb[2]], n2, cut) : 0;
+    R.e3 = n3 ? slot_lower(T.pool + T.boff[lb[3]], n3, cut) : 0;
+    R.t1 = 0;
+    while (R.t1 < NB && tb_pk(d, R.t1) < cut) ++R.t1;
+  }
   return R;
 }
 
@@ -1302,7 +1323,9 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
   }
 
   // ---- phase 1: Step 3 candidates per bond
-  for (int lb = tid; lb < 2 * nds; lb += NT) {
+  // (the bonds, sites and parts of sites of these phases are spread evenly over
+  // the warps: a warp's loops run as long as its slowest lane's)
+  for (int lb = spread(tid, NT, 2 * nds); lb < 2 * nds; lb += NT) {
     const int li = lb >> 1, dir = lb & 1;
     const int a = T.gsite(li);
     uint64_t buf[kMaxCandPerBond];
@@ -1327,46 +1350,57 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
   if (misc->err) goto fail;
 
   // ---- phase 2: kept legs + new legs per site, merged in time order.  With
-  // two threads a site to spare (the 512-thread CTA of a 16x16 domain) each
-  // site's circle is cut at time key 2^61 and its two halves are counted and
-  // merged by two threads; each half is in time order and the halves follow
-  // one another, so the leg table is the one a single thread writes.  The
-  // half counts go through the (not yet used) worm-count bytes as scratch.
+  // P threads a site to spare (two in the 512-thread CTA of a 16x16 domain,
+  // four in a 4x4 domain's) each site's circle is cut into P parts at equal
+  // times that P threads count and merge; each part is in time order and the
+  // parts follow one another, so the leg table is the one a single thread
+  // writes.  The parts' counts and first old events go through the (not yet
+  // used) worm-count bytes.
   {
-    const bool two = NT >= 2 * nds && d.legcap >= 8 * nds;
-    const int units = two ? 2 * nds : nds;
-    int* hc = reinterpret_cast<int*>(T.wcnt);
-    for (int un = tid; un < units; un += NT) {
-      const int li = two ? un % nds : un, h = two ? un / nds : -1;
+    int P = 1;
+    while (2 * P * nds <= NT && P < 8 && d.legcap >= 16 * P * nds) P *= 2;
+    const int units = P * nds;
+    const bool scratch = P > 1 || T.early;
+    int* hc = reinterpret_cast<int*>(T.wcnt);  // [P][nds] legs of a part
+    int* ho = hc + units;                      // [P][nds] its first old event
+    for (int un = spread(tid, NT, units); un < units; un += NT) {
+      const int li = un % nds, h = un / nds;
       const int s = T.gsite(li);
       const uint64_t* KO = T.okeys_early(li, s);
       const int nO = cnt_n(d.cntA[s]);
       int lb[4];
       site_bonds(T, li, lb);
-      const MergeRange R = merge_range(T, KO, nO, lb, h);
+      const MergeRange R = merge_range(T, KO, nO, lb, h, P, -1, -1);
       int c = 0;
       for (int k = R.o0; k < R.o1; ++k) c += kept_leg<OTF>(T, li, KO[k]);
       c += (R.e0 - R.s0) + (R.e1 - R.s1) + (R.e2 - R.s2) + (R.e3 - R.s3) + (R.t1 - R.t0);
-      if (two || T.early) hc[(two ? h * nds : 0) + li] = c;
+      if (scratch) hc[un] = c;
       else T.off[li] = c;
+      if (P > 1) ho[un] = R.o0;
     }
-    if (two || T.early) {
+    if (scratch) {
       __syncthreads();
-      for (int li = tid; li < nds; li += NT) T.off[li] = hc[li] + (two ? hc[nds + li] : 0);
+      for (int li = tid; li < nds; li += NT) {
+        int c = 0;
+        for (int h = 0; h < P; ++h) c += hc[h * nds + li];
+        T.off[li] = c;
+      }
     }
     __syncthreads();
     if (block_scan(T.off, nds, wsum) > d.legcap) { if (tid == 0) tile_fail(misc, PMWA_ECAPACITY, 33); }
     __syncthreads();
     if (misc->err) goto fail;
-    for (int un = tid; un < units; un += NT) {
-      const int li = two ? un % nds : un, h = two ? un / nds : -1;
+    for (int un = spread(tid, NT, units); un < units; un += NT) {
+      const int li = un % nds, h = un / nds;
       const int s = T.gsite(li);
       const uint64_t* KO = T.okeys(li, s);
       const int nO = cnt_n(d.cntA[s]);
       int lb[4];
       site_bonds(T, li, lb);
-      const MergeRange R = merge_range(T, KO, nO, lb, h);
-      merge_site<OTF>(T, li, KO, nO, cnt_base(d.cntA[s]), lb, R, T.off[li] + (h == 1 ? hc[li] : 0));
+      int o = T.off[li];
+      for (int e = 0; e < h; ++e) o += hc[e * nds + li];
+      const MergeRange R = merge_range(T, KO, nO, lb, h, P, P > 1 ? ho[un] : -1, h + 1 < P ? ho[un + nds] : -1);
+      merge_site<OTF>(T, li, KO, nO, cnt_base(d.cntA[s]), lb, R, o);
     }
   }
   __syncthreads();
