@@ -384,6 +384,51 @@ __device__ __forceinline__ uint64_t grid_gap(uint64_t Ef, GridScale S) {
   return 1 + g;
 }
 
+// A WarpStream whose words also stand as gaps of a process of mean spacing S:
+// when a window of blocks is filled, each lane forms the gap that its two words
+// give as the first word of a draw (0: no draw of one word), so that the warp's
+// one chain takes a gap by two shuffles instead of a draw's arithmetic.
+struct WarpDraws {
+  WarpStream s;
+  GridScale S;
+  uint64_t g0, g1;
+  __device__ __forceinline__ void init(uint32_t key0, uint32_t key1, uint32_t u, uint32_t cc2, uint32_t sw,
+                                       GridScale scale) {
+    s.init(key0, key1, u, cc2, sw);
+    S = scale;
+  }
+  __device__ __forceinline__ uint64_t one(const ZigTab& z, uint64_t w) const {
+    const unsigned i = unsigned(w & 255u);
+    const uint64_t u = w >> 11, xf0 = z.XF[i];
+    if (u >= z.K[i]) return 0;
+    return grid_gap((__umul64hi(u, xf0) << 11) | ((u * xf0) >> 53), S);
+  }
+  // the window that holds the next word
+  __device__ __forceinline__ void window(const ZigTab& z) {
+    const uint64_t b = s.pos >> 1;
+    if (b - s.base < 32) return;
+    s.base = b & ~31ull;
+    s.mine = philox(uint32_t(s.base) + (threadIdx.x & 31), s.unit, s.c2, s.sweep, s.k0, s.k1);
+    g0 = one(z, uint64_t(s.mine.x) | (uint64_t(s.mine.y) << 32));
+    g1 = one(z, uint64_t(s.mine.z) | (uint64_t(s.mine.w) << 32));
+  }
+  // the gap that the next word gives (not taken)
+  __device__ __forceinline__ uint64_t gap(const ZigTab& z) {
+    window(z);
+    return __shfl_sync(0xffffffffu, (s.pos & 1) ? g1 : g0, int((s.pos >> 1) - s.base));
+  }
+  __device__ __forceinline__ uint64_t word(const ZigTab& z) {
+    window(z);
+    return s.word();
+  }
+};
+// the stream as sample_worms and zig_exp take it
+struct DrawWords {
+  WarpDraws& d;
+  const ZigTab& z;
+  __device__ __forceinline__ uint64_t word() { return d.word(z); }
+};
+
 // Eq. 1 for hard-core bosons: worms on an interval of M worm grid points with
 // parity sigma.  Rate-eta Bernoulli/Poisson process (mean spacing SW grid
 // points) conditioned on the parity of its count; for sigma = 1 and x <= 1

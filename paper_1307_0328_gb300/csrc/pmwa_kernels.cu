@@ -111,7 +111,7 @@ struct Legs {
 // and above, worms ignored; one interval round the circle if v is alone.
 // With temporal domains a leg also ends at the nearest temporal boundary,
 // whose far state is the worldline's state there.
-__device__ __noinline__ bool site_legs(const Dev& d, const uint64_t* K, int n, uint64_t pv, Legs* L) {
+__device__ __forceinline__ bool site_legs_into(const Dev& d, const uint64_t* K, int n, uint64_t pv, Legs* L) {
   const int iv = slot_find(K, n, pv);
   if (iv < 0) return false;
   int jn = iv, jp = iv, wu = 0, wd = 0;
@@ -135,6 +135,14 @@ __device__ __noinline__ bool site_legs(const Dev& d, const uint64_t* K, int n, u
   L->phi = kpk(K[jn]); L->far_up = kbl(K[jn]); L->Iup = wpts(pv, L->phi);
   L->plo = kpk(K[jp]); L->far_dn = kab(K[jp]); L->Idn = wpts(L->plo, pv);
   return true;
+}
+
+// (wup = -1: there is no event at pv)
+__device__ __noinline__ Legs site_legs(const Dev& d, const uint64_t* K, int n, uint64_t pv) {
+  Legs L;
+  L.wup = 0;
+  if (!site_legs_into(d, K, n, pv, &L)) L.wup = -1;
+  return L;
 }
 
 // Warp-cooperative list edits on a staged site list (all 32 lanes call them
@@ -177,41 +185,136 @@ __device__ __forceinline__ int warp_compact(uint64_t* K, int n, Drop drop) {
   return w;
 }
 
-// first index >= from whose key has tag `tag` (n if none)
-__device__ __forceinline__ int warp_find_tag(const uint64_t* K, int n, int from, int tag) {
+// first index >= from (a multiple of 32) whose key has tag `tag` and is at
+// least `least` (n if none)
+__device__ __forceinline__ int warp_find_tag(const uint64_t* K, int n, int from, int tag, uint64_t least) {
   const int lane = threadIdx.x & 31;
   for (int b = from; b < n; b += 32) {
     const int k = b + lane;
-    const unsigned m = __ballot_sync(0xffffffffu, k < n && ktag(K[k]) == tag);
+    const uint64_t key = k < n ? K[k] : 0;
+    const unsigned m = __ballot_sync(0xffffffffu, k < n && ktag(key) == tag && key >= least);
     if (m) return b + __ffs(int(m)) - 1;
   }
   return n;
 }
 
+// keys below `key` in the sorted list; all of the first `from` (a multiple of
+// 32) are known to be.  32 keys a step, without a bisection's chain of loads.
+__device__ __forceinline__ int warp_lower(const uint64_t* K, int n, int from, uint64_t key) {
+  const int lane = threadIdx.x & 31;
+  for (int b = from; b < n; b += 32) {
+    const unsigned m = __ballot_sync(0xffffffffu, b + lane < n && K[b + lane] < key);
+    if (m != 0xffffffffu) return b + __popc(m);
+  }
+  return n;
+}
+
+// index of the event at time point pv, looked for from `hint` on first (-1: none)
+__device__ __forceinline__ int warp_find_pk(const uint64_t* K, int n, int hint, uint64_t pv) {
+  const int lane = threadIdx.x & 31;
+  for (int turn = 0; turn < 2; ++turn) {
+    for (int b = turn ? 0 : hint & ~31; b < n; b += 32) {
+      const unsigned m = __ballot_sync(0xffffffffu, b + lane < n && kpk(K[b + lane]) == pv);
+      if (m) return b + __ffs(int(m)) - 1;
+    }
+  }
+  return -1;
+}
+
+// the legs of the vertex at index iv, as site_legs without temporal domains:
+// the lanes look at the 32 events on either side at once
+__device__ __forceinline__ void near_legs(const uint64_t* K, int n, int iv, uint64_t pv, Legs* L) {
+  const int lane = threadIdx.x & 31;
+  int jn = iv, jp = iv, wu = 0, wd = 0;
+  for (int b = 0; b < n; b += 32) {
+    int x = iv + 1 + b + lane;
+    if (x >= n) x -= n;
+    const unsigned m = __ballot_sync(0xffffffffu, b + lane < n && !kworm(K[x]));
+    if (m) {
+      wu = b + __ffs(int(m)) - 1;
+      jn = iv + 1 + wu;
+      if (jn >= n) jn -= n;
+      break;
+    }
+  }
+  for (int b = 0; b < n; b += 32) {
+    int x = iv - 1 - b - lane;
+    if (x < 0) x += n;
+    const unsigned m = __ballot_sync(0xffffffffu, b + lane < n && !kworm(K[x]));
+    if (m) {
+      wd = b + __ffs(int(m)) - 1;
+      jp = iv - 1 - wd;
+      if (jp < 0) jp += n;
+      break;
+    }
+  }
+  L->single = (jn == iv);
+  L->wup = wu;
+  L->wdn = wd;
+  if (L->single) { L->plo = L->phi = pv; L->Idn = L->Iup = kTwo59; L->far_dn = L->far_up = 0; return; }
+  const uint64_t kn = K[jn], kp = K[jp];
+  L->phi = kpk(kn); L->far_up = kbl(kn); L->Iup = wpts(pv, L->phi);
+  L->plo = kpk(kp); L->far_dn = kab(kp); L->Idn = wpts(L->plo, pv);
+}
+
 // erase the worms strictly inside (lo, hi) going up (lo == hi: all of them;
 // erase false: the caller knows there are none) and draw new ones with end
 // states p (above lo) and q (below hi); K holds n events (capacity cap).
-__device__ __noinline__ int regen_interval(const Dev& d, const ZigTab& z, WarpStream& st, uint64_t* K, int& n,
-                              uint64_t lo, uint64_t hi, int p, int q, bool erase) {
-  const uint64_t span = (hi > lo) ? hi - lo : hi + kTwo62 - lo;
-  if (erase)
+// (the stream's place and the list's count go in and out by value: a stream or
+// count whose address is taken lives in local memory)
+struct Regen {
+  uint64_t pos;
+  int n, rc;
+};
+__device__ __noinline__ Regen regen_slow(const Dev& d, ZigTab z, uint32_t unit, uint32_t c2, uint64_t pos, uint64_t* K,
+                                         int n, uint64_t lo, uint64_t hi, int p, int q) {
+  uint64_t offs[kMaxWormsPerInterval];
+  int bad = 0;
+  WarpStream st;
+  st.init(d.key0, d.key1, unit, c2, d.sweep);
+  st.pos = pos;
+  const int nw = sample_worms<kMaxWormsPerInterval>(z, st, wpts(lo, hi), p ^ q, d.SWs, d.SWI, offs, &bad);
+  if (bad) return Regen{st.pos, n, bad};
+  const uint64_t m0 = wm_above(lo);
+  for (int k = 0; k < nw; ++k) {
+    if (n >= d.cap) return Regen{st.pos, n, PMWA_ECAPACITY};
+    const uint64_t key = wkey((m0 + offs[k]) & (kTwo59 - 1), 0, p ^ 1 ^ (k & 1));
+    aslot_insert(K, n, warp_lower(K, n, 0, key & ~3ull), key);
+    ++n;
+  }
+  return Regen{st.pos, n, PMWA_OK};
+}
+
+// Two outcomes hold for most intervals and need no draw loop: a first gap
+// longer than the interval is no worm for equal end states, and one uniform
+// worm for different ones (x <= 1: the sampler's next two words, the first
+// always kept).
+__device__ __forceinline__ int regen_interval(const Dev& d, const ZigTab& z, WarpDraws& st, uint64_t* K, int& n,
+                                              uint64_t lo, uint64_t hi, int p, int q, bool erase) {
+  if (erase) {
+    const uint64_t span = (hi > lo) ? hi - lo : hi + kTwo62 - lo;
     n = warp_compact(K, n, [&](uint64_t key) {  // the worms of the interval
       if (!kworm(key)) return false;
       const uint64_t off = (kpk(key) + kTwo62 - lo) & (kTwo62 - 1);
       return off > 0 && off < span;
     });
-  uint64_t offs[kMaxWormsPerInterval];
-  int bad = 0;
-  const int nw = sample_worms<kMaxWormsPerInterval>(z, st, wpts(lo, hi), p ^ q, d.SWs, d.SWI, offs, &bad);
-  if (bad) return bad;
-  const uint64_t m0 = wm_above(lo);
-  for (int k = 0; k < nw; ++k) {
-    if (n >= d.cap) return PMWA_ECAPACITY;
-    const uint64_t key = wkey((m0 + offs[k]) & (kTwo59 - 1), 0, p ^ 1 ^ (k & 1));
-    aslot_insert(K, n, slot_lower(K, n, kpk(key)), key);
-    ++n;
   }
-  return PMWA_OK;
+  const uint64_t M = wpts(lo, hi);
+  if (M > 0 && st.gap(z) > M) {
+    if (p == q) { ++st.s.pos; return PMWA_OK; }
+    if (M <= d.SWI) {
+      st.s.pos += 2;
+      const uint64_t key = wkey((wm_above(lo) + __umul64hi(st.word(z), M)) & (kTwo59 - 1), 0, p ^ 1);
+      if (n >= d.cap) return PMWA_ECAPACITY;
+      aslot_insert(K, n, warp_lower(K, n, 0, key & ~3ull), key);
+      ++n;
+      return PMWA_OK;
+    }
+  }
+  const Regen r = regen_slow(d, z, st.s.unit, st.s.c2, st.s.pos, K, n, lo, hi, p, q);
+  st.s.pos = r.pos;
+  n = r.n;
+  return r.rc;
 }
 
 __device__ __forceinline__ double fsig(int sigma, double em1) { return sigma ? -em1 : __dadd_rn(2.0, em1); }
@@ -226,7 +329,7 @@ __device__ __forceinline__ double fsig(int sigma, double em1) { return sigma ? -
 // picks the same state.  (A state whose binary32 weight vanishes while its
 // binary64 one does not has a fraction below 2^-100 and so sits within the
 // margin of a neighbouring boundary or of 0.)  Returns that state, or -1.
-__device__ int heat_bath_f32(const Dev& d, const Legs& La, const Legs& Lb, uint64_t w, int lane) {
+__device__ __forceinline__ int heat_bath_f32(const Dev& d, const Legs& La, const Legs& Lb, uint64_t w, int lane) {
   float e4 = 0.f;
   if (lane < 4) {
     uint64_t I;
@@ -301,30 +404,40 @@ __device__ __forceinline__ bool in_win_lists(const uint64_t* KA, int nA, const u
 // staged in KA (nA events) and KB (nB events); returns a status.  With
 // d.win_half > 0 the Step-3 part is confined to the windows around the worms
 // of the two sites (on-the-fly vertex generation).
-__device__ int boundary_bond_update(const Dev& d, int a, int dir, uint64_t* KA, int& nA, int& baseA,
+__device__ __forceinline__ int boundary_bond_update(const Dev& d, int a, int dir, uint64_t* KA, int& nA, int& baseA,
                                     uint64_t* KB, int& nB, int& baseB, const ZigTab& Z) {
   const int tag = bond_tag(d, a, dir);
   const int bid = 2 * a + dir;
-  WarpStream st;
-  st.init(d.key0, d.key1, uint32_t(bid), c2_word(dir ? kBy : kBx, 0, d.replica), d.sweep);
+  WarpDraws st;
+  st.init(d.key0, d.key1, uint32_t(bid), c2_word(dir ? kBy : kBx, 0, d.replica), d.sweep, d.SWs);
   int rc = PMWA_OK;
-  // Step 2: the bond's vertices in time order (worms move, vertices do not)
-  uint64_t last = 0;
-  bool any = false;
+  // Step 2: the bond's vertices in time order (worms move, vertices do not).
+  // ia, ib: where the last one stands in the lists now, or before it (0 after
+  // a redraw round the origin, whose worms may come to stand anywhere)
+  uint64_t least = 0;
+  int ia = 0, ib = 0;
   for (;;) {
-    const int k = warp_find_tag(KA, nA, any ? slot_lower(KA, nA, last + 1) : 0, tag);
-    if (k >= nA) break;
-    const uint64_t pv = kpk(KA[k]);
-    last = pv;
-    any = true;
+    const int ka = warp_find_tag(KA, nA, ia & ~31, tag, least);
+    if (ka >= nA) break;
+    const uint64_t pv = kpk(KA[ka]);
+    least = (pv + 1) << 2;
+    const int kb = warp_find_pk(KB, nB, ib, pv);
+    if (kb < 0) return PMWA_EINVARIANT;
     Legs La, Lb;
-    if (!site_legs(d, KA, nA, pv, &La) || !site_legs(d, KB, nB, pv, &Lb)) return PMWA_EINVARIANT;
+    if (d.ntau > 1) {
+      La = site_legs(d, KA, nA, pv);
+      Lb = site_legs(d, KB, nB, pv);
+      if (La.wup < 0 || Lb.wup < 0) return PMWA_EINVARIANT;
+    } else {
+      near_legs(KA, nA, ka, pv, &La);
+      near_legs(KB, nB, kb, pv, &Lb);
+    }
     // heat-bath over the root states (Eq. 4): decided in binary32 when the
     // uniform lies clear of every boundary, else in binary64 with one lane
     // per leg factor and one lane per state and the weights summed in the
     // fixed order S = 0..15
     const int lane = threadIdx.x & 31;
-    const uint64_t wu = st.word();
+    const uint64_t wu = st.word(Z);
     int Sn = heat_bath_f32(d, La, Lb, wu, lane);
     if (Sn < 0) {
     double e4 = 0.0;
@@ -368,23 +481,35 @@ __device__ int boundary_bond_update(const Dev& d, int a, int dir, uint64_t* KA, 
     Sn = hit ? (__ffs(int(hit)) - 1) : lastS;
     }
     const int s0 = Sn & 1, s1 = (Sn >> 1) & 1, s2 = (Sn >> 2) & 1, s3 = (Sn >> 3) & 1;
-    {
-      const int ka = slot_find(KA, nA, pv), kb = slot_find(KB, nB, pv);
-      if (ka < 0 || kb < 0) return PMWA_EINVARIANT;
-      KA[ka] = (KA[ka] & ~3ull) | (uint64_t(s0) << 1) | uint64_t(s2);
-      KB[kb] = (KB[kb] & ~3ull) | (uint64_t(s1) << 1) | uint64_t(s3);
+    KA[ka] = (KA[ka] & ~3ull) | (uint64_t(s0) << 1) | uint64_t(s2);
+    KB[kb] = (KB[kb] & ~3ull) | (uint64_t(s1) << 1) | uint64_t(s3);
+    // the worms of v's four intervals anew: below on the lower and the upper
+    // site, then above (the worm counts of the legs were taken before any
+    // redraw; a redraw below v adds worms only below v, so the counts above v
+    // still hold).  One body for the four: inlined four times it takes the
+    // registers of two more warps.
+    const int nA0 = nA, nB0 = nB;
+    for (int e = 0; e < 4 && !rc; ++e) {
+      const bool onB = e & 1, above = e >= 2;
+      if (e == 2) {
+        ia = (!La.single && La.plo < pv && pv < La.phi) ? ka + nA - nA0 : 0;
+        ib = (!Lb.single && Lb.plo < pv && pv < Lb.phi) ? kb + nB - nB0 : 0;
+      }
+      const int single = onB ? Lb.single : La.single;
+      if (single && !above) continue;
+      const int bot = onB ? s1 : s0, top = onB ? s3 : s2;
+      const uint64_t far = above ? (onB ? Lb.phi : La.phi) : (onB ? Lb.plo : La.plo);
+      const uint64_t lo = above ? pv : far, hi = above ? (single ? pv : far) : pv;
+      const int p = above ? top : (onB ? Lb.far_dn : La.far_dn);
+      const int q = above ? (single ? bot : (onB ? Lb.far_up : La.far_up)) : bot;
+      const int worms = above ? (onB ? Lb.wup : La.wup) : (onB ? Lb.wdn : La.wdn);
+      int n = onB ? nB : nA;
+      rc = regen_interval(d, Z, st, onB ? KB : KA, n, lo, hi, p, q, worms > 0);
+      if (onB) nB = n; else nA = n;
     }
-    // (the worm counts of the legs were taken before any redraw; a redraw
-    // below v adds worms only below v, so the counts above v still hold)
-    if (!La.single) rc = regen_interval(d, Z, st, KA, nA, La.plo, pv, La.far_dn, s0, La.wdn > 0);
-    if (!rc && !Lb.single) rc = regen_interval(d, Z, st, KB, nB, Lb.plo, pv, Lb.far_dn, s1, Lb.wdn > 0);
-    if (!rc) rc = La.single ? regen_interval(d, Z, st, KA, nA, pv, pv, s2, s0, La.wup > 0)
-                            : regen_interval(d, Z, st, KA, nA, pv, La.phi, s2, La.far_up, La.wup > 0);
-    if (!rc) rc = Lb.single ? regen_interval(d, Z, st, KB, nB, pv, pv, s3, s1, Lb.wup > 0)
-                            : regen_interval(d, Z, st, KB, nB, pv, Lb.phi, s3, Lb.far_up, Lb.wup > 0);
     if (rc) return rc;
   }
-  if (st.pos >= (uint64_t(1) << 33)) return PMWA_ETIMEOUT;
+  if (st.s.pos >= (uint64_t(1) << 33)) return PMWA_ETIMEOUT;
   // states at the start of the circles after Step 2 (used if a list empties)
   if (nA) baseA = kab(KA[nA - 1]);
   if (nB) baseB = kab(KB[nB - 1]);
@@ -406,32 +531,40 @@ __device__ int boundary_bond_update(const Dev& d, int a, int dir, uint64_t* KA, 
     if (gone != removed) return PMWA_EINVARIANT;
   }
   if (!d.has_vertices) return PMWA_OK;
-  WarpStream sv;
-  sv.init(d.key0, d.key1, uint32_t(bid), c2_word(kVertex, 0, d.replica), d.sweep);
+  WarpDraws sv;
+  sv.init(d.key0, d.key1, uint32_t(bid), c2_word(kVertex, 0, d.replica), d.sweep, d.SVs);
   uint64_t pos = 0;
   bool first = true;
-  int bad = 0;
+  int bad = 0, xa = 0, xb = 0;  // events of the lists below the last candidate
   for (;;) {
-    const uint64_t E = zig_exp(Z, sv, &bad);
-    if (bad) return bad;
-    const uint64_t g = grid_gap(E, d.SVs);
+    uint64_t g = sv.gap(Z);
+    if (g) {
+      ++sv.s.pos;
+    } else {
+      DrawWords words{sv, Z};
+      const uint64_t E = zig_exp(Z, words, &bad);
+      if (bad) return bad;
+      g = grid_gap(E, d.SVs);
+    }
     const uint64_t nxt = first ? g - 1 : pos + g;
     first = false;
     if (nxt >= kTwo59) break;
     pos = nxt;
-    const uint64_t pk = (pos << 3) | uint64_t(tag);
+    const uint64_t pk = (pos << 3) | uint64_t(tag), key = pk << 2;
     if (otf && !in_win_lists(KA, nA, KB, nB, pos, d.win_half)) continue;
-    if (slot_find(KA, nA, pk) >= 0) continue;
-    const int na = slot_state(KA, nA, baseA, pk), nb = slot_state(KB, nB, baseB, pk);
+    xa = warp_lower(KA, nA, xa & ~31, key);
+    if (xa < nA && kpk(KA[xa]) == pk) continue;
+    xb = warp_lower(KB, nB, xb & ~31, key);
+    const int na = nA ? kab(KA[(xa ? xa : nA) - 1]) : baseA, nb = nB ? kab(KB[(xb ? xb : nB) - 1]) : baseB;
     const int si = na | (nb << 1);
     if (d.TV[si] < kTwo32) {
-      const uint64_t w = sv.word();
+      const uint64_t w = sv.word(Z);
       if ((w >> 32) >= d.TV[si]) continue;
     }
     if (nA >= d.cap || nB >= d.cap) return PMWA_ECAPACITY;
-    aslot_insert(KA, nA, slot_lower(KA, nA, pk), (pk << 2) | (uint64_t(na) << 1) | uint64_t(na));
+    aslot_insert(KA, nA, xa, key | (uint64_t(na) << 1) | uint64_t(na));
     ++nA;
-    aslot_insert(KB, nB, slot_lower(KB, nB, pk), (pk << 2) | (uint64_t(nb) << 1) | uint64_t(nb));
+    aslot_insert(KB, nB, xb, key | (uint64_t(nb) << 1) | uint64_t(nb));
     ++nB;
   }
   return PMWA_OK;
@@ -472,9 +605,19 @@ __device__ void boundary_warp(const Dev& d, int dir, int t, uint64_t* stage, con
   }
 }
 
-constexpr int kBoundaryWarps = 4;  // bonds (warps) per block
+// Bonds (warps) per block.  A bond is one chain of its vertices and their
+// lengths differ, so a block of several warps keeps its place on the SM for the
+// longest; and what bounds the kernel is the number of such chains an SM can
+// interleave (every lane runs the same scalar step, 11 cycles an instruction
+// with 7 warps a scheduler): 28 one-warp blocks an SM, 72 registers.  A launch,
+// against blocks of four warps and bisections, draws and list searches done
+// step by step: 256x256 beta t = 4 0.112 -> 0.066 ms, 512x512 beta t = 16 1.05 ->
+// 0.62 ms, 4x4 domains at V/t = 3 1.02 -> 0.52 ms; with 12 / 16 / 20 / 24 blocks
+// an SM 256x256 took 0.090 / 0.081 / 0.076 / 0.073 ms.  Likewise Step 1's sites
+// (32 blocks: 128x128 in 4 slabs 0.119 -> 0.085 ms).
+constexpr int kBoundaryWarps = 1;
 
-__global__ void __launch_bounds__(32 * kBoundaryWarps, 7) k_boundary(const __grid_constant__ Dev d, int dir) {
+__global__ void __launch_bounds__(32 * kBoundaryWarps, 28) k_boundary(const __grid_constant__ Dev d, int dir) {
   extern __shared__ __align__(16) unsigned char bsm[];
   if (instance_failed(d.err)) return;
   const ZigTab Z = zig_stage(bsm, d.zig_cap, d.worm_tries);
@@ -486,7 +629,7 @@ __global__ void __launch_bounds__(32 * kBoundaryWarps, 7) k_boundary(const __gri
 
 // Batched form: each block serves bonds t0 .. t0 + kBoundaryWarps - 1 of one
 // instance, when that instance's boundary step is due at iteration `it`.
-__global__ void __launch_bounds__(32 * kBoundaryWarps, 7) k_boundary_batch(const Dev* __restrict__ devs,
+__global__ void __launch_bounds__(32 * kBoundaryWarps, 28) k_boundary_batch(const Dev* __restrict__ devs,
                                                                         const BatchBase* __restrict__ base,
                                                                         const int2* __restrict__ work, int it,
                                                                         int dir, int cap) {
@@ -544,9 +687,9 @@ __device__ __forceinline__ void tb_delim(const Dev& d, const uint64_t* K, int n,
   *st = (leg >= 0) ? (up ? kbl(K[leg]) : kab(K[leg])) : slot_state(K, n, base, best);
 }
 
-__device__ int temporal_site(const Dev& d, int s, uint64_t* K, int& n, int& base, const ZigTab& Z) {
-  WarpStream st;
-  st.init(d.key0, d.key1, uint32_t(s), c2_word(kTemporal, 0, d.replica), d.sweep);
+__device__ __forceinline__ int temporal_site(const Dev& d, int s, uint64_t* K, int& n, int& base, const ZigTab& Z) {
+  WarpDraws st;
+  st.init(d.key0, d.key1, uint32_t(s), c2_word(kTemporal, 0, d.replica), d.sweep, d.SWs);
   for (int k = 0; k < d.ntau; ++k) {
     const uint64_t B = tb_pk(d, k);
     uint64_t lo, hi;
@@ -554,7 +697,7 @@ __device__ int temporal_site(const Dev& d, int s, uint64_t* K, int& n, int& base
     tb_delim(d, K, n, base, k, false, &lo, &p);
     tb_delim(d, K, n, base, k, true, &hi, &q);
     const uint64_t I1 = wpts(B, hi), I2 = wpts(lo, B);
-    const uint64_t wu = st.word();
+    const uint64_t wu = st.word(Z);
     // decided in binary32 when the uniform lies more than 2^-12 from the
     // fraction w0 / (w0 + w1) (two leg factors: the binary32 fraction is
     // within 2^-18 of the binary64 one), else in binary64
@@ -575,16 +718,17 @@ __device__ int temporal_site(const Dev& d, int s, uint64_t* K, int& n, int& base
       const double u = __dmul_rn(__dmul_rn(__ull2double_rn(wu >> 11), 0x1p-53), tot);
       sn = (u < w0) ? 0 : 1;
     }
-    int rc = regen_interval(d, Z, st, K, n, lo, B, p, sn, true);
-    if (!rc) rc = regen_interval(d, Z, st, K, n, B, hi, sn, q, true);
+    int rc = PMWA_OK;
+    for (int e = 0; e < 2 && !rc; ++e)
+      rc = regen_interval(d, Z, st, K, n, e ? B : lo, e ? hi : B, e ? sn : p, e ? q : sn, true);
     if (rc) return rc;
     if (n == 0) base = sn;
   }
-  if (st.pos >= (uint64_t(1) << 33)) return PMWA_ETIMEOUT;
+  if (st.s.pos >= (uint64_t(1) << 33)) return PMWA_ETIMEOUT;
   return PMWA_OK;
 }
 
-constexpr int kTemporalWarps = 4;  // sites (warps) per block
+constexpr int kTemporalWarps = 1;  // sites (warps) per block
 
 // one warp: stage site s's list (cap keys at K), update its boundaries, and
 // write it back
@@ -607,7 +751,7 @@ __device__ void temporal_warp(const Dev& d, int s, uint64_t* K, const ZigTab& Z)
   if (lane == 0) d.cntA[s] = cnt_make(n, n ? kab(K[n - 1]) : base);
 }
 
-__global__ void __launch_bounds__(32 * kTemporalWarps, 7) k_temporal(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(32 * kTemporalWarps, 32) k_temporal(const __grid_constant__ Dev d) {
   extern __shared__ __align__(16) unsigned char tsm[];
   if (instance_failed(d.err)) return;
   const ZigTab Z = zig_stage(tsm, d.zig_cap, d.worm_tries);
@@ -620,7 +764,7 @@ __global__ void __launch_bounds__(32 * kTemporalWarps, 7) k_temporal(const __gri
 // Batched form: each block serves sites t0 .. t0 + kTemporalWarps - 1 of one
 // instance, when that instance has temporal domains and its Step 1 is due at
 // iteration `it`.
-__global__ void __launch_bounds__(32 * kTemporalWarps, 7) k_temporal_batch(const Dev* __restrict__ devs,
+__global__ void __launch_bounds__(32 * kTemporalWarps, 32) k_temporal_batch(const Dev* __restrict__ devs,
                                                                         const BatchBase* __restrict__ base,
                                                                         const int2* __restrict__ work, int it,
                                                                         int cap) {
