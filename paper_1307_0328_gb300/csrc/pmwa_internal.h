@@ -141,7 +141,7 @@ int launch_temporal_batch(const Dev* devs, const BatchBase* base, const int2* wo
 int temporal_sites_per_block();
 int prepare_temporal(int cap);
 int launch_tile(const Dev& d, int stop, void* stream);
-int tile_class(const Dev& d);
+int tile_class(const Dev& d, int ctas);
 // batch launch groups: 3 CTA-size classes x residency levels by shared memory
 constexpr int kResidencyLevels = 6;
 constexpr int kBatchGroups = 4 * kResidencyLevels;

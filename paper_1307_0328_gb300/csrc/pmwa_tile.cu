@@ -43,6 +43,7 @@ constexpr int kMaxWormsPerInterval = 128;
 constexpr uint16_t kNone = 0xFFFF;
 constexpr uint32_t kCntMask = 0x7fffffffu;
 constexpr uint64_t kMask62 = kTwo62 - 1;
+constexpr int kSms = 152;
 constexpr int kSmemLimit = 232448;  // opt-in shared memory per block on sm_103a
 
 struct WormRec {
@@ -1795,18 +1796,25 @@ bool plan_tile_smem(Dev* d, double legs_want) {
 
 int upload_zig_tile(const Zig& z) { return upload_constants(z); }
 
-// CTA sizes of the sweep kernel: small domains take small CTAs, so that many
-// of them share an SM (class 0: 64 threads, 1: 128, 2: 256); a large domain
-// whose plan leaves room for one CTA per SM takes 512 threads (class 3),
-// which the registers then allow
-// (a mean of more worms than three quarters of the threads takes the next
-// class: Step 5 runs a worm a thread)
-int tile_class(const Dev& d) {
+// CTA sizes of the sweep kernel, `ctas` domains being launched together (class
+// 0: 64 threads, 1: 128, 2: 256, 3: 512).  A domain takes a thread for every
+// other bond at least (its sites), and three quarters of a thread for a worm
+// of the bound on their mean: Step 5 runs a worm a thread.  Beyond that a CTA
+// takes as many threads as cost no other CTA its place on the SM, which its
+// shared memory or the number of domains limits: the work of Step 3, Step 4 and
+// the output is then spread over more warps, and a merge cut into more parts.
+// A sweep, with the sites' classes alone and now: one 8x8 domain 127 -> 116 us,
+// 9 of 8x12 sites 251 -> 224 us, 16 of 16x16 sites 277 -> 251 us, 144 of 4x4 sites
+// 156 -> 145 us.
+int tile_class(const Dev& d, int ctas) {
   const int sites = d.dom_x * d.dom_y;
   const double worms = d.beta * d.eta * sites;
-  if (sites <= 32 && worms <= 48.0) return 0;
-  if (sites <= 96 && worms <= 96.0) return 1;
-  return (228LL * 1024) / (static_cast<long long>(d.sm_total) + 2048) <= 1 ? 3 : 2;
+  int c = sites <= 32 && worms <= 48.0 ? 0 : sites <= 96 && worms <= 96.0 ? 1 : 2;
+  // CTAs an SM has to hold (registers hold 8 >> c of class c)
+  const int by_smem = std::max(1, int((228LL * 1024) / (static_cast<long long>(d.sm_total) + 2048)));
+  const int held = std::min(by_smem, (ctas - 1) / kSms + 1);
+  while (c < 3 && (8 >> (c + 1)) >= held) ++c;
+  return c;
 }
 
 int prepare_tile_batch(int cls, int smem) {
@@ -1842,7 +1850,7 @@ static int launch_tile_k(const Dev& d, int stop, cudaStream_t st) {
 }
 
 int launch_tile(const Dev& d, int stop, void* stream) {
-  const int cls = tile_class(d);
+  const int cls = tile_class(d, d.ndom);
   const cudaStream_t st = cudaStream_t(stream);
   const bool otf = d.win_half > 0;
   switch (cls) {
