@@ -1,6 +1,6 @@
 """Checkpoints that are packed and checked on the device: the same bytes as
 the oracle's, the same statuses as a check in buffer order, and slots too full
-for the packed form (which then take the host's)."""
+or too few for the packed form (which then take the host's)."""
 import numpy as np
 import pytest
 
@@ -13,13 +13,14 @@ from oracle import oracle as O  # noqa: E402
 import paper_1307_0328_gb300 as P  # noqa: E402
 
 
+@pytest.mark.parametrize("cap_site", [0, 2048])  # (8x8 and up: 2048 slots a site take the packed form)
 @pytest.mark.parametrize("kw", [
     dict(Lx=2, Ly=2, beta=1.5, eta=0.5, n_cycle=4, seed=3, init=0),
     dict(Lx=19, Ly=17, beta=2.0, eta=0.3, V=0.5, mu=0.4, n_cycle=4, seed=29),
     dict(Lx=8, Ly=8, beta=4.0, eta=0.2, n_cycle=4, seed=1),
 ])
-def test_export_and_import(kw):
-    g, o = P.Sim(**kw), O.Oracle(**kw)
+def test_export_and_import(kw, cap_site):
+    g, o = P.Sim(**dict(kw, cap_site=cap_site)), O.Oracle(**kw)
     assert np.array_equal(g.export(), o.export())  # no events yet
     o.sweep(6)
     snap = o.export()
@@ -41,11 +42,12 @@ def test_export_and_import(kw):
         assert e.value.status == P.PMWA_ECAPACITY
 
 
-def test_first_wrong_site_names_the_status():
+@pytest.mark.parametrize("cap_site", [0, 2048])
+def test_first_wrong_site_names_the_status(cap_site):
     """An invariant broken at an earlier site comes before a header that is
     wrong at a later one, and after one that is wrong earlier."""
     kw = dict(Lx=8, Ly=8, beta=2.0, eta=0.3, n_cycle=4, seed=5)
-    g, o = P.Sim(**kw), O.Oracle(**kw)
+    g, o = P.Sim(**dict(kw, cap_site=cap_site)), O.Oracle(**kw)
     o.sweep(6)
     snap = o.export()
     heads, k = [], 1
