@@ -30,9 +30,10 @@ def _divisors(L):
 
 
 def _threads(sites, smem=None):
-    """Threads of the sweep kernel's CTA for a domain plan, as the library
-    picks them: 64, 128 or 256 by the domain's sites, 512 for a large domain
-    whose plan leaves room for one CTA per SM."""
+    """Threads of the sweep kernel's CTA that a domain plan is ranked by: 64,
+    128 or 256 by the domain's sites, 512 for a large domain whose plan leaves
+    room for one CTA per SM.  (The least that the library launches: a CTA takes
+    more where that costs no CTA its place on the SM.)"""
     if sites <= 32:
         return 64
     if sites <= 96:

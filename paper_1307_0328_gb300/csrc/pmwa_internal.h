@@ -142,7 +142,7 @@ int temporal_sites_per_block();
 int prepare_temporal(int cap);
 int launch_tile(const Dev& d, int stop, void* stream);
 int tile_class(const Dev& d, int ctas);
-// batch launch groups: 3 CTA-size classes x residency levels by shared memory
+// batch launch groups: CTA-size classes x residency levels by shared memory
 constexpr int kResidencyLevels = 6;
 constexpr int kBatchGroups = 4 * kResidencyLevels;
 int launch_tile_batch(int cls, const Dev* devs, const BatchBase* base, const int2* work, int n_work, int smem,

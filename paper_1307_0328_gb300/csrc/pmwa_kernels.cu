@@ -3,7 +3,10 @@
 //   k_boundary   Step 2 (Eq. 4) + Step 3 on the bonds between domains;
 //                one warp per boundary bond, x bonds then y bonds, in
 //                place on the current configuration.
-//   k_rho        Supplement S-I worm density at equal-time slices.
+//   k_temporal   Step 1 (Eq. 3), one warp per site.
+//   k_rho        Supplement S-I worm density at equal-time slices, k_green
+//                its equal-time sums, k_npoint products on listed sites.
+//   k_pack, k_packed_check, k_unpack   checkpoints.
 //   k_check      invariants of the current configuration, one warp per site.
 // Steps 3-6 of every other bond and site run in k_tile (pmwa_tile.cu).
 //

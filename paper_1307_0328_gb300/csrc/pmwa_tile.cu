@@ -2,13 +2,15 @@
 // domain, the domain's vertex legs and worms resident in shared memory.
 //
 //   phase 1  Step 3 candidates, one thread per bond of the domain, written to
-//            a shared pool (the current configuration is read from HBM/L2,
-//            prefetched into L2 by bulk copies at kernel start)
-//   phase 2  per site: the kept vertex legs of the current configuration
-//            merged in time order with the new ones into the shared leg array
-//   phase 3  Step 4, one thread per site: worms of every interval (Eq. 1)
-//            into the shared worm table; each worm records its site and the
-//            index of the vertex leg just below it (its interval)
+//            a shared pool (the current configuration is read from a staged
+//            copy in shared memory where it fits, else from HBM/L2, prefetched
+//            into L2 by bulk copies at kernel start)
+//   phase 2  per site, or per part of a site's circle: the kept vertex legs of
+//            the current configuration merged in time order with the new ones
+//            into the shared leg array
+//   phase 3  Step 4, one thread per site, a random word a step: worms of every
+//            interval (Eq. 1) into the shared worm table; each worm records its
+//            site and the index of the vertex leg just below it (its interval)
 //   phase 4  Step 5, N_cycle passes of the shifted sub-block schedule: the
 //            worms of a sub-block move in label order (Eq. 2); a move waits
 //            only for the earlier ones whose intervals meet its own, which
@@ -22,8 +24,8 @@
 //            still move.  One 16x16-site domain, cycles a pass: 10.1k -> 6.4k
 //            at beta t = 4 (95 worms), 19.6k -> 10.9k at beta t = 16 (381
 //            worms); an 8x8 domain of one group (22 worms): 19.0k -> 5.4k
-//   phase 5  legs and worms merged per site into the next configuration in
-//            HBM, with the Step-6 counters and the Supplement S-I estimator
+//   phase 5  legs and worms, each at its counted place, into the next
+//            configuration in HBM, with the Step-6 counters and the Supplement S-I estimator
 //
 // The arithmetic and the order of every random draw are those of the
 // deterministic specification, so the result is bit-identical to the CPU
