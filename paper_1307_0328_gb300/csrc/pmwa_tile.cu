@@ -1354,7 +1354,7 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
 
   // ---- phase 2: kept legs + new legs per site, merged in time order.  With
   // P threads a site to spare (two in the 512-thread CTA of a 16x16 domain,
-  // four in a 4x4 domain's) each site's circle is cut into P parts at equal
+  // eight in a 4x4 domain's of 128) each site's circle is cut into P parts at equal
   // times that P threads count and merge; each part is in time order and the
   // parts follow one another, so the leg table is the one a single thread
   // writes.  The parts' counts and first old events go through the (not yet
