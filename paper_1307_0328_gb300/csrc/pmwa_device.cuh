@@ -70,6 +70,15 @@ __device__ __forceinline__ P4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint
   return P4{c0, c1, c2, c3};
 }
 
+// The same inside a loop with keys that the loop does not change: hidden from
+// the compiler, which forms the ten rounds' keys before the loop and holds them
+// in 18 registers, and spills others for them.
+__device__ __forceinline__ P4 philox_in_loop(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
+                                             uint32_t k0, uint32_t k1) {
+  asm volatile("" : "+r"(k0), "+r"(k1));
+  return philox(c0, c1, c2, c3, k0, k1);
+}
+
 // Sequence of 64-bit words of the blocks with counter (block, unit, c2, sweep):
 // word w is the low (w even) or high (w odd) half of block w/2.
 struct Stream {
@@ -107,7 +116,7 @@ struct WarpStream {
     const uint64_t b = pos >> 1;
     if (b - base >= 32) {
       base = b & ~31ull;
-      mine = philox(uint32_t(base) + (threadIdx.x & 31), unit, c2, sweep, k0, k1);
+      mine = philox_in_loop(uint32_t(base) + (threadIdx.x & 31), unit, c2, sweep, k0, k1);
     }
     const int src = int(b - base);
     const bool odd = pos & 1;
@@ -408,7 +417,7 @@ struct WarpDraws {
     const uint64_t b = s.pos >> 1;
     if (b - s.base < 32) return;
     s.base = b & ~31ull;
-    s.mine = philox(uint32_t(s.base) + (threadIdx.x & 31), s.unit, s.c2, s.sweep, s.k0, s.k1);
+    s.mine = philox_in_loop(uint32_t(s.base) + (threadIdx.x & 31), s.unit, s.c2, s.sweep, s.k0, s.k1);
     g0 = one(z, uint64_t(s.mine.x) | (uint64_t(s.mine.y) << 32));
     g1 = one(z, uint64_t(s.mine.z) | (uint64_t(s.mine.w) << 32));
   }

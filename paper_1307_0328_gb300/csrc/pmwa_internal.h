@@ -104,9 +104,9 @@ struct BatchBase {
   int active;
 };
 
-// An instance's parameters advanced to sweep iteration `it` of a batched call
-__host__ __device__ inline Dev at_iteration(const Dev& d0, const BatchBase& b, int it) {
-  Dev d = d0;
+// An instance's parameters d0 advanced to sweep iteration `it` of a batched
+// call (set_iteration: in d, a copy of d0)
+__host__ __device__ inline void set_iteration(Dev& d, const Dev& d0, const BatchBase& b, int it) {
   const int cur = (b.flip + it) & 1;
   d.keyA = d0.bufk[cur];
   d.cntA = d0.bufc[cur];
@@ -114,6 +114,10 @@ __host__ __device__ inline Dev at_iteration(const Dev& d0, const BatchBase& b, i
   d.cntB = d0.bufc[cur ^ 1];
   d.sweep = b.sweep0 + uint32_t(it);
   d.row = b.row0 + it;
+}
+__host__ __device__ inline Dev at_iteration(const Dev& d0, const BatchBase& b, int it) {
+  Dev d = d0;
+  set_iteration(d, d0, b, it);
   return d;
 }
 

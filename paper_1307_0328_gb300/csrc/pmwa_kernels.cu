@@ -30,6 +30,18 @@ __device__ __forceinline__ int cnt_n(uint32_t c) { return int(c & kCntMask); }
 __device__ __forceinline__ int cnt_base(uint32_t c) { return int(c >> 31); }
 __device__ __forceinline__ uint32_t cnt_make(int n, int base) { return uint32_t(n) | (uint32_t(base) << 31); }
 
+// An instance's record advanced to sweep iteration `it` of a batched call, in
+// shared memory (all threads; the caller synchronises): at_iteration, copied a
+// word a thread.
+__device__ __forceinline__ void stage_record(Dev* sd, const Dev* g, const BatchBase& bb, int it) {
+  static_assert(sizeof(Dev) % 8 == 0, "copied by words");
+  const uint64_t* from = reinterpret_cast<const uint64_t*>(g);
+  uint64_t* to = reinterpret_cast<uint64_t*>(sd);
+  for (int k = threadIdx.x; k < int(sizeof(Dev) / 8); k += blockDim.x) to[k] = from[k];
+  __syncthreads();
+  if (threadIdx.x == 0) set_iteration(*sd, *g, bb, it);
+}
+
 // Supplement S-I worm density at K equal-time slices tau_k = k beta / K:
 // eta g_sigma(x) of the interval between vertex legs holding tau_k.  2^sh
 // threads a site (slice_lanes: the power of two from K up to a warp), one a
@@ -263,19 +275,17 @@ __device__ __forceinline__ void near_legs(const uint64_t* K, int n, int iv, uint
 // erase the worms strictly inside (lo, hi) going up (lo == hi: all of them;
 // erase false: the caller knows there are none) and draw new ones with end
 // states p (above lo) and q (below hi); K holds n events (capacity cap).
-// (the stream's place and the list's count go in and out by value: a stream or
-// count whose address is taken lives in local memory)
+// (the stream -- with the window of blocks that the lanes hold, so that it is not
+// drawn again -- and the list's count go in and out by value: a stream or count
+// whose address is taken lives in local memory)
 struct Regen {
   uint64_t pos;
   int n, rc;
 };
-__device__ __noinline__ Regen regen_slow(const Dev& d, ZigTab z, uint32_t unit, uint32_t c2, uint64_t pos, uint64_t* K,
-                                         int n, uint64_t lo, uint64_t hi, int p, int q) {
+__device__ __noinline__ Regen regen_slow(const Dev& d, ZigTab z, WarpStream st, uint64_t* K, int n, uint64_t lo,
+                                         uint64_t hi, int p, int q) {
   uint64_t offs[kMaxWormsPerInterval];
   int bad = 0;
-  WarpStream st;
-  st.init(d.key0, d.key1, unit, c2, d.sweep);
-  st.pos = pos;
   const int nw = sample_worms<kMaxWormsPerInterval>(z, st, wpts(lo, hi), p ^ q, d.SWs, d.SWI, offs, &bad);
   if (bad) return Regen{st.pos, n, bad};
   const uint64_t m0 = wm_above(lo);
@@ -314,7 +324,7 @@ __device__ __forceinline__ int regen_interval(const Dev& d, const ZigTab& z, War
       return PMWA_OK;
     }
   }
-  const Regen r = regen_slow(d, z, st.s.unit, st.s.c2, st.s.pos, K, n, lo, hi, p, q);
+  const Regen r = regen_slow(d, z, st.s, K, n, lo, hi, p, q);
   st.s.pos = r.pos;
   n = r.n;
   return r.rc;
@@ -618,7 +628,19 @@ __device__ void boundary_warp(const Dev& d, int dir, int t, uint64_t* stage, con
 // 0.62 ms, 4x4 domains at V/t = 3 1.02 -> 0.52 ms; with 12 / 16 / 20 / 24 blocks
 // an SM 256x256 took 0.090 / 0.081 / 0.076 / 0.073 ms.  Likewise Step 1's sites
 // (32 blocks: 128x128 in 4 slabs 0.119 -> 0.085 ms).
-constexpr int kBoundaryWarps = 1;
+//
+// Registers, spill stores and loads (bytes): k_boundary 72, 24 and 24,
+// k_temporal 56 without spills.  The batched forms have the instance's record
+// in shared memory instead of the constant bank and its fields in registers; a
+// spill is costly, as beside 200 KB of shared memory the L1 has no room for
+// the blocks' local memory.  They take 20 (96 registers, 244 and 176) and 24 blocks
+// (80, 76 and 128): at 28 and 32, where the spills are 612 / 460 and 360 / 276, most
+// replica sets were slower, at 16 those of long lists.  Against 28 and 32 blocks
+// with the round keys kept in registers and the record copied by one lane
+// (684 / 940 and 372 / 352), 400 replicas of 32x32 sites: 8x8 domains at beta t
+// = 4, eta = 0.2 0.597 -> 0.483 ms a launch (blocks of four warps: 0.504), four
+// slabs at beta t = 8 1.78 -> 1.36 ms of Step 1 (1.62).
+constexpr int kBoundaryWarps = 1, kBatchBlocks = 20;
 
 __global__ void __launch_bounds__(32 * kBoundaryWarps, 28) k_boundary(const __grid_constant__ Dev d, int dir) {
   extern __shared__ __align__(16) unsigned char bsm[];
@@ -632,7 +654,7 @@ __global__ void __launch_bounds__(32 * kBoundaryWarps, 28) k_boundary(const __gr
 
 // Batched form: each block serves bonds t0 .. t0 + kBoundaryWarps - 1 of one
 // instance, when that instance's boundary step is due at iteration `it`.
-__global__ void __launch_bounds__(32 * kBoundaryWarps, 28) k_boundary_batch(const Dev* __restrict__ devs,
+__global__ void __launch_bounds__(32 * kBoundaryWarps, kBatchBlocks) k_boundary_batch(const Dev* __restrict__ devs,
                                                                         const BatchBase* __restrict__ base,
                                                                         const int2* __restrict__ work, int it,
                                                                         int dir, int cap) {
@@ -641,7 +663,7 @@ __global__ void __launch_bounds__(32 * kBoundaryWarps, 28) k_boundary_batch(cons
   const int2 w = work[blockIdx.x];
   const BatchBase bb = base[w.x];
   if (!bb.active) return;
-  if (threadIdx.x == 0) sd = at_iteration(devs[w.x], bb, it);
+  stage_record(&sd, devs + w.x, bb, it);
   ZigTab Z = zig_stage(bsm);
   __syncthreads();
   Z.zcap = sd.zig_cap;
@@ -731,7 +753,7 @@ __device__ __forceinline__ int temporal_site(const Dev& d, int s, uint64_t* K, i
   return PMWA_OK;
 }
 
-constexpr int kTemporalWarps = 1;  // sites (warps) per block
+constexpr int kTemporalWarps = 1, kBatchSiteBlocks = 24;  // sites (warps) per block; blocks an SM
 
 // one warp: stage site s's list (cap keys at K), update its boundaries, and
 // write it back
@@ -767,7 +789,7 @@ __global__ void __launch_bounds__(32 * kTemporalWarps, 32) k_temporal(const __gr
 // Batched form: each block serves sites t0 .. t0 + kTemporalWarps - 1 of one
 // instance, when that instance has temporal domains and its Step 1 is due at
 // iteration `it`.
-__global__ void __launch_bounds__(32 * kTemporalWarps, 32) k_temporal_batch(const Dev* __restrict__ devs,
+__global__ void __launch_bounds__(32 * kTemporalWarps, kBatchSiteBlocks) k_temporal_batch(const Dev* __restrict__ devs,
                                                                         const BatchBase* __restrict__ base,
                                                                         const int2* __restrict__ work, int it,
                                                                         int cap) {
@@ -776,7 +798,7 @@ __global__ void __launch_bounds__(32 * kTemporalWarps, 32) k_temporal_batch(cons
   const int2 w = work[blockIdx.x];
   const BatchBase bb = base[w.x];
   if (!bb.active) return;
-  if (threadIdx.x == 0) sd = at_iteration(devs[w.x], bb, it);
+  stage_record(&sd, devs + w.x, bb, it);
   ZigTab Z = zig_stage(tsm);
   __syncthreads();
   Z.zcap = sd.zig_cap;
