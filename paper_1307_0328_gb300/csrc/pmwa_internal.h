@@ -51,6 +51,7 @@ struct Dev {
   int sm_part;          // [legcap] u16: index of each vertex leg's partner leg (Step 5)
   int use_part;         // 1: the partner table is planned; 0: Step 5 searches for partners
   int gtab;             // 1: Step 5 holds tables of its groups' members; 0: lists only
+  int gslots;           // members a table holds (a multiple of 4)
   int ghash;            // heads of Step 5's chains of worms by leg (a power of two; 0: none)
   int oldcap;           // events it can hold; 0 = read the configuration from HBM
   unsigned long long* phase_cycles;  // 8 counters when profiling, else null

@@ -350,8 +350,45 @@ __device__ __forceinline__ int look_ahead(const Tile& T, uint64_t key, int li, i
   return PMWA_OK;
 }
 
-// The Step-5 move of a worm (key, site li, interval L; updated here) to the
-// vertex v of `o`.  each(f) calls f(leg, key) for (at least) every other
+// What a Step-5 move decides and the exact lengths of v's legs (own site down,
+// other site down, own up, other up), in full words, for a move whose 32-bit
+// lengths leave a doubt: worm k at (key, interval L), nw worms.  Only worms of v's
+// four intervals count, and the interval's leg names them, so all of the domain's
+// are looked at.  Out of line, as it is rare and a move's code long.
+struct Exact {
+  bool blocked, enter;
+  uint64_t E0, E1, E2, E3;
+};
+__device__ __noinline__ Exact exact_lengths(const uint64_t* leg, const WormRec* W, int k, int nw, uint32_t fp,
+                                            uint32_t dns, uint32_t ups, uint64_t kv, uint64_t key, int L,
+                                            uint32_t z1) {
+  const int iv = int(fp & 0xffff), ip = int(fp >> 16), i_dn = int(dns & 0xffff), p_dn = int(dns >> 16);
+  const bool up = kdir(key);
+  const uint64_t pv = kpk(kv), my = up ? (pv - kpk(key)) & kMask62 : (kpk(key) - pv) & kMask62;
+  Exact x;
+  x.E0 = wpts(kpk(leg[i_dn]), pv);
+  x.E1 = wpts(kpk(leg[p_dn]), pv);
+  x.E2 = wpts(pv, kpk(leg[ups & 0xffff]));
+  x.E3 = wpts(pv, kpk(leg[ups >> 16]));
+  x.blocked = false;
+  for (int e = 0; e < nw; ++e) {
+    if (e == k) continue;
+    const int lg = W[e].leg;
+    const uint64_t po = kpk(W[e].key);
+    if (lg == L && (up ? ((pv - po) & kMask62) < my : ((po - pv) & kMask62) < my)) x.blocked = true;
+    if (lg == iv) x.E2 = min(x.E2, wpts(pv, po));
+    if (lg == ip) x.E3 = min(x.E3, wpts(pv, po));
+    if (lg == i_dn) x.E0 = min(x.E0, wpts(po, pv));
+    if (lg == p_dn) x.E1 = min(x.E1, wpts(po, pv));
+  }
+  // enter iff z1 * L_i < L_min * 2^32 (96-bit comparison)
+  const uint64_t Li = up ? x.E0 : x.E2, lo = uint64_t(z1) * (Li & 0xffffffffull);
+  x.enter = uint64_t(z1) * (Li >> 32) + (lo >> 32) < min(min(x.E0, x.E1), min(x.E2, x.E3));
+  return x;
+}
+
+// The Step-5 move of worm k of nw (key, site li, interval L; updated here) to
+// the vertex v of `o`.  each(f) calls f(leg, key) for (at least) every other
 // worm in v's four intervals; it is used only when there is one.  The worm
 // reverses at another worm ahead of it in its interval; otherwise it enters v
 // with probability L_min / L_i (w0 >> 32 against the exact ratio), leaves by
@@ -369,7 +406,7 @@ __device__ __forceinline__ int look_ahead(const Tile& T, uint64_t key, int li, i
 // branches are the rare cases only, the loads stand together up front.
 template <class Each>
 __device__ __forceinline__ void make_move(const Tile& T, const Ahead& o, uint64_t& key, int& li, int& L, uint64_t w0,
-                                          uint64_t w1, Each each) {
+                                          uint64_t w1, int k, int nw, Each each) {
   const int iv = int(o.fp & 0xffff), ip = int(o.fp >> 16), i_dn = int(o.dns & 0xffff), p_dn = int(o.dns >> 16);
   const uint64_t vi = T.leg[iv], vp = T.leg[ip];
   const int c0 = T.wcnt[i_dn], c1 = T.wcnt[p_dn], c2 = T.wcnt[iv], c3 = T.wcnt[ip];
@@ -420,23 +457,10 @@ __device__ __forceinline__ void make_move(const Tile& T, const Ahead& o, uint64_
   uint64_t Lj = (dj >> 5) - (ju ? 0 : wj);
   if (dn == x && !wj) Lj = kTwo59;
   if (doubt) {
-    const uint64_t pv = kpk(o.kv), my = up ? (pv - kpk(key)) & kMask62 : (kpk(key) - pv) & kMask62;
-    uint64_t E0 = wpts(kpk(T.leg[i_dn]), pv), E1 = wpts(kpk(T.leg[p_dn]), pv);
-    uint64_t E2 = wpts(pv, kpk(T.leg[o.ups & 0xffff])), E3 = wpts(pv, kpk(T.leg[o.ups >> 16]));
-    blocked = false;
-    if (others)
-      each([&](int lg, uint64_t ko) {
-        const uint64_t po = kpk(ko);
-        if (lg == L && (up ? ((pv - po) & kMask62) < my : ((po - pv) & kMask62) < my)) blocked = true;
-        if (lg == iv) E2 = min(E2, wpts(pv, po));
-        if (lg == ip) E3 = min(E3, wpts(pv, po));
-        if (lg == i_dn) E0 = min(E0, wpts(po, pv));
-        if (lg == p_dn) E1 = min(E1, wpts(po, pv));
-      });
-    // enter iff z1 * L_i < L_min * 2^32 (96-bit comparison)
-    const uint64_t Li = up ? E0 : E2, lo = uint64_t(z1) * (Li & 0xffffffffull);
-    enter = uint64_t(z1) * (Li >> 32) + (lo >> 32) < min(min(E0, E1), min(E2, E3));
-    Lj = jo ? (ju ? E2 : E0) : (ju ? E3 : E1);
+    const Exact x = exact_lengths(T.leg, T.W, k, others ? nw : 0, o.fp, o.dns, o.ups, o.kv, key, L, z1);
+    blocked = x.blocked;
+    enter = x.enter;
+    Lj = jo ? (ju ? x.E2 : x.E0) : (ju ? x.E3 : x.E1);
   }
   const uint64_t at = __umul64hi(w1, Lj);
   // the worm leaves leg i and takes leg j: flip their states
@@ -567,35 +591,63 @@ __device__ __forceinline__ void store_place(WormRec& w, int li, int L) {
 }
 
 constexpr int kSpinLimit = 1 << 20;  // polls of a predecessor before the pass gives up (never reached)
-constexpr int kGroupSlots = 8;       // worms of a group's table (16 bits each)
+constexpr int kNeighbours = 64;      // neighbours that a worm holds one by one
+constexpr int kGroupSlots = 8;       // worms of a group's table (16 bits each) at least
+// up to so many groups, of more worms on average: scans and chains by leg
+constexpr int kScanGroups = 9, kScanMembers = 12;
+// worms of a thread at most: a plan of 227 KB and 48 bytes a worm holds 4842,
+// 19 for each of 256 threads, and smaller CTAs run domains of fewer worms
+// (tile_class: the table of 48 expected worms holds 286, that of 384 825)
+constexpr int kMaxTurns = 24;
 
-// All N_cycle passes of a domain whose 32 < nw <= blockDim.x worms have a
-// thread each (called by all threads); W[] is in label order and a thread
-// keeps its worm k in registers throughout.  The worms are spread over the
+// All N_cycle passes of a domain of more than 32 worms (called by all
+// threads); W[] is in label order.  With at most blockDim.x worms a thread
+// keeps its worm k in registers throughout, and the worms are spread over the
 // warps, at least 16 a warp: a warp's loops run as long as its slowest lane's,
 // but more warps issue more instructions.
 //
+// With more a thread takes its worms k = tid, tid + blockDim.x, ... in
+// turns within each pass and looks ahead anew at a turn's start.  A worm waits
+// for smaller k alone, which belong to its own turn or an earlier one of other
+// warps, and an earlier turn waits for no later one: every wait ends.
+//
 // A pass has one barrier.  Behind it every worm goes through its group once,
 // for its rank r (the members with a smaller k) and for the members whose
-// intervals meet its own (nn of them, the first four in `mem`, 16 bits each),
+// intervals meet its own (nn of them, four in `mem`, 16 bits each),
 // draws its Philox block and moves as soon as the earlier ones of those (bits
 // of `deps`) have set their flag dn[] -- no round waits for the slowest worm
 // of the domain.  What it reaches in the next pass depends on its own place
 // and on leg times alone, so it looks ahead and joins its next group right
 // after its move, while other worms still move.
 //
-// A worm with more than four such neighbours goes through the members again
-// at each use.  In a domain with few large groups (sub_block 0: one) going
-// through a group costs more than the moves; there the worms enter their
-// vertex's two legs (one that turns: its interval) in a hash table of chains,
-// entry 2 k + side with its successors in W[k].lab, and a worm looks up the
-// six legs whose owners' intervals can meet its own.  Its rank is k with one
-// group, else counted over the group numbers in nxt[].
+// The members of up to kNeighbours neighbours beyond four are listed by the
+// thread itself (local memory, in a second round through the group); a worm with
+// more looks at every worm of the domain.  Walking the group anew at each poll
+// and in the move, and a form for more worms than threads that looked ahead anew
+// every round, had made domains of many worms an interval up to 4.0 times
+// slower than rounds of precomputed waits (8x8 sites at beta t = 2, eta = 3,
+// now 1.8 times as fast as those; 24x24 at beta t = 4, eta = 0.5 in 4x4 blocks
+// 2.14 -> 5.02 -> 0.91 ms a sweep).
+//
+// The groups' tables hold the expected members and three standard deviations
+// where the plan has room.  In a domain of few large groups (sub_block 0: one)
+// going through a group costs more than the moves; there (kScanGroups,
+// kScanMembers: at more groups, lists of tens of members were the faster by up
+// to 4) the worms enter their vertex's two legs (one that turns: its interval)
+// in a hash table of chains, entry 2 k + side with its successors in W[k].lab,
+// and a worm looks up the six legs whose owners' intervals can meet its own.
+// Its rank is k with one group, else counted over the group numbers in nxt[].
+template <bool kSeveral>
 __device__ void block_passes(const Tile& T, int dom, int nw, long long& tclk) {
   const Dev& d = *T.d;
-  const int nwarps = int(blockDim.x) >> 5, per = max(16, (nw + nwarps - 1) / nwarps), lane = threadIdx.x & 31;
-  const int k = (int(threadIdx.x) >> 5) * per + lane;
-  const bool act = lane < per && k < nw, scan = nw > 12 * T.ngrp, table = d.gtab && !scan, hash = scan && d.ghash;
+  const int NT = int(blockDim.x), nwarps = NT >> 5, lane = threadIdx.x & 31;
+  const int per = kSeveral ? 32 : max(16, (nw + nwarps - 1) / nwarps);
+  const int first = (int(threadIdx.x) >> 5) * per + lane;
+  const int slots = d.gslots;
+  const bool scan = T.ngrp <= kScanGroups && nw > kScanMembers * T.ngrp;
+  const bool table = d.gtab && !scan, hash = scan && d.ghash;
+  int k = first;
+  bool act = lane < per && k < nw;
   uint64_t key = 0;
   int li = 0, L = 0, slab = 0, u = 0, u_old = 0;
   Ahead o;
@@ -605,7 +657,7 @@ __device__ void block_passes(const Tile& T, int dom, int nw, long long& tclk) {
   auto fail = [&](int pass, int rc) { T.perr[pass & 1] = rc; };
   auto prepare = [&](int pass, int b3) {
     u = worm_group(T, li, slab, pass & 3);
-    const int at = table ? atomicAdd(T.gcnt + b3 * T.ngrp + u, 1) : kGroupSlots;
+    const int at = table ? atomicAdd(T.gcnt + b3 * T.ngrp + u, 1) : slots;
     const int rc = look_ahead(T, key, li, L, pass & 3, o);
     if (rc) fail(pass, rc);
     T.fp[(pass & 1) * d.wcap + k] = o.fp;
@@ -619,19 +671,24 @@ __device__ void block_passes(const Tile& T, int dom, int nw, long long& tclk) {
         next[e] = (was >> 16) == stamp ? uint16_t(was) : kNone;
       }
     }
-    if (at < kGroupSlots) T.cell[((pass & 1) * T.ngrp + u) * kGroupSlots + at] = uint16_t(k);
+    if (at < slots) T.cell[((pass & 1) * T.ngrp + u) * slots + at] = uint16_t(k);
     else if (scan) T.nxt[(pass & 1) * d.wcap + k] = uint16_t(u);
     else join_list(T, k, u, pass);
   };
-  if (act) {
+  auto load = [&] {
     const WormRec& w = T.W[k];
     key = w.key;
     li = w.site;
     L = w.leg;
     slab = w.slab;
+  };
+  for (; k < nw && lane < per; k += NT) {
+    load();
     prepare(0, 0);
+    if (!kSeveral) break;
   }
   volatile uint16_t* dn = T.dn;
+  uint16_t more[kNeighbours];
   int b3 = 0;  // pass % 3
   for (int pass = 0; pass < d.n_cycle; ++pass) {
     __syncthreads();
@@ -642,206 +699,163 @@ __device__ void block_passes(const Tile& T, int dom, int nw, long long& tclk) {
     const int stamp = pass + 1;
     const uint32_t* fp = T.fp + (pass & 1) * d.wcap;
     const uint16_t* nxt = T.nxt + (pass & 1) * d.wcap;
-    const uint16_t* cell = T.cell + ((pass & 1) * T.ngrp + u) * kGroupSlots;
-    const Meet meet(o);
-    bool moved = !act;
-    int r = 0, nn = 0, n = 0;  // n: members in the table
-    bool list = false;         // some members are in the list
-    uint32_t deps = 0;
-    uint64_t mem = 0, w0 = 0, w1 = 0;
     const int b3n = b3 == 2 ? 0 : b3 + 1, b3p = b3 == 0 ? 2 : b3 - 1;
-    if (act && turns(o.fp)) {
-      key ^= 2u;
-      moved = true;
-    }
-    auto look_at = [&](int j, uint32_t g) {
-      const bool m = meet(g) && j != k;
-      r += j < k ? 1 : 0;
-      nn += m ? 1 : 0;
-      mem = m ? (mem << 16) | uint64_t(j) : mem;
-      deps = m ? (deps << 1) | (j < k && !turns(g) ? 1u : 0u) : deps;
-    };
-    // every member again, for a worm with more than four neighbours
-    auto again = [&](auto f) {
-      if (scan) {
-        for (int j = 0; j < nw; ++j)
-          if (nxt[j] == u) f(j);
-      }
-      for (int e = 0; e < n; ++e) f(int(cell[e]));
-      if (list)
-        for (int j = int(T.hd[(pass & 1) * T.hstride + u] & 0xffff); j != kNone; j = nxt[j]) f(j);
-    };
-    if (!moved) {
-      if (table) {
-        const int c = T.gcnt[b3 * T.ngrp + u];
-        n = min(c, kGroupSlots);
-        list = c > kGroupSlots;
-      } else {
-        list = !scan;
-      }
-      for (int e0 = 0; e0 < n; e0 += 4) {
-        const uint2 four = *reinterpret_cast<const uint2*>(cell + e0);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int j = int(((e < 2 ? four.x : four.y) >> (16 * (e & 1))) & 0xffff);
-          if (e0 + e < n) look_at(j, fp[j]);
+    if (kSeveral && table)
+      for (int i = threadIdx.x; i < T.ngrp; i += NT) T.gcnt[b3p * T.ngrp + i] = 0;
+    for (int t0 = 0; t0 < (kSeveral ? nw : 1); t0 += NT) {
+      if (kSeveral) {
+        k = t0 + first;
+        act = k < nw;
+        o.fp = kTurn;
+        if (act) {
+          load();
+          u = worm_group(T, li, slab, pass & 3);
+          look_ahead(T, key, li, L, pass & 3, o);  // (its status was seen when the pass was prepared)
         }
       }
-      if (list)
-        for (int j = int(T.hd[(pass & 1) * T.hstride + u] & 0xffff); j != kNone; j = nxt[j]) look_at(j, fp[j]);
-      if (hash) {
-        const uint32_t* hh = T.hash + (pass & 1) * d.ghash;
-        r = k;
-        if (T.ngrp > 1) {
-          r = 0;
-          for (int j = 0; j < k; ++j) r += nxt[j] == u ? 1 : 0;
+      const uint16_t* cell = T.cell + ((pass & 1) * T.ngrp + u) * slots;
+      const Meet meet(o);
+      bool moved = !act;
+      int r = 0, nn = 0, n = 0;  // n: members in the table
+      bool list = false;         // some members are in the list
+      uint32_t deps = 0;
+      uint64_t mem = 0, waits = 0, w0 = 0, w1 = 0;
+      if (act && turns(o.fp)) {
+        key ^= 2u;
+        if (kSeveral) *reinterpret_cast<uint32_t*>(&T.W[k].key) = uint32_t(key);  // (the word that holds the direction)
+        moved = true;
+      }
+      auto neighbour = [&](bool m, int j, uint32_t g) {
+        nn += m ? 1 : 0;
+        mem = m ? (mem << 16) | uint64_t(j) : mem;
+        deps = m ? (deps << 1) | (j < k && !turns(g) ? 1u : 0u) : deps;
+      };
+      auto look_at = [&](int j, uint32_t g) {
+        r += j < k ? 1 : 0;
+        neighbour(meet(g) && j != k, j, g);
+      };
+      if (!moved) {
+        if (table) {
+          const int c = T.gcnt[b3 * T.ngrp + u];
+          n = min(c, slots);
+          list = c > slots;
+        } else {
+          list = !scan;
         }
-        mem = ~0ull;
-        for (int s = 0; s < 6; ++s) {
-          const uint32_t pair = s < 2 ? o.dns : s < 4 ? o.fp : o.ups, leg = (s & 1) ? pair >> 16 : pair & 0xffffu;
-          const uint32_t h = hh[leg & (d.ghash - 1)];
-          int e = (h >> 16) == uint32_t(stamp) ? int(h & 0xffff) : kNone;
-          while (e != kNone) {
-            const int j = e >> 1;
-            const uint32_t g = fp[j];
-            if (((e & 1) ? g >> 16 : g & 0xffffu) == leg && j != k) {
-              // (a worm can be found by both of its legs)
-              const uint64_t x = mem ^ (uint64_t(j) * 0x0001000100010001ull);
-              if (!((x - 0x0001000100010001ull) & ~x & 0x8000800080008000ull)) {
-                mem = (mem << 16) | uint64_t(j);
-                deps = (deps << 1) | (j < k && !turns(g) ? 1u : 0u);
-                ++nn;
-              }
-            }
-            e = reinterpret_cast<const uint16_t*>(&T.W[j].lab)[2 * (pass & 1) + (e & 1)];
+        for (int e0 = 0; e0 < n; e0 += 4) {
+          const uint2 four = *reinterpret_cast<const uint2*>(cell + e0);
+  #pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int j = int(((e < 2 ? four.x : four.y) >> (16 * (e & 1))) & 0xffff);
+            if (e0 + e < n) look_at(j, fp[j]);
           }
         }
-      } else if (scan) {
-        for (int j = 0; j < nw; ++j)
-          if (nxt[j] == u) look_at(j, fp[j]);
-      }
-      const P4 b = philox(uint32_t(r), uint32_t(dom * T.ngrp + u), c2_word(kScatter, uint32_t(pass), d.replica),
-                          d.sweep, d.key0, d.key1);
-      w0 = uint64_t(b.x) | (uint64_t(b.y) << 32);
-      w1 = uint64_t(b.z) | (uint64_t(b.w) << 32);
-    }
-    if (act && table && pass > 0) T.gcnt[b3p * T.ngrp + u_old] = 0;
-    u_old = u;
-    phase_tick(d, 5, tclk);
-    int spin = 0;
-    while (!__all_sync(0xffffffffu, moved)) {
-      if (!moved) {
-        bool ready = true;
-        if (nn <= 4) {
-          for (uint32_t m = deps; m; m &= m - 1)
-            ready = ready && dn[(mem >> (16 * (__ffs(int(m)) - 1))) & 0xffff] == stamp;
-        } else {
-          again([&](int j) {
-            if (j < k && !turns(fp[j]) && meet(fp[j])) ready = ready && dn[j] == stamp;
-          });
-        }
-        if (ready) {
-          __threadfence_block();
-          make_move(T, o, key, li, L, w0, w1, [&](auto f) {
-            if (nn <= 4) {
-              for (int e = 0; e < nn; ++e) {
-                const WormRec& w = T.W[(mem >> (16 * e)) & 0xffff];
-                f(int(w.leg), w.key);
+        if (list)
+          for (int j = int(T.hd[(pass & 1) * T.hstride + u] & 0xffff); j != kNone; j = nxt[j]) look_at(j, fp[j]);
+        if (hash) {
+          const uint32_t* hh = T.hash + (pass & 1) * d.ghash;
+          r = k;
+          if (T.ngrp > 1) {
+            r = 0;
+            for (int j = 0; j < k; ++j) r += nxt[j] == u ? 1 : 0;
+          }
+          mem = ~0ull;
+          for (int s = 0; s < 6; ++s) {
+            const uint32_t pair = s < 2 ? o.dns : s < 4 ? o.fp : o.ups, leg = (s & 1) ? pair >> 16 : pair & 0xffffu;
+            const uint32_t h = hh[leg & (d.ghash - 1)];
+            int e = (h >> 16) == uint32_t(stamp) ? int(h & 0xffff) : kNone;
+            while (e != kNone) {
+              const int j = e >> 1;
+              const uint32_t g = fp[j];
+              if (((e & 1) ? g >> 16 : g & 0xffffu) == leg && j != k) {
+                // (a worm can be found by both of its legs)
+                const uint64_t x = mem ^ (uint64_t(j) * 0x0001000100010001ull);
+                if (!((x - 0x0001000100010001ull) & ~x & 0x8000800080008000ull)) neighbour(true, j, g);
               }
-            } else {
-              again([&](int j) {
-                if (j != k) f(int(T.W[j].leg), T.W[j].key);
-              });
+              e = reinterpret_cast<const uint16_t*>(&T.W[j].lab)[2 * (pass & 1) + (e & 1)];
             }
-          });
-          WormRec& w = T.W[k];
-          w.key = key;
-          store_place(w, li, L);
-          __threadfence_block();
-          dn[k] = uint16_t(stamp);
-          moved = true;
+          }
+        } else if (scan) {
+          for (int j = 0; j < nw; ++j)
+            if (nxt[j] == u) look_at(j, fp[j]);
         }
+        if (nn > 4) {  // more than mem holds: all of them into the list
+          nn = 0;
+          auto add = [&](int j) {
+            const uint32_t g = fp[j];
+            if (j == k || !meet(g)) return;
+            if (nn < kNeighbours) {
+              more[nn] = uint16_t(j);
+              waits |= uint64_t(j < k && !turns(g) ? 1 : 0) << nn;
+            }
+            ++nn;
+          };
+          if (scan)
+            for (int j = 0; j < nw; ++j)
+              if (nxt[j] == u) add(j);
+          for (int e = 0; e < n; ++e) add(int(cell[e]));
+          if (list)
+            for (int j = int(T.hd[(pass & 1) * T.hstride + u] & 0xffff); j != kNone; j = nxt[j]) add(j);
+          // (a worm found by both of its legs counted twice: the list stays longer than mem, by this worm itself)
+          while (nn < 5) more[nn++] = uint16_t(k);
+        }
+        const P4 b = philox(uint32_t(r), uint32_t(dom * T.ngrp + u), c2_word(kScatter, uint32_t(pass), d.replica),
+                            d.sweep, d.key0, d.key1);
+        w0 = uint64_t(b.x) | (uint64_t(b.y) << 32);
+        w1 = uint64_t(b.z) | (uint64_t(b.w) << 32);
       }
-      if (++spin > kSpinLimit) { fail(pass + 1, PMWA_ETIMEOUT); break; }
+      if (!kSeveral && act && table && pass > 0) T.gcnt[b3p * T.ngrp + u_old] = 0;
+      u_old = u;
+      phase_tick(d, 5, tclk);
+      int spin = 0, seen = 0;
+      while (!__all_sync(0xffffffffu, moved)) {
+        if (!moved) {
+          bool ready = true;
+          if (nn <= 4) {
+            for (uint32_t m = deps; m; m &= m - 1)
+              ready = ready && dn[(mem >> (16 * (__ffs(int(m)) - 1))) & 0xffff] == stamp;
+          } else if (nn <= kNeighbours) {
+            for (; waits; waits &= waits - 1)
+              if (dn[more[__ffsll((long long)waits) - 1]] != stamp) { ready = false; break; }
+          } else {  // (worms of other groups meet none of this one's intervals)
+            for (; seen < k; ++seen)
+              if (dn[seen] != stamp && !turns(fp[seen]) && meet(fp[seen])) { ready = false; break; }
+          }
+          if (ready) {
+            __threadfence_block();
+            make_move(T, o, key, li, L, w0, w1, k, nw, [&](auto f) {
+              if (nn <= 4) {
+                for (int e = 0; e < nn; ++e) {
+                  const WormRec& w = T.W[(mem >> (16 * e)) & 0xffff];
+                  f(int(w.leg), w.key);
+                }
+              } else {  // (the list, or every worm of the domain)
+                const bool listed = nn <= kNeighbours;
+                for (int e = 0; e < (listed ? nn : nw); ++e) {
+                  const int j = listed ? int(more[e]) : e;
+                  if (j != k) f(int(T.W[j].leg), T.W[j].key);
+                }
+              }
+            });
+            WormRec& w = T.W[k];
+            w.key = key;
+            store_place(w, li, L);
+            __threadfence_block();
+            dn[k] = uint16_t(stamp);
+            moved = true;
+          }
+        }
+        if (++spin > kSpinLimit) { fail(pass + 1, PMWA_ETIMEOUT); break; }
+      }
+      if (d.phase_cycles && threadIdx.x == 0) atomicAdd(d.phase_cycles + 7, (unsigned long long)spin);
+      phase_tick(d, 6, tclk);
+      if (act && pass + 1 < d.n_cycle) prepare(pass + 1, b3n);
     }
-    if (d.phase_cycles && threadIdx.x == 0) atomicAdd(d.phase_cycles + 7, (unsigned long long)spin);
-    phase_tick(d, 6, tclk);
-    if (act && pass + 1 < d.n_cycle) prepare(pass + 1, b3n);
     b3 = b3n;
   }
   __syncthreads();
   if (const int rc = T.perr[d.n_cycle & 1]) tile_fail(T.misc, rc, 5);
-  if (act) T.W[k].key = key;
-}
-
-// All N_cycle passes of a domain with more worms than threads (all threads).
-// As block_passes, with the worms of a thread taken in turn, their state in
-// W[ord[k]] and rounds ended by a block barrier: every round moves the worms
-// whose predecessors have moved.
-__device__ void many_passes(const Tile& T, int dom, int nw, long long& tclk) {
-  const Dev& d = *T.d;
-  const int tid = threadIdx.x, NT = blockDim.x;
-  volatile uint16_t* dn = T.dn;
-  for (int pass = 0; pass < d.n_cycle; ++pass) {
-    const int q = pass & 3, stamp = pass + 1;
-    uint32_t* fp = T.fp + (pass & 1) * d.wcap;
-    const uint16_t* nxt = T.nxt + (pass & 1) * d.wcap;
-    for (int k = tid; k < nw; k += NT) {
-      WormRec& w = T.W[T.ord[k]];
-      join_list(T, k, worm_group(T, w.site, w.slab, q), pass);
-      Ahead o;
-      const int rc = look_ahead(T, w.key, w.site, w.leg, q, o);
-      fp[k] = o.fp;
-      if (rc) tile_fail(T.misc, rc, 5);
-      if (turns(o.fp)) w.key ^= 2u;
-    }
-    __syncthreads();
-    phase_tick(d, 5, tclk);
-    for (int round = 0;; ++round) {
-      int pending = 0;
-      for (int k = tid; k < nw; k += NT) {
-        if (turns(fp[k]) || dn[k] == stamp) continue;
-        WormRec& w = T.W[T.ord[k]];
-        const int u = worm_group(T, w.site, w.slab, q), head = int(T.hd[(pass & 1) * T.hstride + u] & 0xffff);
-        uint64_t key = w.key;
-        int li = w.site, L = w.leg;
-        Ahead o;
-        look_ahead(T, key, li, L, q, o);
-        const Meet meet(o);
-        bool ready = true;
-        int r = 0;
-        for (int j = head; j != kNone; j = nxt[j]) {
-          if (j >= k) continue;
-          ++r;
-          if (!turns(fp[j]) && meet(fp[j])) ready = ready && dn[j] == stamp;
-        }
-        if (!ready) { pending = 1; continue; }
-        __threadfence_block();
-        const P4 b = philox(uint32_t(r), uint32_t(dom * T.ngrp + u), c2_word(kScatter, uint32_t(pass), d.replica),
-                            d.sweep, d.key0, d.key1);
-        make_move(T, o, key, li, L, uint64_t(b.x) | (uint64_t(b.y) << 32), uint64_t(b.z) | (uint64_t(b.w) << 32),
-                  [&](auto f) {
-                    for (int j = head; j != kNone; j = nxt[j])
-                      if (j != k) f(int(T.W[T.ord[j]].leg), T.W[T.ord[j]].key);
-                  });
-        w.key = key;
-        store_place(w, li, L);
-        __threadfence_block();
-        dn[k] = uint16_t(stamp);
-      }
-      if (!__syncthreads_or(pending)) {
-        if (d.phase_cycles && tid == 0) atomicAdd(d.phase_cycles + 7, (unsigned long long)(round + 1));
-        break;
-      }
-      if (round >= nw) {  // (each round moves the first waiting worm of every group: never taken)
-        if (tid == 0) tile_fail(T.misc, PMWA_EINVARIANT, 7);
-        break;
-      }
-    }
-    phase_tick(d, 6, tclk);
-    __syncthreads();
-    if (T.misc->err) return;
-  }
+  if (!kSeveral && act) T.W[k].key = key;
 }
 
 // All N_cycle passes of a domain holding nw <= 32 worms, run by one warp
@@ -907,7 +921,7 @@ __device__ int small_passes(const Tile& T, int dom, int nw, int lane) {
     unsigned done = turning;
     while (done != 0xffffffffu) {
       if (!moved && (wait & ~done) == 0) {
-        make_move(T, o, key, li, L, w0, w1, [&](auto f) {
+        make_move(T, o, key, li, L, w0, w1, lane, nw, [&](auto f) {
           for (unsigned m = near; m; m &= m - 1) {
             const int j = __ffs(int(m)) - 1;
             f(int(T.W[j].leg), T.W[j].key);
@@ -1063,8 +1077,12 @@ __device__ __forceinline__ void create_worms(const Tile& T, const ZigTab& Z, int
     }
     const P4 b = philox(block, unit, c2_word(kRegen, 0, d.replica), d.sweep, d.key0, d.key1);
     ++block;
-    if (run) step(uint64_t(b.x) | (uint64_t(b.y) << 32));
-    if (run && state != kDone && !bad) step(uint64_t(b.z) | (uint64_t(b.w) << 32));
+    uint64_t w = uint64_t(b.x) | (uint64_t(b.y) << 32);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      if (run && state != kDone && !bad) step(w);
+      w = uint64_t(b.z) | (uint64_t(b.w) << 32);
+    }
   }
   if (bad) tile_fail(T.misc, bad, 4);
 }
@@ -1181,6 +1199,9 @@ __device__ __forceinline__ void merge_site(const Tile& T, int li, const uint64_t
     }
   }
 }
+
+// the term of a site without legs (out of line: the series' code is long)
+__device__ __noinline__ bool xg_fix_circle(GridScale XQ, uint64_t& v) { return xg_fix(0, kTwo59, XQ, v); }
 
 template <bool OTF>
 __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int stop, unsigned char* sm,
@@ -1462,17 +1483,25 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
       for (int li = tid; li < nds; li += NT) T.rng[li] = uint32_t(T.off[li]) | (uint32_t(T.off[li + 1]) << 16);
       for (int k = tid; k < nw; k += NT) T.dn[k] = 0;
       if (tid < 2) T.perr[tid] = PMWA_OK;
-      if (nw > 0 && nw <= NT) {  // the worms into label order, one a thread
+      if (nw > kMaxTurns * NT) {
+        if (tid == 0) tile_fail(misc, PMWA_EINVARIANT, 7);
+      } else if (nw > NT) {  // the worms into label order, several a thread
+        WormRec w[kMaxTurns];
+        for (int k = tid, t = 0; k < nw; k += NT, ++t) w[t] = T.W[T.ord[k]];
+        __syncthreads();
+        for (int k = tid, t = 0; k < nw; k += NT, ++t) T.W[k] = w[t];
+      } else if (nw > 0) {  // one a thread
         WormRec w{};
         if (tid < nw) w = T.W[T.ord[tid]];
         __syncthreads();
         if (tid < nw) T.W[tid] = w;
       }
       __syncthreads();
+      if (misc->err) goto fail;
       if (nw > NT) {
-        many_passes(T, dom, nw, tclk);
+        block_passes<true>(T, dom, nw, tclk);
       } else if (nw > 32) {
-        block_passes(T, dom, nw, tclk);
+        block_passes<false>(T, dom, nw, tclk);
       } else if (nw > 0 && tid < 32) {  // few worms: one warp, no barrier
         const int rc = small_passes(T, dom, nw, tid);
         if (rc && tid == 0) tile_fail(misc, rc, 5);
@@ -1609,7 +1638,7 @@ __device__ __forceinline__ void tile_body(const Dev& d, const int dom, const int
       if (base) add128(olo, ohi, kTwo62, 0);
       if (nl == 0) {  // a site without legs is one interval of sigma = 0
         uint64_t v;
-        if (xg_fix(0, kTwo59, d.XQ, v)) add128(qlo, qhi, v, 0);
+        if (xg_fix_circle(d.XQ, v)) add128(qlo, qhi, v, 0);
         else q += xg_sigma(0, double(kTwo59) * d.XW);
       }
     }
@@ -1783,14 +1812,20 @@ bool plan_tile_smem(Dev* d, double legs_want) {
   d->sm_bkt = int(w); w = up16(w + size_t(nb) * sizeof(int));
   d->sm_fill = int(w); w = up16(w + size_t(nb) * sizeof(int));
   // the groups' member tables, where the reserve has room for them
-  const size_t cells = up16(size_t(nsub) * 2 * kGroupSlots * sizeof(uint16_t)), counts = up16(size_t(nsub) * 3 * sizeof(int));
-  d->gtab = w + cells + counts <= size_t(d->sm_plan) ? 1 : 0;
-  d->sm_cell = int(w); w += d->gtab ? cells : 0;
+  auto cells = [&](int slots) { return up16(size_t(nsub) * 2 * size_t(slots) * sizeof(uint16_t)); };
+  const size_t counts = up16(size_t(nsub) * 3 * sizeof(int));
+  d->gtab = w + cells(kGroupSlots) + counts <= size_t(d->sm_plan) ? 1 : 0;
+  d->gslots = kGroupSlots;
+  const double root = std::sqrt(std::max(0.0, double(d->wcap) - 64.0)) - 8.0, mean = root * root / nsub;
+  const int want_slots = nsub > kScanGroups || mean < kScanMembers ? int(mean + 3.0 * std::sqrt(mean)) : 0;
+  while (d->gtab && d->gslots < std::min(want_slots, 64) && w + cells(d->gslots + 4) + counts <= size_t(d->sm_plan))
+    d->gslots += 4;
+  d->sm_cell = int(w); w += d->gtab ? cells(d->gslots) : 0;
   d->sm_gcnt = int(w); w += d->gtab ? counts : 0;
   // and chains of worms by leg: as many heads as fit, a power of two
   d->sm_hash = int(w);
   d->ghash = 0;
-  for (int h = 64; h <= 1024 && w + 8 * size_t(h) <= size_t(d->sm_plan); h *= 2) d->ghash = h;
+  for (int h = 64; nsub <= kScanGroups && h <= 1024 && w + 8 * size_t(h) <= size_t(d->sm_plan); h *= 2) d->ghash = h;
   w += 8 * size_t(d->ghash);
   d->sm_total = int(std::max(w, o + pool_bytes + (staged ? size_t(stage) : 0)));
   return d->sm_plan <= kSmemLimit - 1024 && d->sm_total <= d->sm_plan;
@@ -1799,9 +1834,13 @@ bool plan_tile_smem(Dev* d, double legs_want) {
 int upload_zig_tile(const Zig& z) { return upload_constants(z); }
 
 // CTA sizes of the sweep kernel, `ctas` domains being launched together (class
-// 0: 64 threads, 1: 128, 2: 256, 3: 512).  A domain takes a thread for every
-// other bond at least (its sites), and three quarters of a thread for a worm
-// of the bound on their mean: Step 5 runs a worm a thread.  Beyond that a CTA
+// 0: 64 threads, 1: 128, 2: 256, 3: 512).  The least class follows from the
+// sites, up to 32 / 96 / more, and from the bound on the mean of the worms, which
+// Step 5 gives a thread each: up to 48 for 64 threads; for 128 up to 96 of a
+// domain of 32 sites, and up to 384, three turns of a thread, of a larger one,
+// whose other phases fill the 128 threads (8x8 sites at beta t = 4, eta = 0.6,
+// 1600 domains: 1.33 ms with 256 threads, 1.21 with 128; 4x4 at eta = 2: 6.66 and 9.1).
+// There is no such bound above.  Beyond the least class a CTA
 // takes as many threads as cost no other CTA its place on the SM, which its
 // shared memory or the number of domains limits: the work of Step 3, Step 4 and
 // the output is then spread over more warps, and a merge cut into more parts.
@@ -1811,7 +1850,7 @@ int upload_zig_tile(const Zig& z) { return upload_constants(z); }
 int tile_class(const Dev& d, int ctas) {
   const int sites = d.dom_x * d.dom_y;
   const double worms = d.beta * d.eta * sites;
-  int c = sites <= 32 && worms <= 48.0 ? 0 : sites <= 96 && worms <= 96.0 ? 1 : 2;
+  int c = sites <= 32 && worms <= 48.0 ? 0 : sites <= 96 && worms <= (sites <= 32 ? 96.0 : 384.0) ? 1 : 2;
   // CTAs an SM has to hold (registers hold 8 >> c of class c)
   const int by_smem = std::max(1, int((228LL * 1024) / (static_cast<long long>(d.sm_total) + 2048)));
   const int held = std::min(by_smem, (ctas - 1) / kSms + 1);

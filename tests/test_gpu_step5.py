@@ -72,3 +72,54 @@ def test_step5_bit_exact(kw, shift):
     a, b = g.rows(), o.rows()
     for f in ROW_FIELDS:
         assert np.array_equal(a[f], b[f][-len(a):]), f
+
+
+# More worms than the CTA has threads (512 of them with one domain; in a batch
+# a CTA takes what its shared memory leaves room for): a thread's worms in
+# turns, with sub-blocks, temporal slabs, one group (chains by leg) and a few,
+# sparse and with many worms in one interval
+TURNS = [
+    dict(Lx=20, Ly=20, beta=6.0, eta=0.3, sub_block=2, n_cycle=5, seed=11),
+    dict(Lx=20, Ly=20, beta=6.0, eta=0.3, sub_block=4, n_cycle=5, seed=12),
+    dict(Lx=20, Ly=20, beta=6.0, eta=0.3, sub_block=0, n_cycle=5, seed=13),
+    dict(Lx=20, Ly=20, beta=6.0, eta=0.3, sub_block=0, dom_tau=4, n_cycle=5, seed=14),
+    dict(Lx=20, Ly=20, beta=6.0, eta=0.3, sub_block=2, dom_tau=3, n_cycle=5, seed=15),
+    dict(Lx=8, Ly=8, beta=6.0, t=0.5, eta=2.0, sub_block=2, n_cycle=5, seed=16),
+    dict(Lx=8, Ly=8, beta=6.0, t=0.5, eta=2.0, sub_block=4, n_cycle=5, seed=17),
+    dict(Lx=6, Ly=6, beta=8.0, t=0.25, eta=2.5, sub_block=0, n_cycle=5, seed=18),
+    dict(Lx=24, Ly=24, beta=4.0, eta=0.6, sub_block=8, n_cycle=5, seed=19),
+]
+
+
+@pytest.mark.parametrize("shift", [0, 24, 36])
+@pytest.mark.parametrize("kw", TURNS, ids=["c%d" % i for i in range(len(TURNS))])
+def test_more_worms_than_threads_bit_exact(kw, shift):
+    g, o = P.Sim(**kw), O.Oracle(**kw)
+    o.sweep(8)
+    snap = o.export()
+    if shift:
+        snap = squeezed(snap, shift)
+    for s in range(8, 11):
+        for x in (g, o):
+            x.import_(snap)
+            x.sweep_index = s
+            x.sweep(1)
+        snap = o.export()
+        assert np.array_equal(g.export(), snap), "sweep %d" % s
+    a, b = g.rows(), o.rows()
+    for f in ROW_FIELDS:
+        assert np.array_equal(a[f], b[f][-len(a):]), f
+    assert a["n_w"].min() > 512  # worms after a sweep; Step 5 neither makes nor removes any
+
+
+@pytest.mark.parametrize("kw", CASES[2:6] + TURNS, ids=["c%d" % i for i in range(4 + len(TURNS))])
+def test_several_domains_of_a_batch_bit_exact(kw):
+    """The same in the CTA that a full machine would get, and 2x2 domains."""
+    kws = [dict(kw, seed=100 + i, Lx=(1 + i % 2) * kw["Lx"], Ly=(1 + i % 2) * kw["Ly"], dom_x=kw["Lx"],
+                dom_y=kw["Ly"], n_cycle=3) for i in range(2)]
+    batch = P.Batch(kws)
+    batch.sweep(5)
+    for i, k in enumerate(kws):
+        o = O.Oracle(**k)
+        o.sweep(5)
+        assert np.array_equal(batch.export(i), o.export()), k
