@@ -1,7 +1,7 @@
 // pmwa_green.cu -- Supplement S-I estimators resolved by the component of Q.
 //
-//   k_rho_alpha       rho_b and rho_b+ at K equal-time slices, one warp per site
-//   k_green_tau_site  the two-point densities of one site (r = 0), one warp per site
+//   k_rho_alpha       rho_b and rho_b+ at K equal-time slices, a lane a slice
+//   k_green_tau_site  the two-point densities of one site (r = 0), lanes over its slices
 //   k_green_tau_r     products of one-point densities of two sites (r >= 1)
 //
 // For X inside the interval I between two vertex legs of a site (p the state
@@ -155,6 +155,11 @@ __global__ void __launch_bounds__(128) k_rho_alpha(const __grid_constant__ Dev d
 //     handed to the lanes of their dk.
 // The binary64 pipe (2 lanes a cycle and SM) bounds it: with every pair's
 // seven exponentials 128x128 sites and K = 32 took 18.1 ms, now 0.62 ms.
+//
+// With K <= 16 slices a warp takes 32 >> sh sites, 2^sh >= K lanes each (one for
+// K above 16).  The call for 256x256 sites at rmax = 8, a thread a site -> a warp
+// -> now: K = 2 0.296 -> 0.939 -> 0.166 ms, K = 4 1.08 -> 1.07 -> 0.25, K = 8 4.36
+// -> 1.56 -> 0.53, K = 16 17.4 -> 2.24 -> 1.30.
 constexpr int kTauWarps = 4;
 struct TauSlices {
   double rb[kMaxGreenSlices], rbd[kMaxGreenSlices];              // densities of b, b+
@@ -162,62 +167,60 @@ struct TauSlices {
   uint64_t M1[kMaxGreenSlices];
   int iv[kMaxGreenSlices];
   uint8_t pq[kMaxGreenSlices];
-  short first[kMaxGreenSlices + 1];                              // pairs before slice k's
+  short first[kMaxGreenSlices + 32];                             // pairs before slice k's
   double v[2][32];
   short dk[32];
 };
-__global__ void __launch_bounds__(32 * kTauWarps) k_green_tau_site(const __grid_constant__ Dev d, int K,
+__global__ void __launch_bounds__(32 * kTauWarps) k_green_tau_site(const __grid_constant__ Dev d, int K, int sh,
                                                                   double* sums, double* rho) {
-  __shared__ TauSlices sh[kTauWarps];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  TauSlices& t = sh[wid];
+  __shared__ TauSlices sm[kTauWarps];
+  const int G = 1 << sh, lane = threadIdx.x & (G - 1), sub = (threadIdx.x & 31) >> sh, wid = threadIdx.x >> 5;
+  TauSlices& t = sm[wid];
+  const int s0 = sub * G, f0 = sub * (G + 1), per = 32 >> sh;  // this site's places in t (G < 32: K <= G)
   const double eta2 = __dmul_rn(d.eta, d.eta);
   double acc[2] = {0.0, 0.0};  // dk = lane, lane + 32
-  for (long long s = (long long)blockIdx.x * kTauWarps + wid; s < d.N; s += (long long)gridDim.x * kTauWarps) {
-    const uint64_t* Kk = d.keyA + size_t(s) * d.cap;
-    const int n = min(int(d.cntA[s] & kCntMaskG), d.cap), last = last_leg(Kk, n);
+  const long long step = (long long)gridDim.x * kTauWarps * per;
+  for (long long b = ((long long)blockIdx.x * kTauWarps + wid) * per; b < d.N; b += step) {
+    const long long s = b + sub;
+    const bool act = s < d.N;
+    const uint64_t* Kk = d.keyA + size_t(act ? s : 0) * d.cap;
+    const int n = act ? min(int(d.cntA[s] & kCntMaskG), d.cap) : 0, last = act ? last_leg(Kk, n) : -1;
     __syncwarp();
-    for (int k = lane; k < K; k += 32) {
+    for (int k = lane; act && k < K; k += G) {
       SliceInfo z;
       slice_one(Kk, n, last, K, k, &z);
       const Parts e = parts_of(z, d.XW);
-      t.rb[k] = rho_one(z, e, 0, d.eta, d.XW);
-      t.rbd[k] = rho_one(z, e, 1, d.eta, d.XW);
-      if (rho) *reinterpret_cast<double2*>(rho + (size_t(s) * K + k) * 2) = make_double2(t.rb[k], t.rbd[k]);
-      t.elo[k] = e.elo;
-      t.ehi[k] = e.ehi;
-      t.den[k] = e.den;
-      t.M1[k] = z.M1;
-      t.iv[k] = z.iv;
-      t.pq[k] = uint8_t(z.p | (z.q << 1));
+      const double b0 = rho_one(z, e, 0, d.eta, d.XW), b1 = rho_one(z, e, 1, d.eta, d.XW);
+      t.rb[s0 + k] = b0;
+      t.rbd[s0 + k] = b1;
+      if (rho) *reinterpret_cast<double2*>(rho + (size_t(s) * K + k) * 2) = make_double2(b0, b1);
+      t.elo[s0 + k] = e.elo;
+      t.ehi[s0 + k] = e.ehi;
+      t.den[s0 + k] = e.den;
+      t.M1[s0 + k] = z.M1;
+      t.iv[s0 + k] = z.iv;
+      t.pq[s0 + k] = uint8_t(z.p | (z.q << 1));
     }
     __syncwarp();
-    if (last < 0) {  // no legs: every pair by the trace over the circle
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int dk = lane + 32 * h;
-        if (dk == 0 || dk >= K) continue;
-        for (int k = 0; k < K; ++k) {
-          SliceInfo z1, z2;
-          slice_one(Kk, n, last, K, k, &z1);
-          slice_one(Kk, n, last, K, (k + dk) % K, &z2);
-          acc[h] = __dadd_rn(acc[h], rho_two_ring(z1, 1, z2, 0, d.eta, d.XW));
-        }
-      }
-      continue;
-    }
-    // different intervals
+    // no legs: every pair by the trace over the circle; else different intervals
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int dk = lane + 32 * h;
-      if (dk == 0 || dk >= K) continue;
+      const int dk = lane + G * h;
+      if (!act || dk == 0 || dk >= K) continue;
       double a = 0.0;
       int j = dk;
       for (int k = 0; k < K; ++k) {
-        if (t.iv[k] != t.iv[j]) a = __dadd_rn(a, __dmul_rn(t.rbd[k], t.rb[j]));
+        if (last < 0) {
+          SliceInfo z1, z2;
+          slice_one(Kk, n, last, K, k, &z1);
+          slice_one(Kk, n, last, K, j, &z2);
+          acc[h] = __dadd_rn(acc[h], rho_two_ring(z1, 1, z2, 0, d.eta, d.XW));
+        } else if (t.iv[s0 + k] != t.iv[s0 + j]) {
+          a = __dadd_rn(a, __dmul_rn(t.rbd[s0 + k], t.rb[s0 + j]));
+        }
         if (++j == K) j = 0;
       }
-      acc[h] = __dadd_rn(acc[h], a);
+      if (last >= 0) acc[h] = __dadd_rn(acc[h], a);
     }
     // one interval: slice k with the slices behind it up to the interval's end
     int mine[2], sum = 0;
@@ -225,66 +228,71 @@ __global__ void __launch_bounds__(32 * kTauWarps) k_green_tau_site(const __grid_
     for (int h = 0; h < 2; ++h) {
       const int k = 2 * lane + h;
       int run = 0;
-      if (k < K) {
+      if (last >= 0 && k < K) {
         int j = k + 1 == K ? 0 : k + 1;
-        while (run < K - 1 && t.iv[j] == t.iv[k] && t.M1[j] >= t.M1[k]) { ++run; j = j + 1 == K ? 0 : j + 1; }
+        while (run < K - 1 && t.iv[s0 + j] == t.iv[s0 + k] && t.M1[s0 + j] >= t.M1[s0 + k]) {
+          ++run;
+          j = j + 1 == K ? 0 : j + 1;
+        }
       }
       mine[h] = run;
       sum += run;
     }
     int before = sum;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, before, o);
+    for (int o = 1; o < G; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, before, o, G);
       if (lane >= o) before += x;
     }
-    const int total = __shfl_sync(0xffffffffu, before, 31);
+    const int total = __shfl_sync(0xffffffffu, before, G - 1, G);
     before -= sum;
-    if (2 * lane <= K) t.first[2 * lane] = short(before);
-    if (2 * lane + 1 <= K) t.first[2 * lane + 1] = short(before + mine[0]);
-    if (lane == 31 && K == 64) t.first[64] = short(total);
+    if (2 * lane <= K) t.first[f0 + 2 * lane] = short(before);
+    if (2 * lane + 1 <= K) t.first[f0 + 2 * lane + 1] = short(before + mine[0]);
+    if (lane == G - 1 && K == 2 * G) t.first[f0 + K] = short(total);
     __syncwarp();
-    for (int p0 = 0; p0 < total; p0 += 32) {
+    const int most = int(__reduce_max_sync(0xffffffffu, unsigned(total)));
+    for (int p0 = 0; p0 < most; p0 += G) {
       const int p = p0 + lane;
       if (p < total) {
         int lo = 0, hi = K;  // the slice k with first[k] <= p < first[k + 1]
         while (hi - lo > 1) {
           const int mid = (lo + hi) >> 1;
-          if (t.first[mid] <= p) lo = mid; else hi = mid;
+          if (t.first[f0 + mid] <= p) lo = mid; else hi = mid;
         }
-        const int k = lo, dk = p - t.first[k] + 1, j = k + dk >= K ? k + dk - K : k + dk;
-        const double eb = em1_of(t.M1[j] - t.M1[k], d.XW), den = __dmul_rn(4.0, t.den[k]);
-        const int pp = t.pq[k] & 1, qq = t.pq[k] >> 1;
+        const int k = lo, dk = p - t.first[f0 + k] + 1, j = k + dk >= K ? k + dk - K : k + dk;
+        const double eb = em1_of(t.M1[s0 + j] - t.M1[s0 + k], d.XW), den = __dmul_rn(4.0, t.den[s0 + k]);
+        const int pp = t.pq[s0 + k] & 1, qq = t.pq[s0 + k] >> 1;
         // lower operator on k, upper on j: b+ on k and b on j, then the other way round
         auto v = [&](int aL, int aU) {
-          const double num = __dmul_rn(__dmul_rn(F_of(qq ^ q_out(aU), t.ehi[j]), F_of(q_in(aU) ^ q_out(aL), eb)),
-                                       F_of(q_in(aL) ^ pp, t.elo[k]));
+          const double num = __dmul_rn(__dmul_rn(F_of(qq ^ q_out(aU), t.ehi[s0 + j]), F_of(q_in(aU) ^ q_out(aL), eb)),
+                                       F_of(q_in(aL) ^ pp, t.elo[s0 + k]));
           return __dmul_rn(eta2, __ddiv_rn(num, den));
         };
-        t.v[0][lane] = v(1, 0);
-        t.v[1][lane] = v(0, 1);
-        t.dk[lane] = short(dk);
+        t.v[0][s0 % 32 + lane] = v(1, 0);
+        t.v[1][s0 % 32 + lane] = v(0, 1);
+        t.dk[s0 % 32 + lane] = short(dk);
       }
       __syncwarp();
-      const int m = min(32, total - p0);
-      for (int i = 0; i < m; ++i) {
-        const int dk = t.dk[i];
+      for (int i = 0; i < min(G, total - p0); ++i) {
+        const int dk = t.dk[s0 % 32 + i];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          if (lane + 32 * h == dk) acc[h] = __dadd_rn(acc[h], t.v[0][i]);
-          if (lane + 32 * h == K - dk) acc[h] = __dadd_rn(acc[h], t.v[1][i]);
+          if (lane + G * h == dk) acc[h] = __dadd_rn(acc[h], t.v[0][s0 % 32 + i]);
+          if (lane + G * h == K - dk) acc[h] = __dadd_rn(acc[h], t.v[1][s0 % 32 + i]);
         }
       }
       __syncwarp();
     }
   }
   __syncwarp();
-  t.rb[lane] = acc[0];
-  t.rb[lane + 32] = acc[1];
+  t.rb[threadIdx.x & 31] = acc[0];  // (dk = lane of each of the warp's sites)
+  t.rb[(threadIdx.x & 31) + 32] = acc[1];
   __syncthreads();
   const int dk = threadIdx.x;
   if (dk > 0 && dk < K) {  // (K <= 64 <= the block's threads)
     double v = 0.0;
-    for (int w = 0; w < kTauWarps; ++w) v = __dadd_rn(v, sh[w].rb[dk]);
+    const int at = dk < G ? dk : dk - G + 32;  // (dk >= G: its second sum; one site a warp then, or K = 2 G)
+    for (int w = 0; w < kTauWarps; ++w)
+      for (int q = 0; q < per; ++q) v = __dadd_rn(v, sm[w].rb[at + q * G]);
     atomicAdd(sums + dk, v);
   }
 }
@@ -297,32 +305,38 @@ __global__ void __launch_bounds__(32 * kTauWarps) k_green_tau_site(const __grid_
 // registers from site to site: the binary64 pipe is the bound (N 2 rmax K^2
 // multiply-adds; 128x128 sites, K = 32, rmax = 8: 0.43 ms of it; measured 0.47
 // ms, 1.74 ms with a thread a site and two lines a lane for each product).
+// Up to 16 slices a warp takes 32 >> sh sites, 2^sh lanes each.
 constexpr int kTauRowWarps = 8, kTauRowR = 8;
-__global__ void __launch_bounds__(32 * kTauRowWarps) k_green_tau_r(int Lx, int Ly, int K, int rmax,
+__global__ void __launch_bounds__(32 * kTauRowWarps) k_green_tau_r(int Lx, int Ly, int K, int sh, int rmax,
                                                                   const double* __restrict__ rho, double* sums) {
   extern __shared__ __align__(16) double tsm[];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, dir = int(blockIdx.y), r0 = int(blockIdx.z) * kTauRowR;
-  double* bd = tsm + size_t(wid) * 3 * K;  // K densities of b+, then 2 K of b (twice over)
+  const int G = 1 << sh, lane = threadIdx.x & (G - 1), group = threadIdx.x >> sh, groups = int(blockDim.x) >> sh;
+  const int dir = int(blockIdx.y), r0 = int(blockIdx.z) * kTauRowR;
+  double* bd = tsm + size_t(group) * 3 * K;  // K densities of b+, then 2 K of b (twice over)
   double* b = bd + K;
-  double* part = tsm + size_t(kTauRowWarps) * 3 * K;  // the block's sums, [kTauRowR][K]
+  double* part = tsm + size_t(groups) * 3 * K;  // the block's sums, [kTauRowR][K]
   for (int i = threadIdx.x; i < kTauRowR * K; i += blockDim.x) part[i] = 0.0;
   double acc[kTauRowR][2] = {};
-  const long long N = (long long)Lx * Ly;
-  for (long long i = (long long)blockIdx.x * kTauRowWarps + wid; i < N; i += (long long)gridDim.x * kTauRowWarps) {
-    const int x = int(i % Lx), y = int(i / Lx);
-    for (int k = lane; k < K; k += 32) bd[k] = rho[(size_t(i) * K + k) * 2 + 1];
+  const long long N = (long long)Lx * Ly, step = (long long)gridDim.x * groups;
+  for (long long i0 = (long long)blockIdx.x * groups; i0 < N; i0 += step) {
+    const long long i = i0 + group;
+    const bool act = i < N;
+    const int x = int(act ? i % Lx : 0), y = int(act ? i / Lx : 0);
+    if (act)
+      for (int k = lane; k < K; k += G) bd[k] = rho[(size_t(i) * K + k) * 2 + 1];
 #pragma unroll
     for (int e = 0; e < kTauRowR; ++e) {
       const int r = r0 + e + 1;
       if (r > rmax) break;
       const size_t j = dir == 0 ? size_t(y) * Lx + (x + r) % Lx : size_t((y + r) % Ly) * Lx + x;
       __syncwarp();
-      for (int k = lane; k < K; k += 32) b[k] = b[k + K] = rho[(j * K + k) * 2];
+      if (act)
+        for (int k = lane; k < K; k += G) b[k] = b[k + K] = rho[(j * K + k) * 2];
       __syncwarp();
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int dk = lane + 32 * h;
-        if (dk < K) {
+        const int dk = lane + G * h;
+        if (act && dk < K) {
           double a = 0.0;
           for (int k = 0; k < K; ++k) a = fma(b[k + dk], bd[k], a);
           acc[e][h] += a;
@@ -335,8 +349,11 @@ __global__ void __launch_bounds__(32 * kTauRowWarps) k_green_tau_r(int Lx, int L
 #pragma unroll
   for (int e = 0; e < kTauRowR; ++e)
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (r0 + e + 1 <= rmax && lane + 32 * h < K) atomicAdd(part + e * K + lane + 32 * h, acc[e][h]);
+    for (int h = 0; h < 2; ++h) {
+      double v = acc[e][h];  // (the warp's sites first: their sums go to one address)
+      for (int o = G; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (r0 + e + 1 <= rmax && lane + G * h < K && (threadIdx.x & 31) < G) atomicAdd(part + e * K + lane + G * h, v);
+    }
   __syncthreads();
   const int nr = min(kTauRowR, rmax - r0);
   for (int i = threadIdx.x; i < nr * K; i += blockDim.x)
@@ -403,14 +420,18 @@ __device__ double rho_interval(const SliceInfo* z, const int* idx, const int* a,
 // the whole circle of a site without legs) in order of first appearance, each
 // group's points in time order (insertion sort by the offset from the lower
 // leg, or by time point on a site without legs).
-// One warp per tuple, lanes over the shifts (32 at a time), whose products are
-// then added in order: a thread a tuple ran K dependent searches one after the
-// other.  4096 tuples of 3, K = 32: 0.74 -> 0.14 ms.
-__global__ void __launch_bounds__(64) k_npoint_alpha(const __grid_constant__ Dev d, int K, int n, int m,
+// 2^sh lanes a tuple, one a shift at a time, whose products are then added in
+// order: the fewest that fill the machine (tuple_lanes).  A warp a tuple, few of
+// whose lanes have a shift or whose lanes all add the 32 products, is bound by
+// the instructions it issues once there are many tuples; a thread a tuple runs K
+// dependent searches one after the other.  4096 tuples of 3, K = 32: a thread
+// 0.74, a warp 0.14 ms; the call for 10^6 tuples of 1 at K = 1 / 8 / 32: a thread
+// 1.79 / 3.93 / 11.4, a warp 11.2 / 13.4 / 15.1, now 1.77 / 3.87 / 11.2 ms.
+__global__ void __launch_bounds__(64) k_npoint_alpha(const __grid_constant__ Dev d, int K, int sh, int n, int m,
                                                      const int32_t* __restrict__ pts, double* out) {
-  const long long j = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (j >= m) return;
+  const long long id = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> sh;
+  const int lanes = 1 << sh, lane = threadIdx.x & (lanes - 1);
+  const long long j = id < m ? id : m - 1;  // (the last warp's spare lanes repeat the last tuple)
   const int32_t* t = pts + size_t(j) * size_t(n) * 3;
   int last[kMaxNpoint], cnt[kMaxNpoint];
   for (int c = 0; c < n; ++c) {
@@ -418,13 +439,13 @@ __global__ void __launch_bounds__(64) k_npoint_alpha(const __grid_constant__ Dev
     last[c] = last_leg(d.keyA + size_t(t[3 * c]) * d.cap, cnt[c]);
   }
   double acc = 0.0;
-  for (int sh0 = 0; sh0 < K; sh0 += 32) {
-    const int sh = sh0 + lane;
+  for (int k0 = 0; k0 < K; k0 += lanes) {
+    const int k = k0 + lane;
     double prod = 1.0;
-    if (sh < K) {
+    if (k < K) {
       SliceInfo z[kMaxNpoint];
       for (int c = 0; c < n; ++c)
-        slice_one(d.keyA + size_t(t[3 * c]) * d.cap, cnt[c], last[c], K, (t[3 * c + 1] + sh) % K, &z[c]);
+        slice_one(d.keyA + size_t(t[3 * c]) * d.cap, cnt[c], last[c], K, (t[3 * c + 1] + k) % K, &z[c]);
       unsigned done = 0;
       for (int c = 0; c < n; ++c) {
         if (done & (1u << c)) continue;
@@ -433,26 +454,39 @@ __global__ void __launch_bounds__(64) k_npoint_alpha(const __grid_constant__ Dev
           if (!(done & (1u << e)) && t[3 * e] == t[3 * c] && z[e].iv == z[c].iv) { idx[g++] = e; done |= 1u << e; }
         const bool ring = z[c].iv < 0;
         for (int i = 1; i < g; ++i)
-          for (int k = i; k > 0; --k) {
-            const uint64_t ka = ring ? z[idx[k]].pt : z[idx[k]].off, kb = ring ? z[idx[k - 1]].pt : z[idx[k - 1]].off;
-            if (ka < kb) { const int tmp = idx[k]; idx[k] = idx[k - 1]; idx[k - 1] = tmp; } else break;
+          for (int q = i; q > 0; --q) {
+            const uint64_t ka = ring ? z[idx[q]].pt : z[idx[q]].off, kb = ring ? z[idx[q - 1]].pt : z[idx[q - 1]].off;
+            if (ka < kb) { const int tmp = idx[q]; idx[q] = idx[q - 1]; idx[q - 1] = tmp; } else break;
           }
         for (int i = 0; i < g; ++i) a[i] = t[3 * idx[i] + 2];
         prod = __dmul_rn(prod, rho_interval(z, idx, a, g, d.eta, d.XW));
       }
     }
-    for (int i = 0; i < min(32, K - sh0); ++i) acc = __dadd_rn(acc, __shfl_sync(0xffffffffu, prod, i));
+    if (sh == 0)
+      acc = __dadd_rn(acc, prod);
+    else
+      for (int i = 0; i < min(lanes, K - k0); ++i) acc = __dadd_rn(acc, __shfl_sync(0xffffffffu, prod, i, lanes));
   }
   double etan = 1.0;
   for (int c = 0; c < n; ++c) etan = __dmul_rn(etan, d.eta);
-  if (lane == 0) out[j] = __ddiv_rn(__ddiv_rn(acc, double(K)), etan);
+  if (lane == 0 && id < m) out[j] = __ddiv_rn(__ddiv_rn(acc, double(K)), etan);
+}
+
+// log2 of a tuple's lanes: as many as the slices leave work for (slice_lanes),
+// down to where m tuples have a thread for each of a full machine's 152 x 1024
+int tuple_lanes(int K, int m) {
+  int sh = slice_lanes(K);
+  while (sh > 0 && (static_cast<long long>(m) << (sh - 1)) >= 152 * 1024) --sh;
+  return sh;
 }
 
 }  // namespace
 
 int launch_npoint_alpha(const Dev& d, int K, int n, int m, const int32_t* pts, double* out, void* stream) {
   if (m <= 0) return 0;
-  k_npoint_alpha<<<unsigned((static_cast<long long>(m) + 1) / 2), 64, 0, cudaStream_t(stream)>>>(d, K, n, m, pts, out);
+  const int sh = tuple_lanes(K, m);
+  k_npoint_alpha<<<unsigned(((static_cast<long long>(m) << sh) + 63) / 64), 64, 0, cudaStream_t(stream)>>>(d, K, sh, n, m,
+                                                                                                      pts, out);
   return int(cudaGetLastError());
 }
 
@@ -477,13 +511,19 @@ int launch_green_tau(const Dev& d, int K, int rmax, double* rho, double* sums, v
   cudaStream_t st = cudaStream_t(stream);
   const size_t nsum = size_t(2) * size_t(rmax + 1) * size_t(K);
   if (cudaMemsetAsync(sums, 0, nsum * sizeof(double), st) != cudaSuccess) return int(cudaGetLastError());
-  const int bs = std::min((d.N + kTauWarps - 1) / kTauWarps, 152 * 4);
-  k_green_tau_site<<<bs, 32 * kTauWarps, 0, st>>>(d, K, sums, rmax > 0 ? rho : nullptr);
-  if (cudaGetLastError() != cudaSuccess) return PMWA_ECUDA;
+  const int sh = slice_lanes(K), per = 32 >> sh;
+  if (K > 1) {
+    const int bs = std::min((d.N + kTauWarps * per - 1) / (kTauWarps * per), 152 * 4);
+    k_green_tau_site<<<bs, 32 * kTauWarps, 0, st>>>(d, K, sh, sums, rmax > 0 ? rho : nullptr);
+    if (cudaGetLastError() != cudaSuccess) return PMWA_ECUDA;
+  } else if (rmax > 0) {  // one slice: no pairs of slices on one site, the densities alone
+    if (const int rc = launch_rho_alpha(d, K, 0, d.N, rho, nullptr, stream)) return rc;
+  }
   if (rmax > 0) {
-    const size_t smem = (size_t(3 * kTauRowWarps) + kTauRowR) * size_t(K) * sizeof(double);
-    const dim3 grid(std::min((d.N + kTauRowWarps - 1) / kTauRowWarps, 152 * 3), 2, (rmax + kTauRowR - 1) / kTauRowR);
-    k_green_tau_r<<<grid, 32 * kTauRowWarps, smem, st>>>(d.Lx, d.Ly, K, rmax, rho, sums);
+    const int groups = kTauRowWarps * per;
+    const size_t smem = (size_t(3 * groups) + kTauRowR) * size_t(K) * sizeof(double);
+    const dim3 grid(std::min((d.N + groups - 1) / groups, 152 * 3), 2, (rmax + kTauRowR - 1) / kTauRowR);
+    k_green_tau_r<<<grid, 32 * kTauRowWarps, smem, st>>>(d.Lx, d.Ly, K, sh, rmax, rho, sums);
   }
   return int(cudaGetLastError());
 }

@@ -934,25 +934,41 @@ int rho_slices_static(const Dev& d, int K, double* host_out, void* stream) {
 // sums[rmax + r - 1] (r = 1..rmax), and the plaquette product rho_i rho_{i+x}
 // rho_{i+y} rho_{i+x+y} into sums[2 rmax].  A row of the lattice is Lx K
 // consecutive doubles and a shift by r sites is a cyclic shift by r K of it,
-// so every load is coalesced; a block takes rows blockIdx.x, + gridDim.x, ...
-// and kGreenR values of r (blockIdx.y; the last one the plaquette), which
-// share the row's own densities.  256x256 sites, K = 16, rmax = 64: 0.69 ms
-// with a thread a site (a line a lane and load), now 0.32 ms; two fused
-// multiply-adds a site, slice and r are 0.21 ms of the binary64 pipe (two
-// lanes a cycle and SM).
-constexpr int kGreenR = 4;
+// so every load is coalesced; a block takes kGreenR values of r (blockIdx.y;
+// the last one the plaquette), which share the row's own densities, and pieces
+// of kGreenSteps elements a thread: of a row, or of several rows shorter than
+// the block.  There are as many blocks as the machine holds at once: with one a
+// row, a lattice of few rows left it idle, and blocks of short rows spent their
+// time on the sums' reduction.  The call, a thread a site (a line a lane and load)
+// -> a block a row -> now: 256x256 sites, rmax = 128 with K = 16 1.57 -> 0.82 ->
+// 0.71 ms and with K = 1 0.211 -> 0.288 -> 0.114 ms; 65536x2 sites, K = 16, rmax = 1
+// 0.49 -> 2.40 -> 0.41 ms.  Two fused multiply-adds a site, slice and r, on a
+// binary64 pipe of two lanes a cycle and SM, bound the first.
+constexpr int kGreenR = 4, kGreenSteps = 4;
+// elements of a row that a block takes side by side; pieces of the lattice
+__host__ __device__ inline int green_width(long long W) { return int(W < 256 ? W : 256); }
+__host__ __device__ inline unsigned green_pieces(long long W, int Ly) {
+  const long long cw = green_width(W), rows = 256 / cw;
+  return unsigned((Ly + rows - 1) / rows * ((W + cw * kGreenSteps - 1) / (cw * kGreenSteps)));
+}
 __global__ void __launch_bounds__(256) k_green(int Lx, int Ly, int K, int rmax, const double* __restrict__ rho,
                                                double* sums) {
   const int groups = int(gridDim.y) - 1, g = int(blockIdx.y);
   const long long W = static_cast<long long>(Lx) * K;
   double ax[kGreenR] = {}, ay[kGreenR] = {};
-  for (int y = blockIdx.x; y < Ly; y += gridDim.x) {
+  const int cw = green_width(W), rows = 256 / cw, ty = int(threadIdx.x) / cw, tx = int(threadIdx.x) % cw;
+  const long long span = static_cast<long long>(cw) * kGreenSteps;
+  const unsigned pieces = green_pieces(W, Ly), across = unsigned((W + span - 1) / span);
+  for (unsigned u = blockIdx.x; u < pieces; u += gridDim.x) {
+    const int y = int(u / across) * rows + ty;
+    if (ty >= rows || y >= Ly) continue;
+    const long long from = (u % across) * span, end = from + span < W ? from + span : W;
     const double* row = rho + size_t(y) * W;
     if (g < groups) {
       const double* far[kGreenR];
 #pragma unroll
       for (int e = 0; e < kGreenR; ++e) far[e] = rho + size_t((y + min(g * kGreenR + e + 1, rmax)) % Ly) * W;
-      for (long long f = threadIdx.x; f < W; f += blockDim.x) {
+      for (long long f = from + tx; f < end; f += cw) {
         const double c = row[f];
 #pragma unroll
         for (int e = 0; e < kGreenR; ++e) {
@@ -964,7 +980,7 @@ __global__ void __launch_bounds__(256) k_green(int Lx, int Ly, int K, int rmax, 
       }
     } else {
       const double* up = rho + size_t((y + 1) % Ly) * W;
-      for (long long f = threadIdx.x; f < W; f += blockDim.x) {
+      for (long long f = from + tx; f < end; f += cw) {
         const long long fx = f + K >= W ? f + K - W : f + K;
         ax[0] = fma(row[f] * row[fx], up[f] * up[fx], ax[0]);
       }
@@ -974,10 +990,11 @@ __global__ void __launch_bounds__(256) k_green(int Lx, int Ly, int K, int rmax, 
   __shared__ double red[8][2 * kGreenR];
 #pragma unroll
   for (int e = 0; e < kGreenR; ++e) {
-    for (int o = 16; o > 0; o >>= 1) {
-      ax[e] += __shfl_down_sync(0xffffffffu, ax[e], o);
-      ay[e] += __shfl_down_sync(0xffffffffu, ay[e], o);
-    }
+    if (g < groups || e == 0)  // (the plaquette is one sum)
+      for (int o = 16; o > 0; o >>= 1) {
+        ax[e] += __shfl_down_sync(0xffffffffu, ax[e], o);
+        ay[e] += __shfl_down_sync(0xffffffffu, ay[e], o);
+      }
     if ((threadIdx.x & 31) == 0) {
       red[threadIdx.x >> 5][e] = ax[e];
       red[threadIdx.x >> 5][kGreenR + e] = ay[e];
@@ -994,7 +1011,9 @@ __global__ void __launch_bounds__(256) k_green(int Lx, int Ly, int K, int rmax, 
 
 int launch_green(int Lx, int Ly, int K, int rmax, const double* rho, double* sums, void* stream) {
   const int groups = (rmax + kGreenR - 1) / kGreenR;
-  k_green<<<dim3(std::min(Ly, 304), groups + 1), 256, 0, cudaStream_t(stream)>>>(Lx, Ly, K, rmax, rho, sums);
+  const unsigned fill = unsigned((152 * 4 + groups) / (groups + 1));  // (64 registers: 4 blocks an SM)
+  const unsigned blocks = std::min(green_pieces(static_cast<long long>(Lx) * K, Ly), fill);
+  k_green<<<dim3(blocks, groups + 1), 256, 0, cudaStream_t(stream)>>>(Lx, Ly, K, rmax, rho, sums);
   return int(cudaGetLastError());
 }
 
