@@ -800,11 +800,47 @@ int pmwa_export(pmwa_handle* h, void* buf, size_t bytes) {
   return PMWA_OK;
 }
 
+// all slots checked, filled and copied by the host, the sites in one go
+static int import_host(pmwa_handle* h, const uint64_t* in, size_t nw) {
+  const size_t N = size_t(h->d.N), cap = size_t(h->d.cap);
+  std::vector<uint32_t> cnt(N);
+  std::vector<uint64_t> keys(N * cap, 0);
+  size_t k = 1;
+  for (size_t s = 0; s < N; ++s) {
+    if (k >= nw) return PMWA_EINVAL;
+    const uint64_t hd = in[k++];
+    const size_t n = size_t(hd & 0x7fffffffu);
+    if (n > cap) return PMWA_ECAPACITY;
+    if (k + n > nw) return PMWA_EINVAL;
+    for (size_t j = 0; j < n; ++j) {
+      const uint64_t key = in[k + j];
+      if (((key >> 2) & 7) == 6) return PMWA_EINVARIANT;
+      if (j && (in[k + j - 1] >> 2) >= (key >> 2)) return PMWA_EINVARIANT;
+      // continuity: state above each event = state below the next one
+      const uint64_t nx = in[k + (j + 1) % n];
+      const int above = int(key & 1);
+      const int below_next = (((nx >> 2) & 7) == 7) ? int(1 - (nx & 1)) : int((nx >> 1) & 1);
+      if (above != below_next) return PMWA_EINVARIANT;
+    }
+    if (n && int(hd >> 63) != int(in[k + n - 1] & 1)) return PMWA_EINVARIANT;
+    std::memcpy(keys.data() + s * cap, in + k, n * 8);
+    cnt[s] = uint32_t(n) | (uint32_t(hd >> 63) << 31);
+    k += n;
+  }
+  if (cudaStreamSynchronize(h->stream) ||
+      cudaMemcpy(h->d.cntA, cnt.data(), N * 4, cudaMemcpyHostToDevice) ||
+      cudaMemcpy(h->d.keyA, keys.data(), N * cap * 8, cudaMemcpyHostToDevice))
+    return PMWA_ECUDA;
+  h->broken = false;
+  return PMWA_OK;
+}
+
 int pmwa_import(pmwa_handle* h, const void* buf, size_t bytes) {
   if (!h || !buf) return PMWA_EINVAL;
   const uint64_t* in = static_cast<const uint64_t*>(buf);
   const size_t nw = bytes / 8, N = size_t(h->d.N), cap = size_t(h->d.cap);
   if (nw < 1 || in[0] != N) return PMWA_EINVAL;
+  if (N * cap < kPackedImport) return import_host(h, in, nw);
   // the headers, up to the first one that is wrong (at site ns, with status
   // rc): the sites before it are checked for the other invariants first
   std::vector<uint64_t> at(N);
@@ -820,50 +856,23 @@ int pmwa_import(pmwa_handle* h, const void* buf, size_t bytes) {
     at[ns] = words;
     words += 1 + n;
   }
+  // checked and unpacked on the device where the buffer, the places and the
+  // answer fit the scratch (the idle next-configuration slots)
+  if (words + N + 1 > N * cap) return import_host(h, in, nw);
   if (cudaStreamSynchronize(h->stream)) return PMWA_ECUDA;
-  // checked and unpacked on the device (scratch: the idle next-configuration
-  // slots) where the buffer and its places fit there, and there are enough slots
-  if (N * cap >= kPackedImport && words + N + 1 <= N * cap) {
-    uint64_t* dev = h->d.keyB;
-    uint64_t* dat = dev + words;
-    unsigned long long* dbad = reinterpret_cast<unsigned long long*>(dat + N);
-    unsigned long long bad = 0;
-    if (cudaMemcpyAsync(dev, in, words * 8, cudaMemcpyHostToDevice, h->stream) ||
-        cudaMemcpyAsync(dat, at.data(), N * 8, cudaMemcpyHostToDevice, h->stream) ||
-        launch_packed_check(dat, dev, int(ns), dbad, h->stream) ||
-        cudaMemcpyAsync(&bad, dbad, sizeof bad, cudaMemcpyDeviceToHost, h->stream) ||
-        cudaStreamSynchronize(h->stream))
-      return PMWA_ECUDA;
-    if (bad != ~0ull) return PMWA_EINVARIANT;
-    if (rc) return rc;
-    if (launch_unpack(h->d, dat, dev, h->stream) || cudaStreamSynchronize(h->stream)) return PMWA_ECUDA;
-    h->broken = false;
-    return PMWA_OK;
-  }
-  std::vector<uint32_t> cnt(N);
-  std::vector<uint64_t> keys(N * cap, 0);
-  for (size_t s = 0; s < ns; ++s) {
-    const size_t k = at[s] + 1;
-    const uint64_t hd = in[at[s]];
-    const size_t n = size_t(hd & 0x7fffffffu);
-    for (size_t j = 0; j < n; ++j) {
-      const uint64_t key = in[k + j];
-      if (((key >> 2) & 7) == 6) return PMWA_EINVARIANT;
-      if (j && (in[k + j - 1] >> 2) >= (key >> 2)) return PMWA_EINVARIANT;
-      // continuity: state above each event = state below the next one
-      const uint64_t nx = in[k + (j + 1) % n];
-      const int above = int(key & 1);
-      const int below_next = (((nx >> 2) & 7) == 7) ? int(1 - (nx & 1)) : int((nx >> 1) & 1);
-      if (above != below_next) return PMWA_EINVARIANT;
-    }
-    if (n && int(hd >> 63) != int(in[k + n - 1] & 1)) return PMWA_EINVARIANT;
-    std::memcpy(keys.data() + s * cap, in + k, n * 8);
-    cnt[s] = uint32_t(n) | (uint32_t(hd >> 63) << 31);
-  }
-  if (rc) return rc;
-  if (cudaMemcpy(h->d.cntA, cnt.data(), N * 4, cudaMemcpyHostToDevice) ||
-      cudaMemcpy(h->d.keyA, keys.data(), N * cap * 8, cudaMemcpyHostToDevice))
+  uint64_t* dev = h->d.keyB;
+  uint64_t* dat = dev + words;
+  unsigned long long* dbad = reinterpret_cast<unsigned long long*>(dat + N);
+  unsigned long long bad = 0;
+  if (cudaMemcpyAsync(dev, in, words * 8, cudaMemcpyHostToDevice, h->stream) ||
+      cudaMemcpyAsync(dat, at.data(), N * 8, cudaMemcpyHostToDevice, h->stream) ||
+      launch_packed_check(dat, dev, int(ns), dbad, h->stream) ||
+      cudaMemcpyAsync(&bad, dbad, sizeof bad, cudaMemcpyDeviceToHost, h->stream) ||
+      cudaStreamSynchronize(h->stream))
     return PMWA_ECUDA;
+  if (bad != ~0ull) return PMWA_EINVARIANT;
+  if (rc) return rc;
+  if (launch_unpack(h->d, dat, dev, h->stream) || cudaStreamSynchronize(h->stream)) return PMWA_ECUDA;
   h->broken = false;
   return PMWA_OK;
 }

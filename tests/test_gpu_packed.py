@@ -78,3 +78,33 @@ def test_first_wrong_site_names_the_status(cap_site):
         g.import_(snap[:-1])
     assert e.value.status == P.PMWA_EINVAL
     assert np.array_equal(g.export(), snap)  # a refused buffer changes nothing
+
+
+@pytest.mark.parametrize("full", [57342, 57344, 65536])
+def test_slots_at_the_limit_of_the_packed_form(full):
+    """65536 slots whose packed words, places and answer fill the scratch to its
+    last word (57342 events of 4096 sites: 4097 + 4096 + 1 words beside them), do
+    not fit by one event pair, or whose slots are all taken: the same bytes back,
+    and an invariant broken at the last site is found."""
+    kw = dict(Lx=64, Ly=64, dom_x=16, dom_y=16, beta=1.0, eta=0.3, n_cycle=4, seed=5, cap_site=16)
+    n = np.full(4096, {57342: 14, 57344: 14, 65536: 16}[full], dtype=np.int64)
+    if full == 57342:
+        n[7] = 12
+    assert n.sum() == full
+    words = [np.array([4096], dtype=np.uint64)]
+    for s, c in enumerate(n):
+        j = np.arange(c, dtype=np.uint64)
+        m = (j << np.uint64(52)) + np.uint64(977 * s + 1)
+        words.append(np.array([int(c)], dtype=np.uint64))  # state 0 above the last worm
+        words.append((m << np.uint64(5)) | np.uint64(28) | ((j + np.uint64(1)) & np.uint64(1)))
+    buf = np.concatenate(words)
+    g = P.Sim(**kw)
+    g.import_(buf)
+    assert np.array_equal(g.export(), buf)
+    assert g.check() is None
+    bad = buf.copy()
+    bad[-1] ^= np.uint64(1)
+    with pytest.raises(P.PmwaError) as e:
+        g.import_(bad)
+    assert e.value.status == P.PMWA_EINVARIANT
+    assert np.array_equal(g.export(), buf)
