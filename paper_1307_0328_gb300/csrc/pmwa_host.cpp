@@ -1028,7 +1028,7 @@ struct pmwa_batch {
   int2* tile_work = nullptr;  // grouped by launch group (see batch_group)
   int2* bwork[2] = {nullptr, nullptr};
   int n_tile = 0, cap_max = 0;
-  int2* twork = nullptr;  // Step 1: blocks of sites of instances with temporal domains
+  int2* twork = nullptr;  // Step 1: sites of instances with temporal domains
   int tcls_off[kBatchGroups] = {}, tcls_n[kBatchGroups] = {};
   // per launch group: work range, CTA-size class, dynamic shared memory
   int cls_off[kBatchGroups] = {}, cls_n[kBatchGroups] = {}, cls_smem[kBatchGroups] = {}, cls_thr[kBatchGroups] = {};
@@ -1067,10 +1067,10 @@ bool batch_layout(const pmwa_params* p, int n, BatchLayout* L) {
     if (p[i].vertex_window > 0.0) return false;  // the batch kernels run the plain vertex phase
     Derived g;
     derive(p + i, &g);
-    if (g.ntau > 1) L->n_tw += g.N;  // upper bound: one site per block
+    if (g.ntau > 1) L->n_tw += g.N;
     L->n_tile += g.ndom;
     for (int dir = 0; dir < 2; ++dir)
-      L->n_bw[dir] += boundary_bonds(p + i, g, dir);  // upper bound: one bond per block
+      L->n_bw[dir] += boundary_bonds(p + i, g, dir);
     L->inst_bytes[size_t(i)] = layout(p + i, g).total;
   }
   size_t o = 0;
@@ -1124,12 +1124,11 @@ void build_tile_work(pmwa_batch* b, std::vector<int2>* work) {
   }
 }
 
-// Boundary work of both directions: blocks of bonds per instance, grouped
-// by the instance's launch group, so that each group can run as its own
+// Boundary work of both directions: the bonds of each instance, grouped by
+// the instance's launch group, so that each group can run as its own
 // chain of launches.
 int build_boundary_work(pmwa_batch* b) {
   std::vector<int2> bw;
-  const int bpb = boundary_bonds_per_block(b->cap_max);
   for (int dir = 0; dir < 2; ++dir) {
     bw.clear();
     for (int g = 0; g < kBatchGroups; ++g) {
@@ -1138,22 +1137,21 @@ int build_boundary_work(pmwa_batch* b) {
         const Dev& d = b->h[size_t(i)]->d;
         if (batch_group(d) != g) continue;
         const int nb = dir == 0 ? (d.ndx > 1 ? d.ndx * d.Ly : 0) : (d.ndy > 1 ? d.ndy * d.Lx : 0);
-        for (int t0 = 0; t0 < nb; t0 += bpb) bw.push_back(make_int2(i, t0));
+        for (int t = 0; t < nb; ++t) bw.push_back(make_int2(i, t));
       }
       b->bcls_n[dir][g] = int(bw.size()) - b->bcls_off[dir][g];
     }
     if (!bw.empty() && cudaMemcpy(b->bwork[dir], bw.data(), bw.size() * sizeof(int2), cudaMemcpyHostToDevice))
       return PMWA_ECUDA;
   }
-  // Step 1 of the instances with temporal domains: blocks of sites
-  const int spb = temporal_sites_per_block();
+  // Step 1 of the instances with temporal domains: sites
   bw.clear();
   for (int g = 0; g < kBatchGroups; ++g) {
     b->tcls_off[g] = int(bw.size());
     for (int i = 0; i < b->n; ++i) {
       const Dev& d = b->h[size_t(i)]->d;
       if (batch_group(d) != g || d.ntau < 2) continue;
-      for (int s0 = 0; s0 < d.N; s0 += spb) bw.push_back(make_int2(i, s0));
+      for (int s = 0; s < d.N; ++s) bw.push_back(make_int2(i, s));
     }
     b->tcls_n[g] = int(bw.size()) - b->tcls_off[g];
   }

@@ -143,7 +143,6 @@ int launch_boundary(const Dev& d, int dir, void* stream);
 int launch_temporal(const Dev& d, void* stream);  // Step 1, one warp per site
 int launch_temporal_batch(const Dev* devs, const BatchBase* base, const int2* work, int n_work, int it, int cap,
                           void* stream);
-int temporal_sites_per_block();
 int prepare_temporal(int cap);
 int launch_tile(const Dev& d, int stop, void* stream);
 int tile_class(const Dev& d, int ctas);
@@ -154,7 +153,6 @@ int launch_tile_batch(int cls, const Dev* devs, const BatchBase* base, const int
                       int it, int stop, void* stream);
 int launch_boundary_batch(const Dev* devs, const BatchBase* base, const int2* work, int n_work, int it, int dir,
                           int cap, void* stream);
-int boundary_bonds_per_block(int cap);
 int prepare_boundary(int cap);
 int prepare_tile_batch(int cls, int smem);
 int launch_advance(BatchBase* base, int n, int S, void* stream);

@@ -618,7 +618,7 @@ __device__ void boundary_warp(const Dev& d, int dir, int t, uint64_t* stage, con
   }
 }
 
-// Bonds (warps) per block.  A bond is one chain of its vertices and their
+// One bond (warp) a block.  A bond is one chain of its vertices and their
 // lengths differ, so a block of several warps keeps its place on the SM for the
 // longest; and what bounds the kernel is the number of such chains an SM can
 // interleave (every lane runs the same scalar step, 11 cycles an instruction
@@ -640,24 +640,21 @@ __device__ void boundary_warp(const Dev& d, int dir, int t, uint64_t* stage, con
 // (684 / 940 and 372 / 352), 400 replicas of 32x32 sites: 8x8 domains at beta t
 // = 4, eta = 0.2 0.597 -> 0.483 ms a launch (blocks of four warps: 0.504), four
 // slabs at beta t = 8 1.78 -> 1.36 ms of Step 1 (1.62).
-constexpr int kBoundaryWarps = 1, kBatchBlocks = 20;
+constexpr int kBatchBlocks = 20;
 
-__global__ void __launch_bounds__(32 * kBoundaryWarps, 28) k_boundary(const __grid_constant__ Dev d, int dir) {
+__global__ void __launch_bounds__(32, 28) k_boundary(const __grid_constant__ Dev d, int dir) {
   extern __shared__ __align__(16) unsigned char bsm[];
   if (instance_failed(d.err)) return;
   const ZigTab Z = zig_stage(bsm, d.zig_cap, d.worm_tries);
   __syncthreads();
-  const int wid = threadIdx.x >> 5;
-  uint64_t* stage = reinterpret_cast<uint64_t*>(bsm + kZigBytes) + size_t(2 * wid) * d.cap;
-  boundary_warp(d, dir, int(blockIdx.x) * kBoundaryWarps + wid, stage, Z);
+  boundary_warp(d, dir, int(blockIdx.x), reinterpret_cast<uint64_t*>(bsm + kZigBytes), Z);
 }
 
-// Batched form: each block serves bonds t0 .. t0 + kBoundaryWarps - 1 of one
-// instance, when that instance's boundary step is due at iteration `it`.
-__global__ void __launch_bounds__(32 * kBoundaryWarps, kBatchBlocks) k_boundary_batch(const Dev* __restrict__ devs,
-                                                                        const BatchBase* __restrict__ base,
-                                                                        const int2* __restrict__ work, int it,
-                                                                        int dir, int cap) {
+// Batched form: each block serves a bond of one instance, when that instance's
+// boundary step is due at iteration `it`.
+__global__ void __launch_bounds__(32, kBatchBlocks) k_boundary_batch(const Dev* __restrict__ devs,
+                                                                     const BatchBase* __restrict__ base,
+                                                                     const int2* __restrict__ work, int it, int dir) {
   extern __shared__ __align__(16) unsigned char bsm[];
   __shared__ Dev sd;
   const int2 w = work[blockIdx.x];
@@ -670,9 +667,7 @@ __global__ void __launch_bounds__(32 * kBoundaryWarps, kBatchBlocks) k_boundary_
   Z.wtries = sd.worm_tries;
   if (instance_failed(sd.err)) return;
   if (sd.ndom < 2 || sd.sweep % uint32_t(sd.exchange_every) != 0) return;
-  const int wid = threadIdx.x >> 5;
-  uint64_t* stage = reinterpret_cast<uint64_t*>(bsm + kZigBytes) + size_t(2 * wid) * cap;
-  boundary_warp(sd, dir, w.y + wid, stage, Z);
+  boundary_warp(sd, dir, w.y, reinterpret_cast<uint64_t*>(bsm + kZigBytes), Z);
 }
 
 // ---------------------------------------------------------------------------
@@ -753,7 +748,7 @@ __device__ __forceinline__ int temporal_site(const Dev& d, int s, uint64_t* K, i
   return PMWA_OK;
 }
 
-constexpr int kTemporalWarps = 1, kBatchSiteBlocks = 24;  // sites (warps) per block; blocks an SM
+constexpr int kBatchSiteBlocks = 24;
 
 // one warp: stage site s's list (cap keys at K), update its boundaries, and
 // write it back
@@ -776,23 +771,19 @@ __device__ void temporal_warp(const Dev& d, int s, uint64_t* K, const ZigTab& Z)
   if (lane == 0) d.cntA[s] = cnt_make(n, n ? kab(K[n - 1]) : base);
 }
 
-__global__ void __launch_bounds__(32 * kTemporalWarps, 32) k_temporal(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(32, 32) k_temporal(const __grid_constant__ Dev d) {
   extern __shared__ __align__(16) unsigned char tsm[];
   if (instance_failed(d.err)) return;
   const ZigTab Z = zig_stage(tsm, d.zig_cap, d.worm_tries);
   __syncthreads();
-  const int wid = threadIdx.x >> 5;
-  temporal_warp(d, int(blockIdx.x) * kTemporalWarps + wid,
-                reinterpret_cast<uint64_t*>(tsm + kZigBytes) + size_t(wid) * d.cap, Z);
+  temporal_warp(d, int(blockIdx.x), reinterpret_cast<uint64_t*>(tsm + kZigBytes), Z);
 }
 
-// Batched form: each block serves sites t0 .. t0 + kTemporalWarps - 1 of one
-// instance, when that instance has temporal domains and its Step 1 is due at
-// iteration `it`.
-__global__ void __launch_bounds__(32 * kTemporalWarps, kBatchSiteBlocks) k_temporal_batch(const Dev* __restrict__ devs,
-                                                                        const BatchBase* __restrict__ base,
-                                                                        const int2* __restrict__ work, int it,
-                                                                        int cap) {
+// Batched form: each block serves a site of one instance, when that instance
+// has temporal domains and its Step 1 is due at iteration `it`.
+__global__ void __launch_bounds__(32, kBatchSiteBlocks) k_temporal_batch(const Dev* __restrict__ devs,
+                                                                         const BatchBase* __restrict__ base,
+                                                                         const int2* __restrict__ work, int it) {
   extern __shared__ __align__(16) unsigned char tsm[];
   __shared__ Dev sd;
   const int2 w = work[blockIdx.x];
@@ -805,20 +796,17 @@ __global__ void __launch_bounds__(32 * kTemporalWarps, kBatchSiteBlocks) k_tempo
   Z.wtries = sd.worm_tries;
   if (instance_failed(sd.err)) return;
   if (sd.ntau < 2 || sd.sweep % uint32_t(sd.exchange_every) != 0) return;
-  const int wid = threadIdx.x >> 5;
-  temporal_warp(sd, w.y + wid, reinterpret_cast<uint64_t*>(tsm + kZigBytes) + size_t(wid) * cap, Z);
+  temporal_warp(sd, w.y, reinterpret_cast<uint64_t*>(tsm + kZigBytes), Z);
 }
 
-static size_t temporal_smem(int cap) { return size_t(kZigBytes) + size_t(kTemporalWarps) * size_t(cap) * 8; }
-
-int temporal_sites_per_block() { return kTemporalWarps; }
+static size_t temporal_smem(int cap) { return size_t(kZigBytes) + size_t(cap) * 8; }
 
 int launch_temporal(const Dev& d, void* stream) {
   if (d.ntau < 2) return 0;
   const size_t smem = temporal_smem(d.cap);
   cudaError_t e = cudaFuncSetAttribute(k_temporal, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e) return int(e);
-  k_temporal<<<blocks_for(d.N, kTemporalWarps), 32 * kTemporalWarps, smem, cudaStream_t(stream)>>>(d);
+  k_temporal<<<d.N, 32, smem, cudaStream_t(stream)>>>(d);
   return int(cudaGetLastError());
 }
 
@@ -832,8 +820,7 @@ int prepare_temporal(int cap) {
 int launch_temporal_batch(const Dev* devs, const BatchBase* base, const int2* work, int n_work, int it, int cap,
                           void* stream) {
   if (n_work <= 0) return 0;
-  k_temporal_batch<<<n_work, 32 * kTemporalWarps, temporal_smem(cap), cudaStream_t(stream)>>>(devs, base, work, it,
-                                                                                              cap);
+  k_temporal_batch<<<n_work, 32, temporal_smem(cap), cudaStream_t(stream)>>>(devs, base, work, it);
   return int(cudaGetLastError());
 }
 
@@ -857,10 +844,7 @@ int launch_advance(BatchBase* base, int n, int S, void* stream) {
   return int(cudaGetLastError());
 }
 
-// bonds per block of the boundary kernels (one warp each)
-int boundary_bonds_per_block(int cap) { (void)cap; return kBoundaryWarps; }
-
-size_t boundary_smem(int cap) { return size_t(kZigBytes) + size_t(2 * kBoundaryWarps) * size_t(cap) * 8; }
+size_t boundary_smem(int cap) { return size_t(kZigBytes) + 2 * size_t(cap) * 8; }
 
 int prepare_boundary(int cap) {
   cudaError_t e = cudaFuncSetAttribute(k_boundary, cudaFuncAttributeMaxDynamicSharedMemorySize, int(boundary_smem(cap)));
@@ -872,8 +856,7 @@ int prepare_boundary(int cap) {
 int launch_boundary_batch(const Dev* devs, const BatchBase* base, const int2* work, int n_work, int it, int dir,
                           int cap, void* stream) {
   if (n_work <= 0) return 0;
-  k_boundary_batch<<<n_work, 32 * kBoundaryWarps, boundary_smem(cap), cudaStream_t(stream)>>>(devs, base, work, it,
-                                                                                            dir, cap);
+  k_boundary_batch<<<n_work, 32, boundary_smem(cap), cudaStream_t(stream)>>>(devs, base, work, it, dir);
   return int(cudaGetLastError());
 }
 
@@ -883,7 +866,7 @@ int launch_boundary(const Dev& d, int dir, void* stream) {
   cudaError_t e = cudaFuncSetAttribute(k_boundary, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        int(boundary_smem(d.cap)));
   if (e) return int(e);
-  k_boundary<<<blocks_for(n, kBoundaryWarps), 32 * kBoundaryWarps, boundary_smem(d.cap), cudaStream_t(stream)>>>(d, dir);
+  k_boundary<<<unsigned(n), 32, boundary_smem(d.cap), cudaStream_t(stream)>>>(d, dir);
   return int(cudaGetLastError());
 }
 
