@@ -403,8 +403,7 @@ int pmwa_profile_read(pmwa_handle* h, double* ms, int64_t* launches, int32_t n);
    measurement (Step 6), 5 the block-wide passes up to the moves (groups,
    barrier, random words), 6 the moves and the look ahead to the next pass's
    vertices; 7 (a count, not cycles) the times the first warp went round its
-   waiting moves, block-wide rounds where a thread holds several worms;
-   n >= 8 entries,
+   waiting moves; n >= 8 entries,
    cleared after reading.  No paper counterpart: measurement plumbing. */
 int pmwa_profile_phases(pmwa_handle* h, uint64_t* cycles, int32_t n);
 

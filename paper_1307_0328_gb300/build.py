@@ -1,9 +1,10 @@
 """Build libpmwa.so in-tree with nvcc for sm_103a (GB300).
 
 The translation units are compiled in parallel and linked into
-paper_1307_0328_gb300/_build/libpmwa.so.  No FMA contraction anywhere
-(--fmad=false for device code, -ffp-contract=off for host code): the
-deterministic mode reproduces IEEE binary64 results operation by operation.
+paper_1307_0328_gb300/_build/libpmwa.so.  The compilers contract no
+multiply-add (--fmad=false for device code, -ffp-contract=off for host code):
+the deterministic mode reproduces IEEE binary64 results operation by operation.
+Estimators that may round less often call fma themselves.
 """
 import os
 import subprocess

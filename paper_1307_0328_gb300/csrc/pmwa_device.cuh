@@ -255,9 +255,8 @@ __device__ __forceinline__ bool xg_fix(int sigma, uint64_t I, GridScale XQ, uint
 // ---------------------------------------------------------------------------
 // Ziggurat tables as seen by a kernel: the two tables of the fast path (the
 // inner-rectangle thresholds K and the fixed-point strip edges XF) copied
-// into shared memory, because the strip index differs from lane to lane
-// (constant memory would serialise); the wedge test (about 1 % of the words)
-// reads W and F from constant memory.
+// into shared memory, because the strip index differs from lane to lane; the
+// wedge test (about 1 % of the words) reads its tables from global memory.
 struct ZigTab {
   const unsigned long long* K;   // [256] inner-rectangle threshold
   const unsigned long long* XF;  // [256] X[i] 2^58
@@ -284,7 +283,7 @@ __device__ __forceinline__ uint64_t zfix_add(uint64_t a, uint64_t b) { return (a
 // fixed point E 2^58: strip i from the low 8 bits of a word, a 53-bit
 // uniform u from its high bits, the point x = u X[i] / 2^53 as the exact
 // product (u XF[i]) >> 53; accept when u < K[i]; strip 0 past R restarts at
-// R + new deviate; else a binary64 wedge test y < e^-x with a second word.
+// R + new deviate; else the wedge test y < e^-x with a second word.
 // <= z.zcap (64) words.
 
 // The wedge test of strip i > 0 at u, with the second word w2: y < exp_det(-x)
