@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(128) k_rho_alpha(const __grid_constant__ Dev d
 // The binary64 pipe (2 lanes a cycle and SM) bounds it: with every pair's
 // seven exponentials 128x128 sites and K = 32 took 18.1 ms, now 0.62 ms.
 //
-// With K <= 16 slices a warp takes 32 >> sh sites, 2^sh >= K lanes each (one for
-// K above 16).  The call for 256x256 sites at rmax = 8, a thread a site -> a warp
+// With K <= 16 slices and many sites a warp takes 32 >> sh of them, 2^sh >= K lanes
+// each (else one).  The call for 256x256 sites at rmax = 8, a thread a site -> a warp
 // -> now: K = 2 0.296 -> 0.939 -> 0.166 ms, K = 4 1.08 -> 1.07 -> 0.25, K = 8 4.36
 // -> 1.56 -> 0.53, K = 16 17.4 -> 2.24 -> 1.30.
 constexpr int kTauWarps = 4;
@@ -472,12 +472,16 @@ __global__ void __launch_bounds__(64) k_npoint_alpha(const __grid_constant__ Dev
   if (lane == 0 && id < m) out[j] = __ddiv_rn(__ddiv_rn(acc, double(K)), etan);
 }
 
-// log2 of a tuple's lanes: as many as the slices leave work for (slice_lanes),
-// down to where m tuples have a thread for each of a full machine's 152 x 1024
+// log2 of a tuple's lanes: whole warps for few tuples (two in one warp wait for
+// each other's branches), fewer as soon as the tuples have a thread for each of
+// a full machine's 152 x 1024, and no more than there are slices once those fill
+// half of it
 int tuple_lanes(int K, int m) {
-  int sh = slice_lanes(K);
-  while (sh > 0 && (static_cast<long long>(m) << (sh - 1)) >= 152 * 1024) --sh;
-  return sh;
+  const long long full = 152 * 1024, tuples = m;
+  const int own = slice_lanes(K);
+  int sh = 5;
+  while (sh > 0 && (tuples << (sh - 1)) >= full) --sh;
+  return sh > own && (tuples << own) >= full / 2 ? own : sh;
 }
 
 }  // namespace
@@ -511,7 +515,8 @@ int launch_green_tau(const Dev& d, int K, int rmax, double* rho, double* sums, v
   cudaStream_t st = cudaStream_t(stream);
   const size_t nsum = size_t(2) * size_t(rmax + 1) * size_t(K);
   if (cudaMemsetAsync(sums, 0, nsum * sizeof(double), st) != cudaSuccess) return int(cudaGetLastError());
-  const int sh = slice_lanes(K), per = 32 >> sh;
+  // (a warp a site while all sites run at once: two in a warp wait for each other)
+  const int sh = d.N <= 152 * 4 * kTauWarps ? 5 : slice_lanes(K), per = 32 >> sh;
   if (K > 1) {
     const int bs = std::min((d.N + kTauWarps * per - 1) / (kTauWarps * per), 152 * 4);
     k_green_tau_site<<<bs, 32 * kTauWarps, 0, st>>>(d, K, sh, sums, rmax > 0 ? rho : nullptr);

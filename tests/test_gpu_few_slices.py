@@ -38,6 +38,17 @@ def test_unequal_time_at_every_group_of_lanes(kw):
             _close(g.green_tau(K, rmax), o.green_tau(K, rmax))
 
 
+def test_unequal_time_of_several_sites_a_warp():
+    """More sites than warps run at once (2432): 2 to 16 lanes a site, ragged."""
+    kw = dict(Lx=52, Ly=49, dom_x=26, dom_y=7, beta=1.5, eta=0.3, V=0.5, mu=0.4, n_cycle=4, seed=31, cap_site=64)
+    g, o = P.Sim(**kw), O.Oracle(**dict(kw, cap_site=0))
+    o.sweep(6)
+    g.import_(o.export())
+    for K in (1, 2, 3, 4, 5, 8, 9, 13, 16):
+        for rmax in (0, 2):
+            _close(g.green_tau(K, rmax), o.green_tau(K, rmax))
+
+
 def test_more_tuples_than_lanes():
     """Tuples evaluated all at once (few lanes each) and a hundred at a time
     (as many lanes as slices): the same operations in the same order."""
